@@ -76,7 +76,8 @@ def draw(rng):
         frac = rng.choice([0.0, 0.05, 0.1, 0.3, 1.0]) if rng.random() < 0.5 else 0.1
         return dict(base, kind="embed", comp="dense",
                     N=_log(rng, 5000, 2000000 if frac <= 0.1 else 300000), frac=frac,
-                    r_c=rng.choice([8.0, 9.0, 10.0, 12.0]), P=_log(rng, 50, 1000), precision=rng.choice(["fp32_comp", "fp32_comp", "fp32"]),
+                    r_c=rng.choice([8.0, 9.0, 10.0, 12.0]), P=_log(rng, 50, 1000),
+                    precision=rng.choice(["fp32_comp", "fp32_comp", "fp32"]),
                     host=rng.random() < 0.3, energies=rng.random() < 0.6)
     if what == "salt":
         return dict(base, kind="embed", comp="salt", N=_log(rng, 3000, 200000), frac=1.0,
@@ -101,7 +102,7 @@ def draw(rng):
                     nvt=True)
     if what == "list":
         return dict(base, kind="md", comp="ions", N=_log(rng, 4000, 400000), frac=1.0, r_c=8.0,
-                    P=_log(rng, 100, 500), skin=rng.choice([0.5, 1.0, 2.0]), steps=10, nvt=True)
+                    P=_log(rng, 100, 200), skin=rng.choice([0.5, 1.0, 2.0]), steps=10, nvt=True)
     return dict(base, kind="batch", comp="dense", lo=2000, hi=_log(rng, 10000, 60000),
                 n=rng.randint(4, 16), frac=0.1, P=_log(rng, 100, 300), steps=5, box="cubic")
 
