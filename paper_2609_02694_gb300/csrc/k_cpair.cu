@@ -14,11 +14,11 @@
 // other. Every particle pair within r_c lies in one such pair of clusters, or inside one
 // cluster (I = J: then only particle a with particle b > a of the cluster).
 //
-// Lanes. Lane (h, a) = (lane / 8, lane % 8) holds particle a of every i-cluster of the
-// super-cluster (coordinates and force in registers) and particles h and h + 4 of the
-// j-cluster being visited, so one visit evaluates the 8 x 8 pairs of every i-cluster the
-// visit's mask names, two per lane. The reaction on j is summed over the 8 lanes that
-// share h by shuffles, once per visit, and added to j's force.
+// Lanes. Lane (h, a) = (lane / 8, lane % 8) holds the forces on particle a of every i-cluster
+// of the super-cluster (its coordinates come from shared memory) and particles h and h + 4 of
+// the j-cluster being visited, so one visit evaluates the 8 x 8 pairs of every i-cluster the
+// visit's mask names, two per lane: in the FP32 forms as one packed pair. The reaction on j is
+// summed over the 8 lanes that share h by shuffles, once per visit, and added to j's force.
 //
 // Forces are summed in 64-bit fixed point by integer atomics. Integer sums do not depend on
 // their order, so the forces are the same run to run; a final pass converts them to
@@ -40,6 +40,7 @@
 #include <climits>
 #include <cmath>
 
+#include "f32x2.cuh"
 #include "pair_common.cuh"
 
 namespace rbe {
@@ -47,6 +48,8 @@ namespace rbe {
 constexpr int kClSize = 8;              // particles per cluster
 constexpr int kCpMaxRows = 49;          // (2R+1)^2 stencil rows for R <= 3
 constexpr int kCpMaxSeg = 2 * kCpMaxRows;
+constexpr int kCpMaxWarps = 4;          // FP32 forms: warps a block,
+constexpr int kCpWarpsLJ = 28, kCpWarpsCoul = 20;  // and resident warps an SM
 
 struct ClusterArgs {
   PairSet set;                 // full sorted set
@@ -57,6 +60,7 @@ struct ClusterArgs {
   const LJTable *table;        // device copy, multi-type only
   const int32_t *cl_base;      // nrows + 1: first global cluster of each row
   const int32_t *sc_base;      // nrows + 1: first super-cluster of each row
+  const int4 *sc_info;         // per super-cluster: row, first cluster and particle, counts
   const uint4 *cl_lo, *cl_hi;  // per cluster: (min s_x, s_y, s_z, first particle), (max..., count)
   const uint4 *jrec;           // FP32 forms: 8 slots per cluster (s_x, y and z offsets from the
                                // box corner as FP32 bits, q bits); empty slots y = -3e18
@@ -64,6 +68,7 @@ struct ClusterArgs {
   long long *facc;             // 3 x N fixed-point forces (x block, y, z)
   int64_t N;
   float fscale;                // fixed-point scale (FP32 forms)
+  float fscale_lj, kappa;      // the same times 12 A, and B / (2 A) (6 B over 12 A; one LJ type)
   double fscale_d;             // (FP64 form)
   double *epart;               // per-block partials (NQ_PAIR doubles)
   int32_t *nbr;                // neighbour counts (sorted order, zeroed before), nullable
@@ -73,6 +78,9 @@ struct ClusterArgs {
   float rc2_mid, rc2_half;     // band test: |r^2 - rc2_mid| <= rc2_half covers [rc2_lo, rc2_hi]
   int *err;
   int64_t nslots;              // the pass's energy partial slots (at least the grid)
+  int nsplit;                  // FP32 forms: blocks a super-cluster
+  int64_t wfix[2];             // 2^48 / cells in y and z (rounded down): a cell's width
+  ErfcFit fit;                 // FP32 forms
 };
 
 // ---------------------------------------------------------------------------------------
@@ -93,6 +101,9 @@ struct BoundsArgs {
   uint4 *lo, *hi;
   uint4 *jrec;                 // nullable (FP64 form)
   float hy, hz;                // length of one fractional unit in y and z
+  const int32_t *sc_base;
+  int nc_sc;
+  int4 *sc_info;               // (row, first cluster, first particle, clusters | particles << 8)
 };
 struct FinishArgs {
   long long *facc;
@@ -204,6 +215,11 @@ __device__ __forceinline__ void cluster_bounds_body(const BoundsArgs &a, int bx,
   if (k == 0) {
     a.lo[g] = make_uint4(x0, y0, z0, (uint32_t)b);
     a.hi[g] = make_uint4(x1, y1, z1, (uint32_t)n);
+    const int kc = (int)(g - cl_base[r]);  // the row's cluster; each super-cluster's first one
+    if (kc % a.nc_sc == 0) {               // writes its record
+      const int ncl = min(a.nc_sc, cl_base[r + 1] - (int)g), npt = min(a.nc_sc * kClSize, pe - b);
+      a.sc_info[a.sc_base[r] + kc / a.nc_sc] = make_int4(r, (int)g, b, ncl | (npt << 8));
+    }
   }
   if (a.jrec)
     a.jrec[t] = v ? make_uint4(x, __float_as_uint((float)(int)(y - y0) * a.hy),
@@ -275,103 +291,699 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return y;
 }
 
-template <typename real>
 struct CpAcc {
-  real u0, u1;   // single type: sum r^-12, sum r^-6; several types: U_LJ, W_LJ
-  real uc, wc, cuc, cwc;  // Coulomb energy and virial (Kahan compensations)
+  double u0, u1;  // single type: sum r^-12, sum r^-6; several types: U_LJ, W_LJ
+  double uc, wc;  // Coulomb energy and virial
 };
 
-// LJ and Coulomb terms of one pair at squared distance r2 inside the cutoff (1/r^2 = 0 and
-// qq = 0 give exact zeros); returns the force factor g (F_i += g (r_i - r_j)).
-template <typename real, bool COUL, bool MULTI>
-__device__ __forceinline__ real cp_terms(const ClusterArgs &a, bool in, real r2, real ir2,
-                                         real qi, real qj, int ti, int tj, CpAcc<real> &acc) {
-  real g;
-  const real ir6 = ir2 * ir2 * ir2;
+// FP64 form: LJ and Coulomb terms of one pair at squared distance r2 inside the cutoff
+// (1/r^2 = 0 and qq = 0 give exact zeros); returns the force factor g (F_i += g (r_i - r_j)).
+template <bool COUL, bool MULTI>
+__device__ __forceinline__ double cp_terms(const ClusterArgs &a, bool in, double r2, double ir2,
+                                           double qi, double qj, int ti, int tj, CpAcc &acc) {
+  double g;
+  const double ir6 = ir2 * ir2 * ir2;
   if (MULTI) {
     const LJTable *tab = a.table;
     const int pt = ti * tab->nt + tj;
-    real A, B, A12, B6;
-    if (sizeof(real) == 8) { A = (real)tab->Ad[pt]; B = (real)tab->Bd[pt]; A12 = (real)tab->A12d[pt]; B6 = (real)tab->B6d[pt]; }
-    else { A = (real)tab->A[pt]; B = (real)tab->B[pt]; A12 = (real)tab->A12[pt]; B6 = (real)tab->B6[pt]; }
-    const real w = ir6 * mad(A12, ir6, -B6);
+    const double w = ir6 * mad(tab->A12d[pt], ir6, -tab->B6d[pt]);
     g = w * ir2;
-    acc.u0 = mad(ir6, mad(A, ir6, -B), acc.u0);
+    acc.u0 = mad(ir6, mad(tab->Ad[pt], ir6, -tab->Bd[pt]), acc.u0);
     acc.u1 += w;
   } else {
-    const real A12 = sizeof(real) == 8 ? (real)a.ljA12d : (real)a.ljA12;
-    const real B6 = sizeof(real) == 8 ? (real)a.ljB6d : (real)a.ljB6;
-    g = ir6 * ir2 * mad(A12, ir6, -B6);
+    g = ir6 * ir2 * mad(a.ljA12d, ir6, -a.ljB6d);
     acc.u0 = mad(ir6, ir6, acc.u0);
     acc.u1 += ir6;
   }
   if (COUL) {
-    const real qq = qi * qj;
-    if (in && qq != (real)0) {
+    const double qq = qi * qj;
+    if (in && qq != 0.0) {
       const PairConst &pc = a.pc;
-      real r, rinv, erfcv, expv;
-      if (sizeof(real) == 8) {
-        r = (real)sqrt((double)r2);
-        rinv = (real)1 / r;
-        erfcv = (real)erfc(pc.sqrt_alpha_d * (double)r);
-        expv = (real)exp(-pc.alpha_d * (double)r2);
-      } else {
-        rinv = (real)rsqrtf((float)r2);
-        r = r2 * rinv;
-        erfcv = (real)erfcf(pc.sqrt_alpha * (float)r);
-        expv = (real)expf(-pc.alpha * (float)r2);
-      }
-      const real Cqq = (sizeof(real) == 8 ? (real)pc.C_d : (real)pc.C) * qq;
-      const real tsp = sizeof(real) == 8 ? (real)pc.two_sqrt_alpha_over_sqrt_pi_d
-                                         : (real)pc.two_sqrt_alpha_over_sqrt_pi;
-      const real rinv2 = rinv * rinv;
-      const real gc = Cqq * mad(erfcv * rinv, rinv2, tsp * expv * rinv2);
+      const double r = sqrt(r2), rinv = 1.0 / r;
+      const double erfcv = erfc(pc.sqrt_alpha_d * r);
+      const double expv = exp(-pc.alpha_d * r2);
+      const double Cqq = pc.C_d * qq;
+      const double rinv2 = rinv * rinv;
+      const double gc = Cqq * mad(erfcv * rinv, rinv2, pc.two_sqrt_alpha_over_sqrt_pi_d * expv * rinv2);
       g += gc;
-      if (a.comp) {
-        kahan_add(acc.uc, acc.cuc, Cqq * erfcv * rinv);
-        kahan_add(acc.wc, acc.cwc, gc * r2);
-      } else {
-        acc.uc = mad(Cqq * erfcv, rinv, acc.uc);
-        acc.wc = mad(gc, r2, acc.wc);
-      }
+      acc.uc = mad(Cqq * erfcv, rinv, acc.uc);
+      acc.wc = mad(gc, r2, acc.wc);
     }
   }
   return g;
 }
 
-// ---------------------------------------------------------------------------------------
-// The kernel: one warp per super-cluster.
+// Candidate j-clusters of a group of i-clusters with box [lo, hi] and frame centre (rx, ry, rz)
+// in row (cy, cz), by one warp: for each stencil row (dy, dz), the clusters holding the row's
+// particles within the group's x-reach (one lane per row; a row wraps into at most two parts),
+// from cluster jmin on; a warp scan gives their offsets. Writes the runs (first cluster, offset;
+// the total last) to seg_beg / seg_pre and returns the total.
+__device__ __forceinline__ int cp_segments(const ClusterArgs &a, int lane, int cy, int cz,
+                                           uint32_t rx, uint32_t ry, uint32_t rz, uint32_t xlo,
+                                           uint32_t xhi, uint32_t ylo, uint32_t yhi, uint32_t zlo,
+                                           uint32_t zhi, int jmin, int32_t *seg_beg,
+                                           int32_t *seg_pre) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const PairConst &pc = a.pc;
+  const int n0 = a.grid.n[0], n1 = a.grid.n[1], n2 = a.grid.n[2];
+  const int R1 = a.grid.R[1], R2 = a.grid.R[2];
+  const int ny = 2 * R1 + 1, nrst = ny * (2 * R2 + 1);
+  const int gxlo = (int)(xlo - rx), gxhi = (int)(xhi - rx);
+  const int gylo = (int)(ylo - ry), gyhi = (int)(yhi - ry);
+  const int gzlo = (int)(zlo - rz), gzhi = (int)(zhi - rz);
+  int carry = 0;
+  for (int rb = 0; rb < nrst; rb += 32) {
+    const int t = rb + lane;
+    int b0 = 0, l0 = 0, b1 = 0, l1 = 0;
+    if (t < nrst) {
+      const int dz = t / ny - R2, dy = t % ny - R1;
+      const int ryw = ((cy + dy) % n1 + n1) % n1, rzw = ((cz + dz) % n2 + n2) % n2;
+      const int r2i = ryw + n1 * rzw;
+      const int qs = a.set.cell_start[(int64_t)r2i * n0];
+      const int qe = a.set.cell_start[(int64_t)(r2i + 1) * n0];
+      if (qe > qs) {
+        // the row's y and z extent in frame units (unwrapped; cell edges from the width in
+        // 2^-16 units, within 2 units up to 2^16 cells, widened by 4 or more), its distance from
+        // the group's box, and the x-reach that is left
+        const int my = 4 + (n1 >> 16), mz = 4 + (n2 >> 16);
+        const int64_t y0 = (((int64_t)(cy + dy) * a.wfix[0]) >> 16) - (int64_t)ry - my;
+        const int64_t y1 = (((int64_t)(cy + dy + 1) * a.wfix[0]) >> 16) - (int64_t)ry + my;
+        const int64_t z0 = (((int64_t)(cz + dz) * a.wfix[1]) >> 16) - (int64_t)rz - mz;
+        const int64_t z1 = (((int64_t)(cz + dz + 1) * a.wfix[1]) >> 16) - (int64_t)rz + mz;
+        const int64_t ey = max((int64_t)0, max(y0 - gyhi, (int64_t)gylo - y1));
+        const int64_t ez = max((int64_t)0, max(z0 - gzhi, (int64_t)gzlo - z1));
+        const float dyl = (float)ey * pc.h[1], dzl = (float)ez * pc.h[2];
+        const float rx2 = a.bb2 - dyl * dyl - dzl * dzl;
+        if (rx2 > 0.f) {
+          const int64_t reach = (int64_t)(sqrtf(rx2) * (1.0f + 1e-5f) / pc.h[0]) + 4;
+          const int64_t X0 = (int64_t)rx + gxlo - reach, X1 = (int64_t)rx + gxhi + reach;
+          const int64_t W = (int64_t)1 << 32;
+          // the particles of the row's cells from key k0 to key k1 (whole cells: the box test
+          // rejects the clusters past the reach; a search of the row by x would cost its chain of
+          // dependent loads at every block's start)
+          auto cell_beg = [&](int64_t key) {
+            return a.set.cell_start[(int64_t)r2i * n0 + (int)((key * n0) >> 32)];
+          };
+          auto cell_end = [&](int64_t key) {
+            return a.set.cell_start[(int64_t)r2i * n0 + (int)((key * n0) >> 32) + 1];
+          };
+          int uH = qs, vH = qs, uL = qs, vL = qs;  // particle ranges: high part, low part
+          if (X1 - X0 + 1 >= W) { uL = qs; vL = qe; }
+          else if (X0 < 0) { uH = cell_beg(X0 + W); vH = qe; uL = qs; vL = cell_end(X1); }
+          else if (X1 >= W) { uH = cell_beg(X0); vH = qe; uL = qs; vL = cell_end(X1 - W); }
+          else { uL = cell_beg(X0); vL = cell_end(X1); }
+          // to cluster ranges of the row (merged when both parts reach one cluster)
+          int kL0 = 0, kL1 = -1, kH0 = 0, kH1 = -1;
+          if (vL > uL) { kL0 = (uL - qs) / kClSize; kL1 = (vL - 1 - qs) / kClSize; }
+          if (vH > uH) { kH0 = (uH - qs) / kClSize; kH1 = (vH - 1 - qs) / kClSize; }
+          if (kL1 >= kL0 && kH1 >= kH0 && kL1 >= kH0 - 1) { kL1 = max(kL1, kH1); kH1 = kH0 - 1; }
+          const int base = a.cl_base[r2i];
+          if (kL1 >= kL0) {
+            const int j0 = max(base + kL0, jmin), j1 = base + kL1;
+            if (j1 >= j0) { b0 = j0; l0 = j1 - j0 + 1; }
+          }
+          if (kH1 >= kH0) {
+            const int j0 = max(base + kH0, jmin), j1 = base + kH1;
+            if (j1 >= j0) { b1 = j0; l1 = j1 - j0 + 1; }
+          }
+        }
+      }
+    }
+    const int tot = l0 + l1;
+    int incl = tot;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(FULL, incl, o);
+      if (lane >= o) incl += v;
+    }
+    const int excl = carry + incl - tot;
+    if (t < nrst) {
+      seg_beg[2 * t] = b0;
+      seg_pre[2 * t] = excl;
+      seg_beg[2 * t + 1] = b1;
+      seg_pre[2 * t + 1] = excl + l0;
+    }
+    carry += __shfl_sync(FULL, incl, 31);
+  }
+  if (lane == 0) seg_pre[2 * nrst] = carry;
+  return carry;
+}
 
-template <typename real, bool COUL, bool MULTI, bool COUNT>
-__device__ __forceinline__ void cpair_body(const ClusterArgs &a, int bx, int nbx) {
-  constexpr bool F64 = sizeof(real) == 8;
-  constexpr int NC = F64 ? 4 : 8;          // clusters per super-cluster
+// ---------------------------------------------------------------------------------------
+// The FP32 forms' kernel. A super-cluster's visits are shared by `nsplit` blocks of blockDim.y
+// warps: warp number w of the W = nsplit * blockDim.y takes every W-th candidate, so the warps
+// of a super-cluster carry equal shares. (cpair_shape gives the split and its reason.)
+//
+// What bounds it: instruction issue and, in the pair loop, latency. A lane's two j particles are
+// a packed pair of FP32 values (f32x2.cuh), so the 8 x 8 pairs of an i-cluster cost a warp about
+// 33 instructions (49 with scalar pairs); the reaction of a visit is reduced while the next
+// visit's j records load; a block's start reads its super-cluster from one record and its
+// stencil rows by cell. On 2^20 particles the LJ pass went from 0.99e9 to 0.87e9 instructions
+// and from 1,101 to 957 us (issue 73% of the slots, FMA pipe 47%). Per visit (3.3e6 of them):
+// the pair loop about 120 instructions, its branches 24, the loads and conversions 38, the
+// reaction 31.
+
+__device__ __forceinline__ float min3(float a, float b, float c) {
+  float r;
+  asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+// 1.0 where a < b, else 0.0
+__device__ __forceinline__ float lt_one(float a, float b) {
+  float r;
+  asm("set.lt.f32.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
+struct CpAcc2 {
+  f32x2 u0, u1;            // one type: sum r^-12, sum r^-6; several: sum A12 r^-12, sum -B6 r^-6
+  f32x2 uc, wc, cuc, cwc;  // Coulomb energy and virial (Kahan compensations)
+};
+
+// FP32 forms: terms of one pair inside the cutoff that the exact decision admitted (lj: 12 A and
+// -6 B), added to the first half of the sums; returns the force factor.
+template <bool COUL, bool MULTI>
+__device__ __forceinline__ float cp_band_terms(const ClusterArgs &a, float r2, float qi, float qj,
+                                               float2 lj, CpAcc2 &acc) {
+  const float ir2 = rcp_approx(r2), ir6 = ir2 * ir2 * ir2;
+  float g = ir6 * ir2 * fmaf(lj.x, ir6, lj.y);
+  acc.u0 = add2(acc.u0, pk(MULTI ? lj.x * ir6 * ir6 : ir6 * ir6, 0.f));
+  acc.u1 = add2(acc.u1, pk(MULTI ? lj.y * ir6 : ir6, 0.f));
+  if (COUL) {
+    const PairConst &pc = a.pc;
+    const float Cqq = pc.C * qi * qj, rinv = rsqrtf(r2), r = r2 * rinv;
+    const float u = Cqq * erfcf(pc.sqrt_alpha * r) * rinv;
+    const float gc = fmaf(Cqq * pc.two_sqrt_alpha_over_sqrt_pi, expf(-pc.alpha * r2), u) * ir2;
+    g += gc;
+    acc.uc = add2(acc.uc, pk(u, 0.f));
+    acc.wc = add2(acc.wc, pk(gc * r2, 0.f));
+  }
+  return g;
+}
+
+// COUL: 0 none, 1 with the erfcx fit (ErfcFit), 2 with erfcf and expf
+template <int COUL, bool MULTI, bool COUNT>
+__device__ __forceinline__ void cpair32_body(const ClusterArgs &a, int bx, int nbx) {
+  constexpr int NC = 8;                    // clusters per super-cluster
   constexpr int NP = NC * kClSize;         // particles per super-cluster
   constexpr unsigned FULL = 0xffffffffu;
+  // scale of the pair loop's force sums (the LJ pass of one type sums forces in units of 12 A)
+  const float fsc = COUL || MULTI ? a.fscale : a.fscale_lj;
   __shared__ uint4 si[NP];                 // s_x, s_y, s_z, charge bits
   __shared__ int32_t sti[MULTI ? NP : 1];
+  __shared__ float4 ibl[NC];               // i-cluster boxes in frame coordinates: -hi x, lo x,
+  __shared__ float2 ibz[NC];               // -hi y, lo y; -hi z, lo z
+  // the group's i particles in frame coordinates (x, y, z, charge); slots outside the group hold
+  // a point no j reaches
+  __shared__ float4 sif[NP];
+  __shared__ float2 stab[MULTI ? kMaxTypes * kMaxTypes : 1];  // (12 A, -6 B) per type pair
+  __shared__ int32_t seg_beg[kCpMaxSeg], seg_pre[kCpMaxSeg + 1];
+  __shared__ int T_s;
+  __shared__ double wred[kCpMaxWarps][NQ_PAIR];
+  // candidates a warp visits: (J, mask | count << 8, first particle, -corner y), -corner z
+  extern __shared__ uint4 rec_dyn[];
+  const int lane = threadIdx.x, wid = threadIdx.y, W = blockDim.y, a8 = lane & 7, hh = lane >> 3;
+  const int tid = wid * 32 + lane, nthr = W * 32;
+  uint4 *const rec = rec_dyn + wid * 32;
+  float *const recz = reinterpret_cast<float *>(rec_dyn + W * 32) + wid * 32;
+  const int w = bx / a.nsplit, part = (bx - w * a.nsplit) * W + wid, nparts = a.nsplit * W;
+  const PairConst &pc = a.pc;
+  const int64_t N = a.N;
+  // this lane's j particles of a visited cluster, and where it adds their reaction (lanes with
+  // bits 1 and 2 of a8 set add nothing)
+  const bool b0 = a8 & 1, b1 = a8 & 2, b2 = a8 & 4;
+  const int ja = hh + (b0 ? 4 : 0), jb_ = hh + (b0 ? 0 : 4);
+  const int rslot = b1 && b2 ? INT_MAX : ja;
+  long long *const fdst = a.facc + (int64_t)(b2 ? 2 : (b1 ? 1 : 0)) * N + ja;
+  CpAcc2 acc;
+  acc.u0 = acc.u1 = acc.uc = acc.wc = acc.cuc = acc.cwc = pk(0.f);
+  const int nrows = a.nrows;
+  if (w < a.sc_base[nrows]) {
+    const int4 info = a.sc_info[w];
+    const int g0 = info.y, nc = info.w & 0xff, p0 = info.z, np = info.w >> 8;
+    const int cy = info.x % a.grid.n[1], cz = info.x / a.grid.n[1];
+    // (slots past the particles hold type 0 and no charge: masked lanes still look up the
+    // LJ table by type before their result is zeroed)
+    for (int t = tid; t < NP; t += nthr) {
+      uint4 v = make_uint4(0u, 0u, 0u, 0u);
+      int ty = 0;
+      if (t < np) {
+        const int p = p0 + t;
+        v = make_uint4(a.set.sx[p], a.set.sy[p], a.set.sz[p],
+                       COUL ? __float_as_uint(a.set.qf[p]) : 0u);
+        if (MULTI) ty = a.set.type[p];
+      }
+      si[t] = v;
+      if (MULTI) sti[t] = ty;
+    }
+    const int nt = MULTI ? a.table->nt : 1;
+    if (MULTI)
+      for (int t = tid; t < nt * nt; t += nthr) stab[t] = make_float2(a.table->A12[t], -a.table->B6[t]);
+    __syncthreads();
+    // Groups of consecutive clusters whose x extent the frame allows (normally one group).
+    // A single cluster wider than that is taken one particle at a time (asub), as a group
+    // of one point.
+    int cb = 0, asub = -1;
+    while (cb < nc) {
+      int ce = cb + 1;
+      if (asub < 0) {
+        const uint32_t xfirst = si[kClSize * cb].x;
+        while (ce < nc && si[min(np, kClSize * (ce + 1)) - 1].x - xfirst <= a.xlim) ++ce;
+        if (si[min(np, kClSize * ce) - 1].x - xfirst > a.xlim) asub = 0;
+      }
+      const int q0 = asub < 0 ? kClSize * cb : kClSize * cb + asub;
+      const int q1 = asub < 0 ? min(np, kClSize * ce) : q0 + 1;
+      // group box and frame centre (no wrap inside a row: x ascending, y and z in one cell)
+      uint32_t ylo = 0xffffffffu, yhi = 0u, zlo = 0xffffffffu, zhi = 0u;
+      for (int t = q0 + lane; t < q1; t += 32) {
+        const uint4 v = si[t];
+        ylo = min(ylo, v.y); yhi = max(yhi, v.y);
+        zlo = min(zlo, v.z); zhi = max(zhi, v.z);
+      }
+      ylo = __reduce_min_sync(FULL, ylo); yhi = __reduce_max_sync(FULL, yhi);
+      zlo = __reduce_min_sync(FULL, zlo); zhi = __reduce_max_sync(FULL, zhi);
+      const uint32_t xlo = si[q0].x, xhi = si[q1 - 1].x;
+      const uint32_t rx = xlo + ((xhi - xlo) >> 1), ry = ylo + ((yhi - ylo) >> 1),
+                     rz = zlo + ((zhi - zlo) >> 1);
+      for (int t = tid; t < NP; t += nthr) {
+        const int c = t / kClSize, a_ = t % kClSize;
+        const bool v = c >= cb && c < ce && t < np && (asub < 0 || a_ == asub);
+        const uint4 s = si[t];
+        const float x = v ? (float)(int)(s.x - rx) * pc.h[0] : 3e18f;
+        const float y = v ? (float)(int)(s.y - ry) * pc.h[1] : 3e18f;
+        const float z = v ? (float)(int)(s.z - rz) * pc.h[2] : 3e18f;
+        const float q = v && COUL ? __uint_as_float(s.w) : 0.f;
+        sif[t] = make_float4(x, y, z, q);
+      }
+      if (wid == 0) {
+        // i-cluster boxes in the frame (lanes cb..ce-1)
+        if (lane < NC) {
+          float4 lo4 = make_float4(3e18f, 3e18f, 3e18f, 0.f), hi4 = make_float4(3e18f, 3e18f, 3e18f, 0.f);
+          if (lane >= cb && lane < ce) {
+            uint4 l, u;
+            if (asub < 0) { l = a.cl_lo[g0 + lane]; u = a.cl_hi[g0 + lane]; }
+            else { l = u = si[q0]; }  // the one particle of a point group
+            lo4 = make_float4((float)(int)(l.x - rx) * pc.h[0], (float)(int)(l.y - ry) * pc.h[1],
+                              (float)(int)(l.z - rz) * pc.h[2], 0.f);
+            hi4 = make_float4((float)(int)(u.x - rx) * pc.h[0], (float)(int)(u.y - ry) * pc.h[1],
+                              (float)(int)(u.z - rz) * pc.h[2], 0.f);
+          }
+          ibl[lane] = make_float4(-hi4.x, lo4.x, -hi4.y, lo4.y);
+          ibz[lane] = make_float2(-hi4.z, lo4.z);
+        }
+        const int T0 = cp_segments(a, lane, cy, cz, rx, ry, rz, xlo, xhi, ylo, yhi, zlo, zhi, g0 + cb,
+                                   seg_beg, seg_pre);
+        if (lane == 0) T_s = T0;
+      }
+      __syncthreads();
+      const int T = T_s;
+      const int nseg = 2 * (2 * a.grid.R[1] + 1) * (2 * a.grid.R[2] + 1);
+      // forces on particle a8 of each i-cluster
+      float fxi[NC], fyi[NC], fzi[NC];
+      int cnti[NC];
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        fxi[c] = fyi[c] = fzi[c] = 0.f;
+        cnti[c] = 0;
+      }
+      // Minus the reaction on the j-cluster visited last (particles ja, jb of the cluster), its
+      // first particle and count. It is summed and added at the next visit, while that visit's
+      // j records load: over the 8 lanes sharing h, first with lane a8 xor 1, which holds the
+      // same two particles in the other order (each keeps its first one's sums: no selection),
+      // then x or y (the lane's bit 1 tells which) and z with lanes a8 xor 2 and xor 4. Every
+      // sum is the tree ((v_a + v_a^1) + (v_a^2 + v_a^3)) + (...). (The scale's sign turns it.)
+      f32x2 fxj = pk(0.f), fyj = pk(0.f), fzj = pk(0.f);
+      int pvb = 0, pvn = 0;
+      auto reaction = [&]() {
+        const float x0 = fxj.x + __shfl_xor_sync(FULL, fxj.y, 1);
+        const float y0 = fyj.x + __shfl_xor_sync(FULL, fyj.y, 1);
+        float z0 = fzj.x + __shfl_xor_sync(FULL, fzj.y, 1);
+        float u = (b1 ? y0 : x0) + __shfl_xor_sync(FULL, b1 ? x0 : y0, 2);
+        z0 += __shfl_xor_sync(FULL, z0, 2);
+        u += __shfl_xor_sync(FULL, u, 4);
+        z0 += __shfl_xor_sync(FULL, z0, 4);
+        if (rslot < pvn) fx_add(fdst + pvb, b2 ? z0 : u, -fsc, a.err);
+      };
+      // This warp's candidates in chunks of 32, one per lane: the box test against every
+      // i-cluster of the group gives a mask, the candidates with a mask are compacted into the
+      // warp's records, and the warp visits them.
+      for (int base = part; base < T; base += 32 * nparts) {
+        const int cc = base + lane * nparts;
+        uint32_t msk = 0u;
+        int J = 0, jb = 0, jn = 0;
+        float jy0 = 0.f, jz0 = 0.f;  // the candidate box's low corner in y and z (frame)
+        if (cc < T) {
+          int s = 0, e = nseg;       // the candidate's run: the last one starting at or before it
+          while (e - s > 1) {
+            const int mid = (s + e) >> 1;
+            if (seg_pre[mid] <= cc) s = mid; else e = mid;
+          }
+          J = seg_beg[s] + (cc - seg_pre[s]);
+          const uint4 l = a.cl_lo[J], u = a.cl_hi[J];
+          jb = (int)l.w;
+          jn = (int)u.w;
+          const float jx0 = (float)(int)(l.x - rx) * pc.h[0];
+          jy0 = (float)(int)(l.y - ry) * pc.h[1];
+          jz0 = (float)(int)(l.z - rz) * pc.h[2];
+          const float jx1 = (float)(int)(u.x - rx) * pc.h[0];
+          const float jy1 = (float)(int)(u.y - ry) * pc.h[1];
+          const float jz1 = (float)(int)(u.z - rz) * pc.h[2];
+          // a box that reaches past L/2 from the frame centre wraps (its ends swap sides): its
+          // distance is then that of the nearer of its two pieces
+          const bool wx = jx0 > jx1, wy = jy0 > jy1, wz = jz0 > jz1;
+          const f32x2 px = pk(jx0, -jx1), py = pk(jy0, -jy1), pz = pk(jz0, -jz1);
+          if (!(wx || wy || wz)) {
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+              const float4 bxy = ibl[c];
+              const f32x2 ex = add2(px, pk(bxy.x, bxy.y)), ey = add2(py, pk(bxy.z, bxy.w));
+              const f32x2 ez = add2(pz, ibz[c]);
+              const float gx = max3(0.f, ex.x, ex.y), gy = max3(0.f, ey.x, ey.y),
+                          gz = max3(0.f, ez.x, ez.y);
+              msk |= fmaf(gx, gx, fmaf(gy, gy, gz * gz)) <= a.bb2 ? (1u << c) : 0u;
+            }
+          } else {
+            for (int c = 0; c < NC; ++c) {
+              const float4 bxy = ibl[c];
+              const float2 bz = ibz[c];
+              const float ax = jx0 + bxy.x, bx_ = bxy.y - jx1;
+              const float ay = jy0 + bxy.z, by_ = bxy.w - jy1;
+              const float az = jz0 + bz.x, bz_ = bz.y - jz1;
+              const float gx = fmaxf(0.f, wx ? fminf(ax, bx_) : fmaxf(ax, bx_));
+              const float gy = fmaxf(0.f, wy ? fminf(ay, by_) : fmaxf(ay, by_));
+              const float gz = fmaxf(0.f, wz ? fminf(az, bz_) : fmaxf(az, bz_));
+              msk |= fmaf(gx, gx, fmaf(gy, gy, gz * gz)) <= a.bb2 ? (1u << c) : 0u;
+            }
+          }
+          // the group's clusters at or before J (a pair of clusters is taken once)
+          const int last = min(ce - 1, J - g0);
+          msk &= (2u << last) - (1u << cb);
+        }
+        const unsigned vis = __ballot_sync(FULL, msk != 0u);
+        if (msk) {
+          const int k = __popc(vis & ((1u << lane) - 1u));
+          rec[k] = make_uint4((uint32_t)J, msk | ((uint32_t)jn << 8), (uint32_t)jb,
+                              __float_as_uint(-jy0));
+          recz[k] = -jz0;
+        }
+        __syncwarp();
+        const int nv = __popc(vis);
+        for (int v = 0; v < nv; ++v) {
+          const uint4 rc4 = rec[v];
+          const float ncz = recz[v];
+          const int Jv = (int)rc4.x, vb = (int)rc4.z, vn = (int)(rc4.y >> 8);
+          const uint32_t M = rc4.y & 0xffu;
+          const float ncy = __uint_as_float(rc4.w);
+          const int cdiag = Jv - g0;  // the visited cluster's place in the super-cluster
+          // This lane's j particles, ja and jb of the cluster, as negated coordinates: x from
+          // the exact integer offset from the frame centre, y and z from the cluster's corner
+          // plus the record's offsets (an empty slot's offset of -3e18 puts it out of reach).
+          const uint4 *jr = a.jrec + ((int64_t)Jv << 3);
+          const uint4 pj0 = __ldg(jr + ja), pj1 = __ldg(jr + jb_);
+          reaction();
+          const f32x2 nx = pk((float)(int)(rx - pj0.x) * pc.h[0], (float)(int)(rx - pj1.x) * pc.h[0]);
+          const f32x2 ny = pk(ncy - __uint_as_float(pj0.y), ncy - __uint_as_float(pj1.y));
+          const f32x2 nz = pk(ncz - __uint_as_float(pj0.z), ncz - __uint_as_float(pj1.z));
+          f32x2 qjC = pk(0.f);
+          if (COUL) qjC = mul2(pk(__uint_as_float(pj0.w), __uint_as_float(pj1.w)), pk(pc.C));
+          int tj0 = 0, tj1 = 0;
+          if (MULTI) {
+            tj0 = ja < vn ? a.set.type[vb + ja] : 0;
+            tj1 = jb_ < vn ? a.set.type[vb + jb_] : 0;
+          }
+          fxj = fyj = fzj = pk(0.f);
+          int cntj0 = 0, cntj1 = 0;
+          float bmin = 3e38f;  // smallest |r^2 - r_c^2| of the visit (band test)
+          // Force factors of an i particle with this lane's two j particles, their displacements,
+          // and the force on j. (ok0, ok1: the pair counts, for a cluster with itself)
+          auto pairs = [&](f32x2 xi, f32x2 yi, f32x2 zi, f32x2 qi, int ti, bool self, bool ok0,
+                           bool ok1, f32x2 &dx, f32x2 &dy, f32x2 &dz, bool &in0, bool &in1) -> f32x2 {
+            dx = add2(xi, nx);
+            dy = add2(yi, ny);
+            dz = add2(zi, nz);
+            f32x2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
+            float ra = r2.x, rb = r2.y;
+            const f32x2 bd = add2(r2, pk(-a.rc2_mid));
+            bmin = min3(bmin, fabsf(bd.x), fabsf(bd.y));
+            if (self) {
+              ra = ok0 ? ra : 3e37f;
+              rb = ok1 ? rb : 3e37f;
+            }
+            in0 = ra < pc.rc2_lo;
+            in1 = rb < pc.rc2_lo;
+            const f32x2 m = pk(lt_one(ra, pc.rc2_lo), lt_one(rb, pc.rc2_lo));
+            const f32x2 ir2 = mul2(pk(rcp_approx(ra), rcp_approx(rb)), m);
+            const f32x2 ir6 = mul2(mul2(ir2, ir2), ir2);
+            f32x2 g;
+            if (MULTI) {
+              const float2 t0 = stab[ti * nt + tj0], t1 = stab[ti * nt + tj1];
+              const f32x2 A = pk(t0.x, t1.x), B = pk(t0.y, t1.y);
+              g = mul2(mul2(ir6, ir2), fma2(A, ir6, B));
+              acc.u0 = fma2(mul2(A, ir6), ir6, acc.u0);
+              acc.u1 = fma2(B, ir6, acc.u1);
+            } else {
+              if (COUL)
+                g = mul2(mul2(ir6, ir2), fma2(pk(a.ljA12), ir6, pk(-a.ljB6)));
+              else  // (in units of 12 A, which the fixed-point scale carries)
+                g = mul2(mul2(ir6, ir2), add2(ir6, pk(-a.kappa)));
+              acc.u0 = fma2(ir6, ir6, acc.u0);
+              acc.u1 = add2(acc.u1, ir6);
+            }
+            if (COUL) {
+              const f32x2 qq = mul2(qi, qjC);
+              const float ca = fminf(ra, pc.rc2_hi), cbb = fminf(rb, pc.rc2_hi);
+              const f32x2 r2c = pk(ca, cbb);
+              const f32x2 rinv = pk(rsqrtf(ca), rsqrtf(cbb));
+              const f32x2 rr = mul2(r2c, rinv);
+              f32x2 er, ex;
+              if (COUL == 1) {
+                erfc_exp2(a.fit, rr, r2c, er, ex);
+              } else {
+                er = pk(erfcf(pc.sqrt_alpha * rr.x), erfcf(pc.sqrt_alpha * rr.y));
+                ex = pk(expf(-pc.alpha * ca), expf(-pc.alpha * cbb));
+              }
+              const f32x2 u = mul2(mul2(qq, er), mul2(rinv, m));
+              const f32x2 ts = pk(pc.two_sqrt_alpha_over_sqrt_pi);
+              const f32x2 gc = mul2(fma2(mul2(qq, ts), ex, u), ir2);
+              g = add2(g, gc);
+              if (a.comp) {
+                kahan_add2(acc.uc, acc.cuc, u);
+                kahan_add2(acc.wc, acc.cwc, mul2(gc, r2c));
+              } else {
+                acc.uc = add2(acc.uc, u);
+                acc.wc = fma2(gc, r2c, acc.wc);
+              }
+            }
+            fxj = fma2(g, dx, fxj);
+            fyj = fma2(g, dy, fyj);
+            fzj = fma2(g, dz, fzj);
+            if (COUNT) {
+              cntj0 += in0 ? 1 : 0;
+              cntj1 += in1 ? 1 : 0;
+            }
+            return g;
+          };
+          // The visited cluster may be one of the super-cluster's own (cdiag): its pairs with
+          // itself count once (particle a8 with a later one). They are taken here, with the i
+          // particle's force added by atomics, so that the loop below carries no exclusion.
+          uint32_t Mh = M;
+          if (cdiag >= 0 && cdiag < NC && ((M >> cdiag) & 1u)) {
+            Mh &= ~(1u << cdiag);
+            const int t = kClSize * cdiag + a8;
+            const bool vd = t < np && (asub < 0 || a8 == asub);
+            const float4 pi = sif[t];
+            f32x2 dx, dy, dz;
+            bool in0, in1;
+            const f32x2 g = pairs(pk(pi.x), pk(pi.y), pk(pi.z), pk(pi.w), MULTI ? sti[t] : 0, true, vd && a8 < ja,
+                                  vd && a8 < jb_, dx, dy, dz, in0, in1);
+            float fdx = fmaf(g.y, dx.y, g.x * dx.x), fdy = fmaf(g.y, dy.y, g.x * dy.x),
+                  fdz = fmaf(g.y, dz.y, g.x * dz.x);
+            fdx += __shfl_xor_sync(FULL, fdx, 8); fdx += __shfl_xor_sync(FULL, fdx, 16);
+            fdy += __shfl_xor_sync(FULL, fdy, 8); fdy += __shfl_xor_sync(FULL, fdy, 16);
+            fdz += __shfl_xor_sync(FULL, fdz, 8); fdz += __shfl_xor_sync(FULL, fdz, 16);
+            if (vd && hh < 3)
+              fx_add(a.facc + (int64_t)hh * N + p0 + t, hh == 0 ? fdx : (hh == 1 ? fdy : fdz),
+                     fsc, a.err);
+            if (COUNT) {
+              int cd = (in0 ? 1 : 0) + (in1 ? 1 : 0);
+              cd += __shfl_xor_sync(FULL, cd, 8);
+              cd += __shfl_xor_sync(FULL, cd, 16);
+              if (vd && hh == 3 && cd) atomicAdd(a.nbr + p0 + t, cd);
+            }
+          }
+#pragma unroll
+          for (int c = 0; c < NC; ++c) {
+            if ((Mh >> c) & 1u) {
+              const int t = kClSize * c + a8;
+              const float4 pi = sif[t];
+              f32x2 dx, dy, dz;
+              bool in0, in1;
+              const f32x2 g = pairs(pk(pi.x), pk(pi.y), pk(pi.z), pk(pi.w), MULTI ? sti[t] : 0, false, true, true,
+                                    dx, dy, dz, in0, in1);
+              fxi[c] = fmaf(g.y, dx.y, fmaf(g.x, dx.x, fxi[c]));
+              fyi[c] = fmaf(g.y, dy.y, fmaf(g.x, dy.x, fyi[c]));
+              fzi[c] = fmaf(g.y, dz.y, fmaf(g.x, dz.x, fzi[c]));
+              if (COUNT) cnti[c] += (in0 ? 1 : 0) + (in1 ? 1 : 0);
+            }
+          }
+          // Band pairs: the exact decision; a pair inside is added by atomics.
+          if (__any_sync(FULL, bmin <= a.rc2_half)) {
+            for (int c = cb; c < ce; ++c) {
+              if (!((M >> c) & 1u)) continue;
+              const int t = kClSize * c + a8;
+              if (t >= np || (asub >= 0 && a8 != asub)) continue;
+              const uint4 s = si[t];
+              const float x0 = sif[t].x, y0 = sif[t].y, z0 = sif[t].z;
+              for (int k = 0; k < 2; ++k) {
+                const int j = k ? jb_ : ja;
+                if (!(j < vn) || !(c != cdiag || a8 < j)) continue;
+                const float dx = x0 + (k ? nx.y : nx.x), dy = y0 + (k ? ny.y : ny.x),
+                            dz = z0 + (k ? nz.y : nz.x);
+                const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                if (!(r2 >= pc.rc2_lo && r2 <= pc.rc2_hi)) continue;
+                const int pj = vb + j;
+                const int dsx = (int)(s.x - a.set.sx[pj]), dsy = (int)(s.y - a.set.sy[pj]),
+                          dsz = (int)(s.z - a.set.sz[pj]);
+                if (!(exact_r2(pc, dsx, dsy, dsz) <= pc.rc2d)) continue;
+                const float g = cp_band_terms<COUL != 0, MULTI>(
+                    a, r2, COUL ? __uint_as_float(s.w) : 0.f, COUL ? a.set.qf[pj] : 0.f,
+                    MULTI ? stab[sti[t] * nt + (k ? tj1 : tj0)] : make_float2(a.ljA12, -a.ljB6), acc);
+                const int pi = p0 + t;
+                fx_add(a.facc + pi, g * dx, a.fscale, a.err);
+                fx_add(a.facc + N + pi, g * dy, a.fscale, a.err);
+                fx_add(a.facc + 2 * N + pi, g * dz, a.fscale, a.err);
+                fx_add(a.facc + pj, -g * dx, a.fscale, a.err);
+                fx_add(a.facc + N + pj, -g * dy, a.fscale, a.err);
+                fx_add(a.facc + 2 * N + pj, -g * dz, a.fscale, a.err);
+                if (COUNT) { atomicAdd(a.nbr + pi, 1); atomicAdd(a.nbr + pj, 1); }
+              }
+            }
+          }
+          if (COUNT) {
+            const unsigned gm = 0xffu << (8 * hh);
+            const int c0 = __reduce_add_sync(gm, b0 ? cntj1 : cntj0);
+            const int c1 = __reduce_add_sync(gm, b0 ? cntj0 : cntj1);
+            if (a8 == 0) {
+              if (hh < vn && c0) atomicAdd(a.nbr + vb + hh, c0);
+              if (hh + 4 < vn && c1) atomicAdd(a.nbr + vb + hh + 4, c1);
+            }
+          }
+          pvb = vb;
+          pvn = vn;
+        }
+        __syncwarp();
+      }
+      reaction();
+      // i forces: sum over the four lanes sharing a8, then lane (h, a8) adds clusters c with
+      // c % 4 == h
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        float fx = fxi[c], fy = fyi[c], fz = fzi[c];
+        fx += __shfl_xor_sync(FULL, fx, 8); fx += __shfl_xor_sync(FULL, fx, 16);
+        fy += __shfl_xor_sync(FULL, fy, 8); fy += __shfl_xor_sync(FULL, fy, 16);
+        fz += __shfl_xor_sync(FULL, fz, 8); fz += __shfl_xor_sync(FULL, fz, 16);
+        if (COUNT) {
+          cnti[c] += __shfl_xor_sync(FULL, cnti[c], 8);
+          cnti[c] += __shfl_xor_sync(FULL, cnti[c], 16);
+        }
+        const int t = kClSize * c + a8;
+        if ((c & 3) == hh && c >= cb && c < ce && t < np && (asub < 0 || a8 == asub)) {
+          const int64_t pi = p0 + t;
+          fx_add(a.facc + pi, fx, fsc, a.err);
+          fx_add(a.facc + N + pi, fy, fsc, a.err);
+          fx_add(a.facc + 2 * N + pi, fz, fsc, a.err);
+          if (COUNT && cnti[c]) atomicAdd(a.nbr + pi, cnti[c]);
+        }
+      }
+      __syncthreads();  // (the group's shared arrays are free for the next one)
+      if (asub < 0) {
+        cb = ce;
+      } else if (++asub >= min(kClSize, np - kClSize * cb)) {
+        asub = -1;
+        ++cb;
+      }
+    }
+  }
+  // block partials of the energies and virials (each pair counted once)
+  double ulj, wlj, v[NQ_PAIR];
+  const double u0 = (double)acc.u0.x + (double)acc.u0.y, u1 = (double)acc.u1.x + (double)acc.u1.y;
+  if (MULTI) {
+    ulj = u0 / 12.0 + u1 / 6.0;
+    wlj = u0 + u1;
+  } else {
+    const double A = (double)a.ljA, B = (double)a.ljB;
+    ulj = A * u0 - B * u1;
+    wlj = 12.0 * A * u0 - 6.0 * B * u1;
+  }
+  v[Q_ULJ] = ulj;
+  v[Q_WLJ] = wlj;
+  v[Q_UREAL] = v[Q_WREAL] = 0.0;
+  if (COUL) {
+    v[Q_UREAL] = ((double)acc.uc.x - (double)acc.cuc.x) + ((double)acc.uc.y - (double)acc.cuc.y);
+    v[Q_WREAL] = ((double)acc.wc.x - (double)acc.cwc.x) + ((double)acc.wc.y - (double)acc.cwc.y);
+  }
+#pragma unroll
+  for (int k = 0; k < NQ_PAIR; ++k) {
+    const bool used = COUL || k == Q_ULJ || k == Q_WLJ;
+    const double s = used ? warp_sum(v[k]) : 0.0;
+    if (W == 1) {
+      if (lane == 0) a.epart[(int64_t)bx * NQ_PAIR + k] = s;
+    } else if (lane == 0) {
+      wred[wid][k] = s;
+    }
+  }
+  if (W > 1) {
+    __syncthreads();
+    if (tid < NQ_PAIR) {
+      double s = 0.0;
+      for (int k = 0; k < W; ++k) s += wred[k][tid];
+      a.epart[(int64_t)bx * NQ_PAIR + tid] = s;
+    }
+  }
+  // the pass's partial slots past the grid (the range is sized for the per-particle kernel,
+  // the grid for the super-clusters) hold zeros
+  for (int64_t z = (int64_t)bx + nbx; z < a.nslots; z += nbx)
+    if (tid < NQ_PAIR) a.epart[z * NQ_PAIR + tid] = 0.0;
+}
+
+// (Register caps: 72 for the LJ pass, 28 warps an SM at 60 spilled bytes; 80 without spills
+// ran 2% slower, 96 8% slower. 96 with Coulomb terms, 20 warps; 128 ran 10% slower.)
+template <int COUL, bool MULTI, bool COUNT>
+__global__ void __launch_bounds__(32 * kCpMaxWarps,
+                                  (COUL ? kCpWarpsCoul : kCpWarpsLJ) / kCpMaxWarps)
+    cpair32_kernel(const ClusterArgs a) {
+  cpair32_body<COUL, MULTI, COUNT>(a, (int)blockIdx.x, (int)gridDim.x);
+}
+
+// ---------------------------------------------------------------------------------------
+// The FP64 form's kernel: one warp per super-cluster.
+
+template <bool COUL, bool MULTI, bool COUNT>
+__device__ __forceinline__ void cpair64_body(const ClusterArgs &a, int bx, int nbx) {
+  using real = double;
+  constexpr int NC = 4;                    // clusters per super-cluster
+  constexpr int NP = NC * kClSize;         // particles per super-cluster
+  constexpr unsigned FULL = 0xffffffffu;
+  __shared__ uint4 si[NP];                 // s_x, s_y, s_z
+  __shared__ int32_t sti[MULTI ? NP : 1];
   __shared__ float4 ibl[NC], ibh[NC];      // i-cluster boxes in frame coordinates
-  // FP32 forms: the group's i particles in frame coordinates (x, y, z, charge), read once
-  // per i-cluster and visit; slots outside the group hold a point no j can reach
-  __shared__ float4 sif[F64 ? 1 : NP];
   __shared__ int32_t seg_beg[kCpMaxSeg], seg_pre[kCpMaxSeg + 1];
   const int lane = threadIdx.x, a8 = lane & 7, hh = lane >> 3;
   const int w = bx;
   const PairConst &pc = a.pc;
   const int64_t N = a.N;
-  CpAcc<real> acc;
-  acc.u0 = acc.u1 = acc.uc = acc.wc = acc.cuc = acc.cwc = (real)0;
+  CpAcc acc;
+  acc.u0 = acc.u1 = acc.uc = acc.wc = 0.0;
   const int nrows = a.nrows;
   if (w < a.sc_base[nrows]) {
-    const int r = row_of(a.sc_base, nrows, w);
-    const int n0 = a.grid.n[0], n1 = a.grid.n[1], n2 = a.grid.n[2];
-    const int ps = a.set.cell_start[(int64_t)r * n0], pe = a.set.cell_start[(int64_t)(r + 1) * n0];
-    const int ksc = w - a.sc_base[r];
-    const int g0 = a.cl_base[r] + ksc * NC;
-    const int nc = min(NC, a.cl_base[r + 1] - a.cl_base[r] - ksc * NC);
-    const int p0 = ps + ksc * NP;
-    const int np = min(NP, pe - p0);
-    const int cy = r % n1, cz = r / n1;
+    const int4 info = a.sc_info[w];
+    const int g0 = info.y, nc = info.w & 0xff, p0 = info.z, np = info.w >> 8;
+    const int cy = info.x % a.grid.n[1], cz = info.x / a.grid.n[1];
     // (slots past the particles hold type 0 and no charge: masked lanes still look up the
     // LJ table by type before their result is zeroed)
     for (int t = lane; t < NP; t += 32) {
@@ -379,8 +991,7 @@ __device__ __forceinline__ void cpair_body(const ClusterArgs &a, int bx, int nbx
       int ty = 0;
       if (t < np) {
         const int p = p0 + t;
-        v = make_uint4(a.set.sx[p], a.set.sy[p], a.set.sz[p],
-                       COUL ? __float_as_uint(a.set.qf[p]) : 0u);
+        v = make_uint4(a.set.sx[p], a.set.sy[p], a.set.sz[p], 0u);
         if (MULTI) ty = a.set.type[p];
       }
       si[t] = v;
@@ -423,21 +1034,10 @@ __device__ __forceinline__ void cpair_body(const ClusterArgs &a, int bx, int nbx
         vi[c] = v;
         const uint4 s = si[t];
         oxi[c] = (int)(s.x - rx); oyi[c] = (int)(s.y - ry); ozi[c] = (int)(s.z - rz);
-        qi[c] = COUL ? (real)__uint_as_float(s.w) : (real)0;
-        if (COUL && F64 && v) qi[c] = (real)a.set.qd[p0 + t];
+        qi[c] = COUL && v ? a.set.qd[p0 + t] : 0.0;
         ti[c] = MULTI ? sti[t] : 0;
         fxi[c] = fyi[c] = fzi[c] = (real)0;
         cnti[c] = 0;
-      }
-      if (!F64) {
-        for (int t = lane; t < NP; t += 32) {
-          const int c = t / kClSize, a_ = t % kClSize;
-          const bool v = c >= cb && c < ce && t < np && (asub < 0 || a_ == asub);
-          const uint4 s = si[t];
-          sif[t] = v ? make_float4((float)(int)(s.x - rx) * pc.h[0], (float)(int)(s.y - ry) * pc.h[1],
-                                   (float)(int)(s.z - rz) * pc.h[2], __uint_as_float(s.w))
-                     : make_float4(3e18f, 3e18f, 3e18f, 0.f);
-        }
       }
       // i-cluster boxes in the frame (lanes cb..ce-1)
       if (lane < NC) {
@@ -454,92 +1054,9 @@ __device__ __forceinline__ void cpair_body(const ClusterArgs &a, int bx, int nbx
         ibl[lane] = lo4;
         ibh[lane] = hi4;
       }
-      // Candidate j-clusters: for each stencil row (dy, dz), the clusters holding the row's
-      // particles within the group's x-reach (one lane per row; a row wraps into at most
-      // two parts), from the group's first global cluster on; a warp scan gives offsets.
-      const int R1 = a.grid.R[1], R2 = a.grid.R[2];
-      const int ny = 2 * R1 + 1, nrst = ny * (2 * R2 + 1);
-      const int gxlo = (int)(xlo - rx), gxhi = (int)(xhi - rx);
-      const int gylo = (int)(ylo - ry), gyhi = (int)(yhi - ry);
-      const int gzlo = (int)(zlo - rz), gzhi = (int)(zhi - rz);
-      const int jmin = g0 + cb;
-      int carry = 0;
-      for (int rb = 0; rb < nrst; rb += 32) {
-        const int t = rb + lane;
-        int b0 = 0, l0 = 0, b1 = 0, l1 = 0;
-        if (t < nrst) {
-          const int dz = t / ny - R2, dy = t % ny - R1;
-          const int ryw = ((cy + dy) % n1 + n1) % n1, rzw = ((cz + dz) % n2 + n2) % n2;
-          const int r2i = ryw + n1 * rzw;
-          const int qs = a.set.cell_start[(int64_t)r2i * n0];
-          const int qe = a.set.cell_start[(int64_t)(r2i + 1) * n0];
-          if (qe > qs) {
-            // the row's y and z extent in frame units (unwrapped, widened by 2 units), its
-            // distance from the group's box, and the x-reach that is left
-            const int64_t W32 = (int64_t)1 << 32;
-            const int64_t y0 = (int64_t)(cy + dy) * W32 / n1 - (int64_t)ry - 2;
-            const int64_t y1 = (int64_t)(cy + dy + 1) * W32 / n1 - (int64_t)ry + 2;
-            const int64_t z0 = (int64_t)(cz + dz) * W32 / n2 - (int64_t)rz - 2;
-            const int64_t z1 = (int64_t)(cz + dz + 1) * W32 / n2 - (int64_t)rz + 2;
-            const int64_t ey = max((int64_t)0, max(y0 - gyhi, (int64_t)gylo - y1));
-            const int64_t ez = max((int64_t)0, max(z0 - gzhi, (int64_t)gzlo - z1));
-            const float dyl = (float)ey * pc.h[1], dzl = (float)ez * pc.h[2];
-            const float rx2 = a.bb2 - dyl * dyl - dzl * dzl;
-            if (rx2 > 0.f) {
-              const int64_t reach = (int64_t)(sqrtf(rx2) * (1.0f + 1e-5f) / pc.h[0]) + 4;
-              const int64_t X0 = (int64_t)rx + gxlo - reach, X1 = (int64_t)rx + gxhi + reach;
-              const int64_t W = (int64_t)1 << 32;
-              // first particle of [qs, qe) with s_x >= key (rows are sorted by s_x)
-              auto first_ge = [&](int64_t key) {
-                int lo = qs, hi = qe;
-                while (lo < hi) {
-                  const int mid = (lo + hi) >> 1;
-                  if ((int64_t)a.set.sx[mid] < key) lo = mid + 1;
-                  else hi = mid;
-                }
-                return lo;
-              };
-              int uH = qs, vH = qs, uL = qs, vL = qs;  // particle ranges: high part, low part
-              if (X1 - X0 + 1 >= W) { uL = qs; vL = qe; }
-              else if (X0 < 0) { uH = first_ge(X0 + W); vH = qe; uL = qs; vL = first_ge(X1 + 1); }
-              else if (X1 >= W) { uH = first_ge(X0); vH = qe; uL = qs; vL = first_ge(X1 - W + 1); }
-              else { uL = first_ge(X0); vL = first_ge(X1 + 1); }
-              // to cluster ranges of the row (merged when both parts reach one cluster)
-              int kL0 = 0, kL1 = -1, kH0 = 0, kH1 = -1;
-              if (vL > uL) { kL0 = (uL - qs) / kClSize; kL1 = (vL - 1 - qs) / kClSize; }
-              if (vH > uH) { kH0 = (uH - qs) / kClSize; kH1 = (vH - 1 - qs) / kClSize; }
-              if (kL1 >= kL0 && kH1 >= kH0 && kL1 >= kH0 - 1) { kL1 = max(kL1, kH1); kH1 = kH0 - 1; }
-              const int base = a.cl_base[r2i];
-              if (kL1 >= kL0) {
-                const int j0 = max(base + kL0, jmin), j1 = base + kL1;
-                if (j1 >= j0) { b0 = j0; l0 = j1 - j0 + 1; }
-              }
-              if (kH1 >= kH0) {
-                const int j0 = max(base + kH0, jmin), j1 = base + kH1;
-                if (j1 >= j0) { b1 = j0; l1 = j1 - j0 + 1; }
-              }
-            }
-          }
-        }
-        const int tot = l0 + l1;
-        int incl = tot;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int v = __shfl_up_sync(FULL, incl, o);
-          if (lane >= o) incl += v;
-        }
-        const int excl = carry + incl - tot;
-        if (t < nrst) {
-          seg_beg[2 * t] = b0;
-          seg_pre[2 * t] = excl;
-          seg_beg[2 * t + 1] = b1;
-          seg_pre[2 * t + 1] = excl + l0;
-        }
-        carry += __shfl_sync(FULL, incl, 31);
-      }
-      if (lane == 0) seg_pre[2 * nrst] = carry;
+      const int T = cp_segments(a, lane, cy, cz, rx, ry, rz, xlo, xhi, ylo, yhi, zlo, zhi, g0 + cb,
+                                seg_beg, seg_pre);
       __syncwarp();
-      const int T = carry;
       // Candidates in chunks of 32, one per lane: the box test against every i-cluster of
       // the group gives a mask; the warp then visits each candidate with a mask.
       int sg = 0;
@@ -547,7 +1064,6 @@ __device__ __forceinline__ void cpair_body(const ClusterArgs &a, int bx, int nbx
         const int cc = base + lane;
         int s = sg, J = 0, jb = 0, jn = 0;
         uint32_t msk = 0u;
-        float jy0 = 0.f, jz0 = 0.f;  // the candidate box's low corner in y and z (frame)
         if (cc < T) {
           while (seg_pre[s + 1] <= cc) ++s;
           J = seg_beg[s] + (cc - seg_pre[s]);
@@ -555,8 +1071,8 @@ __device__ __forceinline__ void cpair_body(const ClusterArgs &a, int bx, int nbx
           jb = (int)l.w;
           jn = (int)u.w;
           const float jx0 = (float)(int)(l.x - rx) * pc.h[0];
-          jy0 = (float)(int)(l.y - ry) * pc.h[1];
-          jz0 = (float)(int)(l.z - rz) * pc.h[2];
+          const float jy0 = (float)(int)(l.y - ry) * pc.h[1];
+          const float jz0 = (float)(int)(l.z - rz) * pc.h[2];
           const float jx1 = (float)(int)(u.x - rx) * pc.h[0];
           const float jy1 = (float)(int)(u.y - ry) * pc.h[1];
           const float jz1 = (float)(int)(u.z - rz) * pc.h[2];
@@ -585,13 +1101,10 @@ __device__ __forceinline__ void cpair_body(const ClusterArgs &a, int bx, int nbx
           const int Jv = __shfl_sync(FULL, J, t0);
           const uint32_t M = __shfl_sync(FULL, msk, t0);
           const int vb = __shfl_sync(FULL, jb, t0), vn = __shfl_sync(FULL, jn, t0);
-          const float cyj = F64 ? 0.f : __shfl_sync(FULL, jy0, t0);
-          const float czj = F64 ? 0.f : __shfl_sync(FULL, jz0, t0);
           const int cdiag = Jv - g0;  // the visited cluster's place in the super-cluster
-          // This lane's j particles, h and h + 4 of the cluster: x from the exact integer
-          // offset from the frame centre, y and z from the cluster's corner plus the record's
-          // offsets, in FP32 (exact integer offsets in the FP64 form).
-          real xj[2], yj[2], zj[2], qj[2], fxj[2], fyj[2], fzj[2];
+          // This lane's j particles, h and h + 4 of the cluster: exact integer offsets from the
+          // frame centre.
+          real qj[2], fxj[2], fyj[2], fzj[2];
           int oxj[2], oyj[2], ozj[2], tj[2], cntj[2];
           bool vj[2];
 #pragma unroll
@@ -599,56 +1112,30 @@ __device__ __forceinline__ void cpair_body(const ClusterArgs &a, int bx, int nbx
             const int t = hh + 4 * k;
             vj[k] = t < vn;
             const int p = vb + (vj[k] ? t : 0);
-            oxj[k] = oyj[k] = ozj[k] = 0;
-            qj[k] = (real)0;
-            if (!F64) {
-              // (an empty slot's y of -3e18 puts it out of reach)
-              const uint4 pj = __ldg(&a.jrec[((int64_t)Jv << 3) + t]);
-              xj[k] = (real)((float)(int)(pj.x - rx) * pc.h[0]);
-              yj[k] = (real)(cyj + __uint_as_float(pj.y));
-              zj[k] = (real)(czj + __uint_as_float(pj.z));
-              if (COUL) qj[k] = (real)__uint_as_float(pj.w);
-            } else {
-              oxj[k] = (int)(a.set.sx[p] - rx);
-              oyj[k] = (int)(a.set.sy[p] - ry);
-              ozj[k] = (int)(a.set.sz[p] - rz);
-              xj[k] = yj[k] = zj[k] = (real)0;
-              if (COUL) qj[k] = (real)a.set.qd[p];
-            }
+            oxj[k] = (int)(a.set.sx[p] - rx);
+            oyj[k] = (int)(a.set.sy[p] - ry);
+            ozj[k] = (int)(a.set.sz[p] - rz);
+            qj[k] = COUL ? a.set.qd[p] : 0.0;
             tj[k] = MULTI ? a.set.type[p] : 0;
             fxj[k] = fyj[k] = fzj[k] = (real)0;
             cntj[k] = 0;
           }
-          float bmin = 3e38f;  // FP32 forms: smallest |r^2 - r_c^2| of the visit (band test)
-          // Pair force of i (frame coordinates or integer offsets) with this lane's j particle k,
-          // when `ok`; adds the reaction to j and returns the force factor and displacement.
-          auto pair_one = [&](bool ok, real xi_, real yi_, real zi_, int oxi_, int oyi_,
-                              int ozi_, real qi_, int ti_, int k, real &dx, real &dy, real &dz,
-                              bool &in) -> real {
-            real r2, ir2;
-            if (F64) {
-              // the offsets' difference (mod 2^32) is the exact minimum-image displacement
-              const int dsx = (int)((uint32_t)oxi_ - (uint32_t)oxj[k]);
-              const int dsy = (int)((uint32_t)oyi_ - (uint32_t)oyj[k]);
-              const int dsz = (int)((uint32_t)ozi_ - (uint32_t)ozj[k]);
-              dx = (real)__dmul_rn((double)dsx, pc.hd[0]);
-              dy = (real)__dmul_rn((double)dsy, pc.hd[1]);
-              dz = (real)__dmul_rn((double)dsz, pc.hd[2]);
-              r2 = (real)__dadd_rn(__dadd_rn(__dmul_rn((double)dx, (double)dx),
-                                             __dmul_rn((double)dy, (double)dy)),
-                                   __dmul_rn((double)dz, (double)dz));
-              in = ok && vj[k] && (double)r2 <= pc.rc2d;
-              ir2 = in ? (real)(1.0 / (double)r2) : (real)0;
-            } else {
-              dx = xi_ - xj[k];
-              dy = yi_ - yj[k];
-              dz = zi_ - zj[k];
-              r2 = (real)fmaf((float)dx, (float)dx, fmaf((float)dy, (float)dy, (float)(dz * dz)));
-              in = ok && (float)r2 < pc.rc2_lo;
-              bmin = fminf(bmin, fabsf((float)r2 - a.rc2_mid));
-              ir2 = in ? (real)rcp_approx((float)r2) : (real)0;
-            }
-            const real g = cp_terms<real, COUL, MULTI>(a, in, r2, ir2, qi_, qj[k], ti_, tj[k], acc);
+          // Pair force of i (integer offsets) with this lane's j particle k, when `ok`; adds the
+          // reaction to j and returns the force factor and displacement.
+          auto pair_one = [&](bool ok, int oxi_, int oyi_, int ozi_, real qi_, int ti_, int k,
+                              real &dx, real &dy, real &dz, bool &in) -> real {
+            // the offsets' difference (mod 2^32) is the exact minimum-image displacement
+            const int dsx = (int)((uint32_t)oxi_ - (uint32_t)oxj[k]);
+            const int dsy = (int)((uint32_t)oyi_ - (uint32_t)oyj[k]);
+            const int dsz = (int)((uint32_t)ozi_ - (uint32_t)ozj[k]);
+            dx = __dmul_rn((double)dsx, pc.hd[0]);
+            dy = __dmul_rn((double)dsy, pc.hd[1]);
+            dz = __dmul_rn((double)dsz, pc.hd[2]);
+            const real r2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)),
+                                      __dmul_rn(dz, dz));
+            in = ok && vj[k] && r2 <= pc.rc2d;
+            const real ir2 = in ? 1.0 / r2 : 0.0;
+            const real g = cp_terms<COUL, MULTI>(a, in, r2, ir2, qi_, qj[k], ti_, tj[k], acc);
             fxj[k] = mad(-g, dx, fxj[k]); fyj[k] = mad(-g, dy, fyj[k]); fzj[k] = mad(-g, dz, fzj[k]);
             if (COUNT) cntj[k] += in ? 1 : 0;
             return g;
@@ -664,11 +1151,7 @@ __device__ __forceinline__ void cpair_body(const ClusterArgs &a, int bx, int nbx
             const bool vd = t < np && (asub < 0 || a8 == asub);
             const uint4 sd = si[t];
             const int ox = (int)(sd.x - rx), oy = (int)(sd.y - ry), oz = (int)(sd.z - rz);
-            const real xd = vd ? (real)((float)ox * pc.h[0]) : (real)3e18f;
-            const real yd = vd ? (real)((float)oy * pc.h[1]) : (real)3e18f;
-            const real zd = vd ? (real)((float)oz * pc.h[2]) : (real)3e18f;
-            real qd = (real)0;
-            if (COUL) qd = F64 ? (vd ? (real)a.set.qd[p0 + t] : (real)0) : (real)__uint_as_float(sd.w);
+            const real qd = COUL && vd ? a.set.qd[p0 + t] : 0.0;
             const int td = MULTI ? sti[t] : 0;
             real fdx = (real)0, fdy = (real)0, fdz = (real)0;
             int cd = 0;
@@ -676,8 +1159,7 @@ __device__ __forceinline__ void cpair_body(const ClusterArgs &a, int bx, int nbx
             for (int k = 0; k < 2; ++k) {
               real dx, dy, dz;
               bool in;
-              const real g = pair_one(vd && a8 < hh + 4 * k, xd, yd, zd, ox, oy, oz, qd, td, k,
-                                      dx, dy, dz, in);
+              const real g = pair_one(vd && a8 < hh + 4 * k, ox, oy, oz, qd, td, k, dx, dy, dz, in);
               fdx = mad(g, dx, fdx); fdy = mad(g, dy, fdy); fdz = mad(g, dz, fdz);
               if (COUNT) cd += in ? 1 : 0;
             }
@@ -690,59 +1172,20 @@ __device__ __forceinline__ void cpair_body(const ClusterArgs &a, int bx, int nbx
             }
             if (vd && hh < 3) {
               const real v = hh == 0 ? fdx : (hh == 1 ? fdy : fdz);
-              long long *dst = a.facc + (int64_t)hh * N + p0 + t;
-              if (F64) fx_add(dst, (double)v, a.fscale_d, a.err);
-              else fx_add(dst, (float)v, a.fscale, a.err);
+              fx_add(a.facc + (int64_t)hh * N + p0 + t, v, a.fscale_d, a.err);
             }
             if (COUNT && vd && hh == 3 && cd) atomicAdd(a.nbr + p0 + t, cd);
           }
 #pragma unroll
           for (int c = 0; c < NC; ++c) {
             if ((Mh >> c) & 1u) {
-              const float4 pi4 = F64 ? make_float4(0.f, 0.f, 0.f, 0.f) : sif[kClSize * c + a8];
 #pragma unroll
               for (int k = 0; k < 2; ++k) {
                 real dx, dy, dz;
                 bool in;
-                const real g = pair_one(!F64 || vi[c], (real)pi4.x, (real)pi4.y, (real)pi4.z,
-                                        oxi[c], oyi[c], ozi[c], COUL && !F64 ? (real)pi4.w : qi[c],
-                                        ti[c], k, dx, dy, dz, in);
+                const real g = pair_one(vi[c], oxi[c], oyi[c], ozi[c], qi[c], ti[c], k, dx, dy, dz, in);
                 fxi[c] = mad(g, dx, fxi[c]); fyi[c] = mad(g, dy, fyi[c]); fzi[c] = mad(g, dz, fzi[c]);
                 if (COUNT) cnti[c] += in ? 1 : 0;
-              }
-            }
-          }
-          // Band pairs (FP32 forms): the exact decision; a pair inside is added by atomics.
-          if (!F64 && __any_sync(FULL, bmin <= a.rc2_half)) {
-            for (int c = cb; c < ce; ++c) {
-              if (!((M >> c) & 1u)) continue;
-              const int t = kClSize * c + a8;
-              if (t >= np || (asub >= 0 && a8 != asub)) continue;
-              const uint4 s = si[t];
-              const float x0 = (float)(int)(s.x - rx) * pc.h[0];
-              const float y0 = (float)(int)(s.y - ry) * pc.h[1];
-              const float z0 = (float)(int)(s.z - rz) * pc.h[2];
-              for (int k = 0; k < 2; ++k) {
-                if (!vj[k] || !(c != cdiag || a8 < hh + 4 * k)) continue;
-                const float dx = x0 - (float)xj[k], dy = y0 - (float)yj[k], dz = z0 - (float)zj[k];
-                const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                if (!(r2 >= pc.rc2_lo && r2 <= pc.rc2_hi)) continue;
-                const int pj = vb + hh + 4 * k;
-                const int dsx = (int)(s.x - a.set.sx[pj]), dsy = (int)(s.y - a.set.sy[pj]),
-                          dsz = (int)(s.z - a.set.sz[pj]);
-                if (!(exact_r2(pc, dsx, dsy, dsz) <= pc.rc2d)) continue;
-                const real qis = COUL ? (real)__uint_as_float(s.w) : (real)0;
-                const real g = cp_terms<real, COUL, MULTI>(a, true, (real)r2, (real)rcp_approx(r2),
-                                                           qis, qj[k], MULTI ? sti[t] : 0, tj[k],
-                                                           acc);
-                const int pi = p0 + t;
-                fx_add(a.facc + pi, (float)(g * dx), a.fscale, a.err);
-                fx_add(a.facc + N + pi, (float)(g * dy), a.fscale, a.err);
-                fx_add(a.facc + 2 * N + pi, (float)(g * dz), a.fscale, a.err);
-                fx_add(a.facc + pj, (float)(-g * dx), a.fscale, a.err);
-                fx_add(a.facc + N + pj, (float)(-g * dy), a.fscale, a.err);
-                fx_add(a.facc + 2 * N + pj, (float)(-g * dz), a.fscale, a.err);
-                if (COUNT) { atomicAdd(a.nbr + pi, 1); atomicAdd(a.nbr + pj, 1); }
               }
             }
           }
@@ -771,9 +1214,7 @@ __device__ __forceinline__ void cpair_body(const ClusterArgs &a, int bx, int nbx
             if (a8 < 6) {
               const int k = a8 / 3, d = a8 - 3 * k;
               if (vj[k]) {
-                long long *dst = a.facc + (int64_t)d * N + vb + hh + 4 * k;
-                if (F64) fx_add(dst, (double)v, a.fscale_d, a.err);
-                else fx_add(dst, (float)v, a.fscale, a.err);
+                fx_add(a.facc + (int64_t)d * N + vb + hh + 4 * k, v, a.fscale_d, a.err);
               }
             }
           }
@@ -802,15 +1243,9 @@ __device__ __forceinline__ void cpair_body(const ClusterArgs &a, int bx, int nbx
         const int t = kClSize * c + a8;
         if ((c & 3) == hh && vi[c]) {
           const int64_t pi = p0 + t;
-          if (F64) {
-            fx_add(a.facc + pi, (double)fxi[c], a.fscale_d, a.err);
-            fx_add(a.facc + N + pi, (double)fyi[c], a.fscale_d, a.err);
-            fx_add(a.facc + 2 * N + pi, (double)fzi[c], a.fscale_d, a.err);
-          } else {
-            fx_add(a.facc + pi, (float)fxi[c], a.fscale, a.err);
-            fx_add(a.facc + N + pi, (float)fyi[c], a.fscale, a.err);
-            fx_add(a.facc + 2 * N + pi, (float)fzi[c], a.fscale, a.err);
-          }
+          fx_add(a.facc + pi, fxi[c], a.fscale_d, a.err);
+          fx_add(a.facc + N + pi, fyi[c], a.fscale_d, a.err);
+          fx_add(a.facc + 2 * N + pi, fzi[c], a.fscale_d, a.err);
           if (COUNT && cnti[c]) atomicAdd(a.nbr + pi, cnti[c]);
         }
       }
@@ -824,16 +1259,12 @@ __device__ __forceinline__ void cpair_body(const ClusterArgs &a, int bx, int nbx
     }
   }
   // block partials of the energies and virials (each pair counted once)
-  double ulj, wlj;
-  if (MULTI) {
-    ulj = (double)acc.u0;
-    wlj = (double)acc.u1;
-  } else {
-    const double A = F64 ? a.ljAd : (double)a.ljA, B = F64 ? a.ljBd : (double)a.ljB;
-    ulj = A * (double)acc.u0 - B * (double)acc.u1;
-    wlj = 12.0 * A * (double)acc.u0 - 6.0 * B * (double)acc.u1;
+  double ulj = acc.u0, wlj = acc.u1;
+  if (!MULTI) {
+    ulj = a.ljAd * acc.u0 - a.ljBd * acc.u1;
+    wlj = 12.0 * a.ljAd * acc.u0 - 6.0 * a.ljBd * acc.u1;
   }
-  double v[NQ_PAIR] = {(double)acc.uc - (double)acc.cuc, ulj, (double)acc.wc - (double)acc.cwc, wlj};
+  const double v[NQ_PAIR] = {acc.uc, ulj, acc.wc, wlj};
 #pragma unroll
   for (int k = 0; k < NQ_PAIR; ++k) {
     const double s = warp_sum(v[k]);
@@ -845,18 +1276,10 @@ __device__ __forceinline__ void cpair_body(const ClusterArgs &a, int bx, int nbx
     if (lane < NQ_PAIR) a.epart[z * NQ_PAIR + lane] = 0.0;
 }
 
-// (occupancy: 24 warps per SM for the FP32 LJ pass, fewer for the register-heavy Coulomb and
-// FP64 instances)
-#ifndef RBE_CP_MINB
-#define RBE_CP_MINB 24
-#endif
-#define RBE_CP_BOUNDS                                                                          \
-  __launch_bounds__(32, (sizeof(real) == 8 ? (COUL ? 8 : 12) : (COUL ? 12 : RBE_CP_MINB)))
-template <typename real, bool COUL, bool MULTI, bool COUNT>
-__global__ void RBE_CP_BOUNDS cpair_kernel(const ClusterArgs a) {
-  cpair_body<real, COUL, MULTI, COUNT>(a, (int)blockIdx.x, (int)gridDim.x);
+template <bool COUL, bool MULTI, bool COUNT>
+__global__ void __launch_bounds__(32, COUL ? 8 : 12) cpair64_kernel(const ClusterArgs a) {
+  cpair64_body<COUL, MULTI, COUNT>(a, (int)blockIdx.x, (int)gridDim.x);
 }
-#undef RBE_CP_BOUNDS
 
 // ---------------------------------------------------------------------------------------
 // Host side
@@ -864,9 +1287,31 @@ __global__ void RBE_CP_BOUNDS cpair_kernel(const ClusterArgs a) {
 int cpair_nc(const Ctx &c) { return c.precision == RBE_FP64 ? 4 : 8; }
 
 // Upper bound of the super-clusters of N particles in the rows of the grid.
-int64_t cpair_blocks_bound(const Ctx &c) {
+static int64_t cpair_super_bound(const Ctx &c) {
   const int64_t nrows = (int64_t)c.grid.n[1] * c.grid.n[2];
   return c.N / (kClSize * cpair_nc(c)) + nrows + 1;
+}
+// FP32 forms: warps a block (they share the block's start: the super-cluster's particles and
+// stencil) and blocks a super-cluster. A super-cluster alone is a chain of some 200 visits, so
+// a box with fewer super-clusters than the GPU holds warps (28 an SM, 20 with Coulomb terms)
+// leaves SMs idle behind that chain: four warps a block, then as many blocks (at most 8) as
+// fill it. With enough super-clusters two warps a block are best: half the starts, and blocks
+// short enough for an even end. Pair phase, us, at (warps, blocks):
+//   3,000 charged (83 super-clusters):  (1,1) 529, (4,1) 150, (4,2) 86, (4,4) 55, (4,8) 43
+//   50,002 charged, two types (1,006):  (1,1) 412, (2,1) 240, (4,1) 141, (4,2) 148, (4,4) 211
+//   1,048,576, 10% charged (18,234):    (1,1) 983, (2,1) 957, (4,1) 986, (4,2) 1,137
+static void cpair_shape(const Ctx &c, int *warps, int *nsplit) {
+  *warps = *nsplit = 1;
+  if (c.precision == RBE_FP64) return;
+  const int64_t n = cpair_super_bound(c);
+  const int64_t fill = (int64_t)c.sms * (c.Nq * 2 > c.N ? kCpWarpsCoul : kCpWarpsLJ);
+  *warps = n >= fill ? 2 : kCpMaxWarps;
+  *nsplit = (int)std::min<int64_t>(8, std::max<int64_t>(1, fill / (kCpMaxWarps * n)));
+}
+int64_t cpair_blocks_bound(const Ctx &c) {
+  int warps, nsplit;
+  cpair_shape(c, &warps, &nsplit);
+  return cpair_super_bound(c) * nsplit;
 }
 int64_t cpair_clusters_bound(const Ctx &c) {
   const int64_t nrows = (int64_t)c.grid.n[1] * c.grid.n[2];
@@ -896,7 +1341,8 @@ cudaError_t launch_cluster_tables(Ctx &c) {
   if (e != cudaSuccess) return e;
   const int64_t ccap = cpair_clusters_bound(c);
   const BoundsArgs ba{c.s[b], c.s[b] + c.N, c.s[b] + 2 * c.N, c.qf[b], c.cell_start, c.grid.n[0],
-                      nrows, c.cl_base, ccap, c.cl_lo, c.cl_hi, c.cjrec, c.pc.h[1], c.pc.h[2]};
+                      nrows, c.cl_base, ccap, c.cl_lo, c.cl_hi, c.cjrec, c.pc.h[1], c.pc.h[2],
+                      c.sc_base, cpair_nc(c), c.sc_info};
   return dispatch(c, cluster_bounds_kernel, cluster_bounds_kernel_b,
                   dim3((unsigned)((kClSize * ccap + 255) / 256)), dim3(256), 0, ba);
 }
@@ -916,12 +1362,15 @@ cudaError_t launch_cluster_pair(Ctx &c, bool coul, bool multi, bool want_counts)
   a.ljA = c.lj.A[0]; a.ljB = c.lj.B[0]; a.ljA12 = c.lj.A12[0]; a.ljB6 = c.lj.B6[0];
   a.ljAd = c.lj.Ad[0]; a.ljBd = c.lj.Bd[0]; a.ljA12d = c.lj.A12d[0]; a.ljB6d = c.lj.B6d[0];
   a.table = reinterpret_cast<const LJTable *>(c.lj_dev);
-  a.cl_base = c.cl_base; a.sc_base = c.sc_base; a.cl_lo = c.cl_lo; a.cl_hi = c.cl_hi;
+  a.cl_base = c.cl_base; a.sc_base = c.sc_base; a.sc_info = c.sc_info; a.cl_lo = c.cl_lo; a.cl_hi = c.cl_hi;
   a.jrec = c.cjrec;
   a.nrows = nrows;
   a.facc = c.facc;
   a.N = c.N;
+  for (int d = 0; d < 2; ++d) a.wfix[d] = ((int64_t)1 << 48) / c.grid.n[d + 1];
   a.fscale = (float)kFixScale32;
+  a.kappa = c.lj.A12[0] > 0.f ? (float)(c.lj.B6d[0] / c.lj.A12d[0]) : 0.f;
+  a.fscale_lj = (float)(kFixScale32 * c.lj.A12d[0]);
   a.fscale_d = kFixScale64;
   a.epart = c.epart + c.off_pair;
   a.nbr = want_counts ? c.nbr : nullptr;
@@ -961,20 +1410,31 @@ cudaError_t launch_cluster_pair(Ctx &c, bool coul, bool multi, bool want_counts)
   // a block per possible super-cluster (blocks past the last one, and each block for the
   // slots past the grid, write zeros to the pass's partial range)
   a.nslots = c.n_pair_blk;
-  const dim3 g((unsigned)std::min<int64_t>(c.n_pair_blk, cpair_blocks_bound(c))), bl(32);
+  int warps;
+  cpair_shape(c, &warps, &a.nsplit);
+  const dim3 g((unsigned)cpair_blocks_bound(c)), bl(32, warps);
+  const size_t shm = (size_t)warps * 32 * (sizeof(uint4) + sizeof(float));
   const bool fp64 = c.precision == RBE_FP64;
+  a.fit = c.fit;
   cudaError_t e;
   // (per replica in a batch)
-#define RBE_CP_LAUNCH(R, CO, MU)                                                             \
-  e = want_counts ? dispatch(c, cpair_kernel<R, CO, MU, true>, nullptr, g, bl, 0, a, true)   \
-                  : dispatch(c, cpair_kernel<R, CO, MU, false>, nullptr, g, bl, 0, a, true)
+#define RBE_CP_LAUNCH(CO, MU)                                                               \
+  e = want_counts ? dispatch(c, cpair32_kernel<CO, MU, true>, nullptr, g, bl, shm, a, true) \
+                  : dispatch(c, cpair32_kernel<CO, MU, false>, nullptr, g, bl, shm, a, true)
+#define RBE_CP_LAUNCH64(CO, MU)                                                           \
+  e = want_counts ? dispatch(c, cpair64_kernel<CO, MU, true>, nullptr, g, bl, 0, a, true) \
+                  : dispatch(c, cpair64_kernel<CO, MU, false>, nullptr, g, bl, 0, a, true)
   if (fp64) {
-    if (coul) { if (multi) RBE_CP_LAUNCH(double, true, true); else RBE_CP_LAUNCH(double, true, false); }
-    else { if (multi) RBE_CP_LAUNCH(double, false, true); else RBE_CP_LAUNCH(double, false, false); }
+    if (coul) { if (multi) RBE_CP_LAUNCH64(true, true); else RBE_CP_LAUNCH64(true, false); }
+    else { if (multi) RBE_CP_LAUNCH64(false, true); else RBE_CP_LAUNCH64(false, false); }
+  } else if (coul && c.fit.ok) {
+    if (multi) RBE_CP_LAUNCH(1, true); else RBE_CP_LAUNCH(1, false);
+  } else if (coul) {
+    if (multi) RBE_CP_LAUNCH(2, true); else RBE_CP_LAUNCH(2, false);
   } else {
-    if (coul) { if (multi) RBE_CP_LAUNCH(float, true, true); else RBE_CP_LAUNCH(float, true, false); }
-    else { if (multi) RBE_CP_LAUNCH(float, false, true); else RBE_CP_LAUNCH(float, false, false); }
+    if (multi) RBE_CP_LAUNCH(0, true); else RBE_CP_LAUNCH(0, false);
   }
+#undef RBE_CP_LAUNCH64
 #undef RBE_CP_LAUNCH
   return e;
 }

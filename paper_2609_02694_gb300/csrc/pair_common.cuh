@@ -3,6 +3,7 @@
 #pragma once
 #include <cuda_fp16.h>
 
+#include "f32x2.cuh"
 #include "rbe_internal.cuh"
 
 namespace rbe {
@@ -66,6 +67,28 @@ __device__ __forceinline__ void kahan_add(real &s, real &c, real x) {
   const real t = s + y;
   c = (t - s) - y;
   s = t;
+}
+
+// erfc(sqrt(alpha) r) and exp(-alpha r^2) of a packed pair, r <= r_c, by the handle's fit
+// (f.ok). The exponent's rounding and alpha log2(e)'s low part go into a linear correction, so
+// the exponential is as close as the unit's 2^x (2 ulp). A third of erfcf and expf's
+// instructions: the Coulomb pair terms were two thirds of a charged pair.
+__device__ __forceinline__ float ex2_approx(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ void erfc_exp2(const ErfcFit &f, f32x2 r, f32x2 r2, f32x2 &er,
+                                          f32x2 &ex) {
+  const f32x2 t = fma2(r, pk(f.ts), pk(-1.f));
+  f32x2 p = pk(f.c[kErfcDeg]);
+#pragma unroll
+  for (int k = kErfcDeg - 1; k >= 0; --k) p = fma2(p, t, pk(f.c[k]));
+  const f32x2 nea = pk(-f.ea), arg = mul2(r2, pk(f.ea));
+  const f32x2 d = fma2(r2, pk(-f.ea_lo), fma2(r2, nea, arg));
+  const f32x2 e = pk(ex2_approx(-arg.x), ex2_approx(-arg.y));
+  ex = fma2(e, mul2(d, pk(0.693147181f)), e);
+  er = mul2(ex, p);
 }
 
 // Squared distance of the exact cutoff decision (the oracle's definition): dx_d =

@@ -84,6 +84,50 @@ void axis_table(double L, double alpha, int M, std::vector<uint64_t> &T, double 
   Z = z;
 }
 
+// Chebyshev interpolant of erfcx(z) = exp(z^2) erfc(z) on z in [0, sqrt(alpha) r_top], as a
+// polynomial in t = 2 z / z_top - 1, kept when it deviates by less than 1e-7 relative.
+void erfc_fit(double alpha, double rc, ErfcFit &f) {
+  constexpr int n = kErfcDeg + 1;
+  const double r_top = rc * (1.0 + 1e-4), z_top = std::sqrt(alpha) * r_top;
+  f.ts = (float)(2.0 / r_top);
+  const double c2 = alpha / std::log(2.0);
+  f.ea = (float)c2;
+  f.ea_lo = (float)(c2 - (double)f.ea);
+  f.ok = 0;
+  if (!(z_top < 5.0)) return;
+  auto erfcx = [&](double t) {
+    const double z = 0.5 * (t + 1.0) * z_top;
+    return std::exp(z * z) * std::erfc(z);
+  };
+  double node[n], cheb[n], mono[n] = {}, tm[n] = {}, tc[n] = {}, tn[n];
+  for (int k = 0; k < n; ++k) node[k] = erfcx(std::cos(kPi * (k + 0.5) / n));
+  for (int j = 0; j < n; ++j) {
+    double s = 0.0;
+    for (int k = 0; k < n; ++k) s += node[k] * std::cos(kPi * j * (k + 0.5) / n);
+    cheb[j] = s * (j == 0 ? 1.0 : 2.0) / n;
+  }
+  tm[0] = 1.0;  // T_0 and T_1, then T_{j+1} = 2 t T_j - T_{j-1}
+  tc[1] = 1.0;
+  for (int k = 0; k < n; ++k) mono[k] = cheb[0] * tm[k] + cheb[1] * tc[k];
+  for (int j = 2; j < n; ++j) {
+    for (int k = 0; k < n; ++k) tn[k] = (k ? 2.0 * tc[k - 1] : 0.0) - tm[k];
+    for (int k = 0; k < n; ++k) {
+      mono[k] += cheb[j] * tn[k];
+      tm[k] = tc[k];
+      tc[k] = tn[k];
+    }
+  }
+  for (int k = 0; k < n; ++k) f.c[k] = (float)mono[k];
+  double worst = 0.0;
+  for (int i = 0; i <= 120; ++i) {  // eight points between the interpolation's zeros
+    const double t = i / 60.0 - 1.0;
+    double p = mono[n - 1];
+    for (int k = n - 2; k >= 0; --k) p = p * t + mono[k];
+    worst = std::max(worst, std::fabs(p / erfcx(t) - 1.0));
+  }
+  f.ok = worst < 1e-7 ? 1 : 0;
+}
+
 uint32_t quantise(double r, double L) {
   const double f = (r / L) * kTwo32;
   const double fm = f - kTwo32 * std::floor(f / kTwo32);
@@ -122,7 +166,7 @@ int free_all(Ctx &c) {
     if (c.fgraph[b]) cudaGraphExecDestroy(c.fgraph[b]);
     c.fgraph[b] = nullptr;
   }
-  dfree(c.F); dfree(c.Fd); dfree(c.facc); dfree(c.cl_base); dfree(c.sc_base); dfree(c.cl_lo);
+  dfree(c.F); dfree(c.Fd); dfree(c.facc); dfree(c.cl_base); dfree(c.sc_base); dfree(c.sc_info); dfree(c.cl_lo);
   dfree(c.cl_hi); dfree(c.cjrec); dfree(c.cq4); dfree(c.cs); dfree(c.cqf); dfree(c.cqd); dfree(c.cmap);
   dfree(c.cell_count); dfree(c.cell_start); dfree(c.key); dfree(c.off); dfree(c.tmp);
   dfree(c.scan_blk);
@@ -445,6 +489,7 @@ int rbe_init(rbe_handle *hout, const rbe_params *p, int64_t N, const double box[
   c.pc.C_d = c.C; c.pc.C = (float)c.C;
   c.pc.two_sqrt_alpha_over_sqrt_pi_d = 2.0 * std::sqrt(c.alpha) / std::sqrt(kPi);
   c.pc.two_sqrt_alpha_over_sqrt_pi = (float)c.pc.two_sqrt_alpha_over_sqrt_pi_d;
+  erfc_fit(c.alpha, c.rc, c.fit);
   // LJ table
   c.lj.nt = c.nt;
   for (int a = 0; a < c.nt; ++a)
@@ -527,6 +572,7 @@ int rbe_init(rbe_handle *hout, const rbe_params *p, int64_t N, const double box[
     rc |= dalloc(c, &c.facc, 3 * N);
     rc |= dalloc(c, &c.cl_base, nrows + 1);
     rc |= dalloc(c, &c.sc_base, nrows + 1);
+    rc |= dalloc(c, &c.sc_info, cpair_blocks_bound(c));
     rc |= dalloc(c, &c.cl_lo, cpair_clusters_bound(c));
     rc |= dalloc(c, &c.cl_hi, cpair_clusters_bound(c));
     if (!fp64) rc |= dalloc(c, &c.cjrec, 8 * cpair_clusters_bound(c));  // 8 slots per cluster

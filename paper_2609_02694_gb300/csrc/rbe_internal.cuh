@@ -74,6 +74,18 @@ struct PairConst {
   double two_sqrt_alpha_over_sqrt_pi_d;
 };
 
+// erfc(z) = exp(-z^2) erfcx(z) with erfcx(z), z = sqrt(alpha) r, as one polynomial in
+// t = r ts - 1 in [-1, 1] for r <= r_c: the Chebyshev interpolant of degree 14, formed on the
+// host in FP64 (erfc_fit). `ok`: within 1e-7 of erfcx over the range (z up to about 3.7); a
+// larger sqrt(alpha) r_c takes erfcf and expf.
+constexpr int kErfcDeg = 14;
+struct ErfcFit {
+  float c[kErfcDeg + 1];
+  float ts;            // 2 / r_c, widened to the top of the exact-decision band
+  float ea, ea_lo;     // alpha log2(e), high and low part
+  int ok;
+};
+
 struct Ctx {
   // --- parameters
   int64_t N = 0, Nq = 0;
@@ -94,6 +106,7 @@ struct Ctx {
   LJTable lj{};
   void *lj_dev = nullptr;     // device copy of lj (multi-type pair kernels)
   PairConst pc{};
+  ErfcFit fit{};
   // --- particle arrays
   int cur = 0;
   uint32_t *s[2] = {nullptr, nullptr};
@@ -110,6 +123,7 @@ struct Ctx {
   // super-cluster offsets (rows + 1 each), per-cluster bounds
   long long *facc = nullptr;
   int32_t *cl_base = nullptr, *sc_base = nullptr;
+  int4 *sc_info = nullptr;     // per super-cluster: row, first cluster and particle, counts
   uint4 *cl_lo = nullptr, *cl_hi = nullptr;
   uint4 *cjrec = nullptr;      // the cluster kernel's j records, 8 slots per cluster, written
                                // with the cluster boxes (FP32 forms)
