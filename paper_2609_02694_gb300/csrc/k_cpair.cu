@@ -29,7 +29,8 @@
 // visited j particle's x is converted the same way; its y and z are the frame coordinates of
 // its cluster's box corner plus its FP32 offsets from that corner, stored per step in the
 // cluster's eight record slots (a cluster lies in one cell in y and z, so the offsets are
-// small and never wrap; the one extra rounding widens the band below).
+// small and never wrap; a cluster across the frame's edge counts from the side in reach; the
+// one extra rounding widens the band below).
 // The difference of two offsets is the minimum-image displacement of a pair within r_c as
 // long as the super-cluster's extent plus 2 r_c stays below L on every axis: the host
 // checks y and z (a cell width), the kernel splits a super-cluster whose x extent is
@@ -285,12 +286,6 @@ __global__ void __launch_bounds__(256)
 // ---------------------------------------------------------------------------------------
 // Pair evaluation
 
-__device__ __forceinline__ float rcp_approx(float x) {
-  float y;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 struct CpAcc {
   double u0, u1;  // single type: sum r^-12, sum r^-6; several types: U_LJ, W_LJ
   double uc, wc;  // Coulomb energy and virial
@@ -443,16 +438,6 @@ __device__ __forceinline__ int cp_segments(const ClusterArgs &a, int lane, int c
 // the pair loop about 120 instructions, its branches 24, the loads and conversions 38, the
 // reaction 31.
 
-__device__ __forceinline__ float min3(float a, float b, float c) {
-  float r;
-  asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-  return r;
-}
-__device__ __forceinline__ float max3(float a, float b, float c) {
-  float r;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-  return r;
-}
 // 1.0 where a < b, else 0.0
 __device__ __forceinline__ float lt_one(float a, float b) {
   float r;
@@ -636,7 +621,7 @@ __device__ __forceinline__ void cpair32_body(const ClusterArgs &a, int bx, int n
         const int cc = base + lane * nparts;
         uint32_t msk = 0u;
         int J = 0, jb = 0, jn = 0;
-        float jy0 = 0.f, jz0 = 0.f;  // the candidate box's low corner in y and z (frame)
+        float cy0 = 0.f, cz0 = 0.f;  // the candidate box's low corner in y and z (frame)
         if (cc < T) {
           int s = 0, e = nseg;       // the candidate's run: the last one starting at or before it
           while (e - s > 1) {
@@ -648,8 +633,10 @@ __device__ __forceinline__ void cpair32_body(const ClusterArgs &a, int bx, int n
           jb = (int)l.w;
           jn = (int)u.w;
           const float jx0 = (float)(int)(l.x - rx) * pc.h[0];
-          jy0 = (float)(int)(l.y - ry) * pc.h[1];
-          jz0 = (float)(int)(l.z - rz) * pc.h[2];
+          const float jy0 = (float)(int)(l.y - ry) * pc.h[1];
+          const float jz0 = (float)(int)(l.z - rz) * pc.h[2];
+          cy0 = jy0;
+          cz0 = jz0;
           const float jx1 = (float)(int)(u.x - rx) * pc.h[0];
           const float jy1 = (float)(int)(u.y - ry) * pc.h[1];
           const float jz1 = (float)(int)(u.z - rz) * pc.h[2];
@@ -668,6 +655,12 @@ __device__ __forceinline__ void cpair32_body(const ClusterArgs &a, int bx, int n
               msk |= fmaf(gx, gx, fmaf(gy, gy, gz * gz)) <= a.bb2 ? (1u << c) : 0u;
             }
           } else {
+            // (a box that straddles the frame's edge in y or z by its lower piece, nearer the
+            // group: its corner counts from below, so that corner plus offset stays in reach)
+            if (wy && (float)(int)(ylo - ry) * pc.h[1] - jy1 < jy0 - (float)(int)(yhi - ry) * pc.h[1])
+              cy0 = jy0 - 4294967296.f * pc.h[1];
+            if (wz && (float)(int)(zlo - rz) * pc.h[2] - jz1 < jz0 - (float)(int)(zhi - rz) * pc.h[2])
+              cz0 = jz0 - 4294967296.f * pc.h[2];
             for (int c = 0; c < NC; ++c) {
               const float4 bxy = ibl[c];
               const float2 bz = ibz[c];
@@ -688,8 +681,8 @@ __device__ __forceinline__ void cpair32_body(const ClusterArgs &a, int bx, int n
         if (msk) {
           const int k = __popc(vis & ((1u << lane) - 1u));
           rec[k] = make_uint4((uint32_t)J, msk | ((uint32_t)jn << 8), (uint32_t)jb,
-                              __float_as_uint(-jy0));
-          recz[k] = -jz0;
+                              __float_as_uint(-cy0));
+          recz[k] = -cz0;
         }
         __syncwarp();
         const int nv = __popc(vis);

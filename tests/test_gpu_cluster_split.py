@@ -55,3 +55,21 @@ def test_erfc_fit_and_fallback_match_oracle(orc, alpha):
     ref = orc.total_forces(sy.s, sy.q, sy.types, sy.box, alpha, RC, C, sy.eps, sy.sig, m, S)
     assert rel_l2(F, ref["F"]) < 1e-5
     assert E["real"] == pytest.approx(ref["U_real"], rel=1e-5)
+
+
+@pytest.mark.parametrize("box,n", [((27.2, 27.2, 27.2), 2001), ((25.7, 25.6, 25.8), 1701),
+                                   ((60.0, 27.0, 26.0), 4201), ((34.2, 31.0, 28.2), 3000)])
+@pytest.mark.parametrize("all_charged", [False, True])
+def test_five_cell_boxes_match_oracle(orc, box, n, all_charged):
+    """Boxes of five cells of r_c / 2 in y or z: stencil rows reach past the frame's edge, and
+    clusters lie across it."""
+    sy = synth.make_system(n, L=box[0], seed=12, all_charged=all_charged)
+    sy.box = np.array(box)
+    with binding.from_system(sy, P=40, alpha=ALPHA, r_c=RC) as h:
+        F, E, _ = h.forces_f64(2)
+        nbr, _ = h.neighbor_counts()
+        m, S = sampled.oracle_modes(orc, h, sy, 40, 2)
+    ref = orc.total_forces(sy.s, sy.q, sy.types, sy.box, ALPHA, RC, C, sy.eps, sy.sig, m, S)
+    assert np.array_equal(nbr, ref["nbr"])
+    assert rel_l2(F, ref["F"]) < 1e-5
+    assert E["lj"] == pytest.approx(ref["U_lj"], rel=2e-6)
