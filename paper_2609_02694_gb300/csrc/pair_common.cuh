@@ -69,6 +69,21 @@ __device__ __forceinline__ void kahan_add(real &s, real &c, real x) {
   s = t;
 }
 
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float min3(float a, float b, float c) {
+  float r;
+  asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
 // erfc(sqrt(alpha) r) and exp(-alpha r^2) of a packed pair, r <= r_c, by the handle's fit
 // (f.ok). The exponent's rounding and alpha log2(e)'s low part go into a linear correction, so
 // the exponential is as close as the unit's 2^x (2 ulp). A third of erfcf and expf's

@@ -607,8 +607,10 @@ int rbe_init(rbe_handle *hout, const rbe_params *p, int64_t N, const double box[
     rc |= dalloc(c, &c.nshell, N);
     rc |= dalloc(c, &c.partners, N * c.p_rbl);
     rc |= dalloc(c, &c.rbl_part, c.n_rbl_blk * 3);
-    rc |= dalloc(c, &c.rbl_masks, rbl_mask_words(c.rbl_nslots));
-    rc |= dalloc(c, &c.rbl_slots, c.rbl_nslots);
+    if (fp64) {
+      rc |= dalloc(c, &c.rbl_masks, rbl_mask_words(c.rbl_nslots));
+      rc |= dalloc(c, &c.rbl_slots, c.rbl_nslots);
+    }
     rc |= dalloc(c, &c.rbl_cpart, rbl_compact_count(c.n_rbl_blk) * (NQ_PAIR + 3));
   }
   rc |= dalloc(c, &c.rbl_mean, 3);
