@@ -143,12 +143,10 @@ __device__ __forceinline__ void coul_body(const CoulArgs a, int bx, int) {
         const int4 e = buf[wid][lane];
         real dx, dy, dz, r2, qj;
         if (F64) {
-          dx = (real)__dmul_rn((double)e.x, pc.hd[0]);
-          dy = (real)__dmul_rn((double)e.y, pc.hd[1]);
-          dz = (real)__dmul_rn((double)e.z, pc.hd[2]);
-          r2 = (real)__dadd_rn(__dadd_rn(__dmul_rn((double)dx, (double)dx),
-                                         __dmul_rn((double)dy, (double)dy)),
-                               __dmul_rn((double)dz, (double)dz));
+          dx = (real)(i2d(e.x) * pc.hd[0]);
+          dy = (real)(i2d(e.y) * pc.hd[1]);
+          dz = (real)(i2d(e.z) * pc.hd[2]);
+          r2 = mad(dx, dx, mad(dy, dy, dz * dz));
           qj = (real)a.qd[e.w];
         } else {
           dx = (real)((float)e.x * pc.h[0]);
@@ -159,8 +157,12 @@ __device__ __forceinline__ void coul_body(const CoulArgs a, int bx, int) {
         }
         real r, rinv, erfcv, expv;
         if (F64) {
-          r = (real)sqrt((double)r2);
-          rinv = (real)1 / r;
+          // 1/r from an FP32 start by one third-order Householder step (as in the pair kernel)
+          const float ex = (float)e.x * pc.h[0], ey = (float)e.y * pc.h[1], ez = (float)e.z * pc.h[2];
+          const double z = f2d(rsqrtf(fmaf(ex, ex, fmaf(ey, ey, ez * ez))));
+          const double c = fma(-((double)r2 * z), z, 1.0);
+          rinv = (real)fma(z, c * fma(c, 0.375, 0.5), z);
+          r = r2 * rinv;
           erfcv = (real)erfc(pc.sqrt_alpha_d * (double)r);
           expv = (real)exp(-pc.alpha_d * (double)r2);
         } else {
@@ -202,15 +204,11 @@ __device__ __forceinline__ void coul_body(const CoulArgs a, int bx, int) {
         if (j != i) {
           const uint4 pj = a.s4[j];
           const int dsx = (int)(pi.x - pj.x), dsy = (int)(pi.y - pj.y), dsz = (int)(pi.z - pj.z);
-          if (F64) {
-            hit = exact_r2(pc, dsx, dsy, dsz) <= pc.rc2d;
-          } else {
-            const float ex = (float)dsx * pc.h[0], ey = (float)dsy * pc.h[1],
-                        ez = (float)dsz * pc.h[2];
-            const float r2 = mad(ex, ex, mad(ey, ey, ez * ez));
-            hit = r2 < pc.rc2_lo;
-            if (r2 >= pc.rc2_lo && r2 <= pc.rc2_hi) hit = exact_r2(pc, dsx, dsy, dsz) <= pc.rc2d;
-          }
+          const float ex = (float)dsx * pc.h[0], ey = (float)dsy * pc.h[1],
+                      ez = (float)dsz * pc.h[2];
+          const float r2 = mad(ex, ex, mad(ey, ey, ez * ez));
+          hit = r2 < pc.rc2_lo;
+          if (r2 >= pc.rc2_lo && r2 <= pc.rc2_hi) hit = exact_r2(pc, dsx, dsy, dsz) <= pc.rc2d;
           rec = make_int4(dsx, dsy, dsz, F64 ? (int)j : (int)pj.w);
         }
       }
@@ -246,8 +244,10 @@ __device__ __forceinline__ void coul_body(const CoulArgs a, int bx, int) {
     }
   }
   // block partials of the Coulomb energy and virial (halves of the per-i sums)
-  const double u = warp_sum((double)uc - (double)cuc), w = warp_sum((double)wc - (double)cwc);
-  if (lane == 0) { wred[wid][0] = u; wred[wid][1] = w; }
+  const double us = F64 ? (double)uc : f2d((float)uc) - f2d((float)cuc);
+  const double ws = F64 ? (double)wc : f2d((float)wc) - f2d((float)cwc);
+  const double uw = warp_sum2(us, ws, lane);
+  if (lane < 2) wred[wid][lane] = uw;
   __syncthreads();
   if (threadIdx.x < NQ_PAIR) {
     double s = 0.0;

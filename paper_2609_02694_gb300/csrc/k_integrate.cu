@@ -156,7 +156,7 @@ __device__ __forceinline__ void kick_body(const KickArgs<V, FT> &a, int bx, int)
     // 1/2 m v^2 / kappa, m = 1 / (1/m): FP64 in the FP64 form; the FP32 forms form each
     // particle's term in FP32 and sum the terms in FP64
     if (sizeof(V) == 8) ke = 0.5 * (double)v2 / (double)invm[i] * inv_kappa;
-    else ke = (double)(0.5f * (float)v2 * __frcp_rn(invm[i]) * (float)inv_kappa);
+    else ke = f2d(0.5f * (float)v2 * __frcp_rn(invm[i]) * (float)inv_kappa);
   }
   sh[threadIdx.x] = ke;
   __syncthreads();
@@ -199,10 +199,10 @@ __device__ __forceinline__ void kick4_body(const KickArgs<float, float> &a, int 
       v2[2] += vv.z * vv.z;
       v2[3] += vv.w * vv.w;
     }
-    ke[0] = (double)(0.5f * v2[0] * __frcp_rn(im.x) * ik);
-    ke[1] = (double)(0.5f * v2[1] * __frcp_rn(im.y) * ik);
-    ke[2] = (double)(0.5f * v2[2] * __frcp_rn(im.z) * ik);
-    ke[3] = (double)(0.5f * v2[3] * __frcp_rn(im.w) * ik);
+    ke[0] = f2d(0.5f * v2[0] * __frcp_rn(im.x) * ik);
+    ke[1] = f2d(0.5f * v2[1] * __frcp_rn(im.y) * ik);
+    ke[2] = f2d(0.5f * v2[2] * __frcp_rn(im.z) * ik);
+    ke[3] = f2d(0.5f * v2[3] * __frcp_rn(im.w) * ik);
   }
 #pragma unroll
   for (int j = 0; j < 4; ++j) sh[4 * t + j] = ke[j];

@@ -70,9 +70,8 @@ constexpr int kListUnroll = 4;
 
 template <typename real, bool LJ, bool COUL, bool MULTI>
 __global__ void __launch_bounds__(kPairWarps * 32) list_pair_kernel(const ListArgs la) {
-  __shared__ double wred[kPairWarps][NQ_PAIR];
   const PairArgs &a = la.pa;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
   const unsigned FULL = 0xffffffffu;
   const int64_t n = a.set.n;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -105,7 +104,7 @@ __global__ void __launch_bounds__(kPairWarps * 32) list_pair_kernel(const ListAr
       real qj = (real)0;
       if (COUL) qj = sizeof(real) == 8 ? (real)a.set.qd[jj[u]] : (real)__uint_as_float(pj[u].w);
       const int tj = MULTI ? a.set.type[jj[u]] : 0;
-      pair_eval_masked<real, LJ, COUL, MULTI>(a, tab, ac[u], (int)(pi.x - pj[u].x),
+      pair_eval_masked<LJ, COUL, MULTI, false>(a, tab, ac[u], (int)(pi.x - pj[u].x),
                                               (int)(pi.y - pj[u].y), (int)(pi.z - pj[u].z),
                                               qi, ti, qj, tj, acc);
     }
@@ -113,6 +112,9 @@ __global__ void __launch_bounds__(kPairWarps * 32) list_pair_kernel(const ListAr
   if (valid) {
     const int64_t o = a.set.map ? (int64_t)a.set.map[i] : i;
     const int64_t S = a.Fstride;
+    if (sizeof(real) == 8) {  // (to length units)
+      acc.fx *= (real)a.fs[0]; acc.fy *= (real)a.fs[1]; acc.fz *= (real)a.fs[2];
+    }
     if (sizeof(real) == 8) {
       if (a.accumulate) { a.Fd[o] += (double)acc.fx; a.Fd[S + o] += (double)acc.fy; a.Fd[2 * S + o] += (double)acc.fz; }
       else { a.Fd[o] = (double)acc.fx; a.Fd[S + o] = (double)acc.fy; a.Fd[2 * S + o] = (double)acc.fz; }
@@ -122,19 +124,13 @@ __global__ void __launch_bounds__(kPairWarps * 32) list_pair_kernel(const ListAr
     }
     if (a.nbr) a.nbr[i] = acc.nbr;
   }
-  double v[NQ_PAIR] = {(double)acc.uc - (double)acc.cuc, (double)acc.ulj,
-                       (double)acc.wc - (double)acc.cwc, (double)acc.wlj};
-#pragma unroll
-  for (int k = 0; k < NQ_PAIR; ++k) {
-    const double w = warp_sum(v[k]);
-    if (lane == 0) wred[wid][k] = w;
-  }
-  __syncthreads();
-  if (threadIdx.x < NQ_PAIR) {
-    double s = 0.0;
-    for (int w = 0; w < kPairWarps; ++w) s += wred[w][threadIdx.x];
-    a.epart[(int64_t)blockIdx.x * NQ_PAIR + threadIdx.x] = 0.5 * s;
-  }
+  double ulj = (double)acc.ulj, wlj = (double)acc.wlj;
+  if (LJ && sizeof(real) == 8 && !MULTI)
+    grid_energies(a, (double)acc.ulj, (double)acc.wlj, ulj, wlj);
+  const double v[8] = {(double)acc.uc - (double)acc.cuc, ulj, (double)acc.wc - (double)acc.cwc, wlj,
+                       0.0, 0.0, 0.0, 0.0};
+  const double s = warp_sum8(v, lane);  // (kPairWarps is 1)
+  if (lane < NQ_PAIR) a.epart[(int64_t)blockIdx.x * NQ_PAIR + lane] = 0.5 * s;
 }
 
 static inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
@@ -187,6 +183,7 @@ cudaError_t launch_list_pair(Ctx &c, bool want_counts) {
   a.epart = c.epart + c.off_pair;
   a.nbr = want_counts ? c.nbr : nullptr;
   a.comp = c.precision == RBE_FP32_COMP;
+  set_grid_units(c, a);
   a.list = c.vl_list; a.len = c.vl_len; a.K = c.vl_K;
   la.s4 = c.s4;
   if (fused) {

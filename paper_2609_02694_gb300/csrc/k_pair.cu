@@ -38,14 +38,24 @@ namespace rbe {
 
 constexpr int kMaxRows = 49;            // (2R+1)^2 stencil rows for R <= 3
 constexpr int kMaxSeg = 2 * kMaxRows;   // a row wraps into at most two runs of cells
-constexpr int kWin = 4;                 // chunks of 32 candidates staged per window
-constexpr int kHitQ = 4;                // hit-mask queue entries per lane (at most 4 pending)
+// Chunks of 32 candidates staged at once (a power of two), and hit-mask queue entries per lane:
+// four in the FP32 forms. Sixteen in the FP64 form, where an iteration's FP64 operations cost
+// every lane's share whether it has a pair or not: the trip count follows the heaviest lane over
+// the staged chunks (65,536 particles: 2,480 us with 4, 2,151 with 8, 2,096 with 16, 2,016 with 32
+// chunks, which leave six warps an SM to charged systems).
+template <typename real>
+struct PairWin {
+  static constexpr int n = sizeof(real) == 8 ? 16 : 4;
+};
 
 // 28 warps per SM (at most 72 registers): occupancy is worth more than registers to this
 // issue-bound loop (32 warps spill and run slower). One-warp blocks: a warp that finishes
 // early frees its slot instead of waiting at a block barrier for the slowest warp.
-template <typename real, bool LJ, bool COUL, bool MULTI, bool WRAP, bool T16, bool BUILD>
+template <typename real, bool LJ, bool COUL, bool MULTI, bool WRAP, bool T16, bool BUILD,
+          bool CUBIC>
 __device__ __forceinline__ void pair_body(const PairArgs &a, int bx, int) {
+  constexpr bool HL = !BUILD && !WRAP;
+  constexpr int kWin = HL ? PairWin<real>::n : 4, kHitQ = kWin;
   __shared__ float4 stage[kPairWarps][kWin][T16 ? 1 : 32];     // FP32 test coordinates
   __shared__ uint4 stage16[kPairWarps][kWin][T16 ? 16 : 1];    // packed half test coordinates
   __shared__ int4 stage_d[kPairWarps][kWin][32];               // exact integer frame coords, type
@@ -55,15 +65,15 @@ __device__ __forceinline__ void pair_body(const PairArgs &a, int bx, int) {
   __shared__ int32_t stage_j[kPairWarps][kWin][NEEDJ ? 32 : 1];
   __shared__ int32_t seg_beg[kPairWarps][kMaxSeg];
   __shared__ int32_t seg_pre[kPairWarps][kMaxSeg + 1];
-  __shared__ double wred[kPairWarps][NQ_PAIR];
   // per-lane queues of pending hit masks: entry e of lane l holds (mask, ring slot base) of
   // one chunk with hits; entry-major, so any mix of entries costs the minimum two wavefronts
-  constexpr bool HL = !BUILD && !WRAP;
   __shared__ uint2 hitq[kPairWarps][HL ? kHitQ : 1][32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const unsigned FULL = 0xffffffffu;
   const int64_t n = a.set.n;
-  const int64_t i0 = ((int64_t)bx * kPairWarps + wid) * 32;
+  const int tile = BUILD ? bx : bx / a.nsplit, part = BUILD ? 0 : bx - tile * a.nsplit;
+  const int nsplit = BUILD ? 1 : a.nsplit;
+  const int64_t i0 = ((int64_t)tile * kPairWarps + wid) * 32;
   const int64_t i = i0 + lane;
   const bool valid = i < n;
   const LJTable *tab = a.table;
@@ -133,8 +143,11 @@ __device__ __forceinline__ void pair_body(const PairArgs &a, int bx, int) {
         int b0 = 0, l0 = 0, b1 = 0, l1 = 0;
         if (r < nrows) {
           const int dz = r / ny - R2, dy = r % ny - R1;
-          const int rz = ((gz + dz) % n2 + n2) % n2;
-          const int ry = ((gy + dy) % n1 + n1) % n1;
+          int rz = gz + dz, ry = gy + dy;  // (|dy| <= R1 < n1, |dz| <= R2 < n2)
+          rz += rz < 0 ? n2 : 0;
+          rz -= rz >= n2 ? n2 : 0;
+          ry += ry < 0 ? n1 : 0;
+          ry -= ry >= n1 ? n1 : 0;
           const int64_t rowbase = (int64_t)n0 * (ry + (int64_t)n1 * rz);
           int sa0, sb0, sa1 = 0, sb1 = -1;
           int64_t sh0 = 0, sh1 = 0;  // unwrapping shift of each segment (x past 0 or L)
@@ -152,20 +165,24 @@ __device__ __forceinline__ void pair_body(const PairArgs &a, int bx, int) {
             l1 = a.set.cell_start[rowbase + sb1 + 1] - b1;
           }
           if (trim) {
-            // the row's y and z extent in frame units (cells gy + dy, gz + dz unwrapped;
-            // edges rounded outward by 2 units), its distance from the group's box, and
-            // the x-reach left (radius widened by 1e-9, reach rounded up, +2 units)
-            const double wy = 4294967296.0 / n1, wz = 4294967296.0 / n2;
-            const double ylo = (gy + dy) * wy - (double)oy - 2.0, yhi = (gy + dy + 1) * wy - (double)oy + 2.0;
-            const double zlo = (gz + dz) * wz - (double)oz - 2.0, zhi = (gz + dz + 1) * wz - (double)oz + 2.0;
-            const double ddy = fmax(0.0, fmax(ylo - gyhi, gylo - yhi)) * a.pc.hd[1];
-            const double ddz = fmax(0.0, fmax(zlo - gzhi, gzlo - zhi)) * a.pc.hd[2];
-            const double rx2 = a.pc.rc2d * (1.0 + 1e-9) - ddy * ddy - ddz * ddz;
-            if (rx2 <= 0.0) {
+            // the row's y and z extent in frame units (cells gy + dy, gz + dz unwrapped; cell
+            // edges within 2 units up to 2^16 cells, widened by 4 or more), its distance from
+            // the group's box, and the x-reach left (an FP32 square root, widened by 2e-5).
+            // (FP64 geometry here took a fifth of the FP64 form's pair pass.)
+            const int my = 4 + (n1 >> 16), mz = 4 + (n2 >> 16);
+            const int64_t y0 = (((int64_t)(gy + dy) * a.wfix[0]) >> 16) - (int64_t)oy - my;
+            const int64_t y1 = (((int64_t)(gy + dy + 1) * a.wfix[0]) >> 16) - (int64_t)oy + my;
+            const int64_t z0 = (((int64_t)(gz + dz) * a.wfix[1]) >> 16) - (int64_t)oz - mz;
+            const int64_t z1 = (((int64_t)(gz + dz + 1) * a.wfix[1]) >> 16) - (int64_t)oz + mz;
+            const int64_t ey = max((int64_t)0, max(y0 - gyhi, (int64_t)gylo - y1));
+            const int64_t ez = max((int64_t)0, max(z0 - gzhi, (int64_t)gzlo - z1));
+            const float ddy = (float)ey * a.pc.h[1], ddz = (float)ez * a.pc.h[2];
+            const float rx2 = (float)a.pc.rc2d * (1.f + 1e-5f) - ddy * ddy - ddz * ddz;
+            if (rx2 <= 0.f) {
               l0 = l1 = 0;
             } else {
-              const double rx = ceil(sqrt(rx2) / a.pc.hd[0]) + 2.0;
-              const int64_t xlo = (int64_t)gxlo - (int64_t)rx, xhi = (int64_t)gxhi + (int64_t)rx;
+              const int64_t rx = (int64_t)(sqrtf(rx2) * (1.f + 2e-5f) / a.pc.h[0]) + 4;
+              const int64_t xlo = (int64_t)gxlo - rx, xhi = (int64_t)gxhi + rx;
               // first member of [b, b + l) at unwrapped x (s_x + shift - o_x, exact) >= key.
               // Runs are sorted by s_x; the minimum-image frame coordinate is not monotone
               // along a run (candidates beyond L/2 of the leader wrap), the unwrapped one is.
@@ -272,29 +289,33 @@ __device__ __forceinline__ void pair_body(const PairArgs &a, int bx, int) {
         //    oldest chunk works ahead on newer ones: the warp's trip count follows its
         //    heaviest lane over four chunks. Each lane evaluates its hits in a fixed order
         //    (chunks in order, within a chunk the highest candidate first).
-        //    At most four masks are queued: after a drain only the three newest chunks can
+        //    At most kWin masks are queued: after a drain only the kWin - 1 newest chunks can
         //    hold pending hits, and the chunk being tested adds one.
         int hd = 0, tl = 0, cnt = 0;  // queue read and write count, pending hits
         uint32_t cm = 0u;             // the mask being consumed (0: take the next queued one)
         int cp = 0;                   // its ring slot base (ring position * 32)
-        uint32_t q4 = 0u;             // hits per ring position (8-bit fields)
-        const int nch = (T + 31) >> 5;
+        // (this block's share of the chunks: every nsplit-th one, so that each block meets every
+        // row of the stencil and its lanes' hits stay balanced)
+        const int nall = (T + 31) >> 5, nch = nall > part ? (nall - part - 1) / nsplit + 1 : 0;
         int sg = 0;
         Cand nx;  // the next chunk's candidate of this lane, loaded ahead
         {
           int s = sg;
-          load_one(lane, s, nx);
+          load_one(32 * part + lane, s, nx);
           sg = __shfl_sync(FULL, s, 31);
         }
         for (int ch = 0; ch <= nch; ++ch) {
           const int p = ch & (kWin - 1);
           if (ch >= kWin || ch == nch) {
-            // The pending hits of ring position p (chunk ch - kWin) are the oldest ones:
-            // all pending minus those of the newer chunks. After the last chunk: all.
+            // The pending hits of ring position p (chunk ch - kWin) are the lane's oldest ones:
+            // the rest of its current mask or its next queued mask, if that is p's. After the
+            // last chunk: all.
             int need = cnt;
             if (ch < nch) {
-              const int newer = (int)((q4 * 0x01010101u) >> 24) - (int)((q4 >> (8 * p)) & 0xffu);
-              need = max(0, cnt - newer);
+              const uint2 e = hitq[wid][hd & (kHitQ - 1)][lane];
+              const bool cur = cm != 0u;
+              const bool of_p = cnt > 0 && (cur ? cp : (int)e.y) == p * 32;
+              need = of_p ? __popc(cur ? cm : e.x) : 0;
             }
             const int nit = __reduce_max_sync(FULL, need);
             const int dummy = ((ch - 1) & (kWin - 1)) * 32;  // a slot of the latest chunk
@@ -315,8 +336,8 @@ __device__ __forceinline__ void pair_body(const PairArgs &a, int bx, int) {
               real qj = (real)0;
               if (COUL) qj = sizeof(real) == 8 ? (real)a.set.qd[sj[slot]] : (real)sq[slot];
               // (the particle itself, at zero displacement, is excluded by the evaluation)
-              pair_eval_masked<real, LJ, COUL, MULTI>(a, tab, act, dsx, dsy, dsz, qi, ti, qj,
-                                                      d.w, acc);
+              pair_eval_masked<LJ, COUL, MULTI, CUBIC>(a, tab, act, dsx, dsy, dsz, qi, ti, qj, d.w,
+                                                       acc);
             }
             cnt = max(0, cnt - nit);
             __syncwarp();  // position p is free for every lane
@@ -325,7 +346,7 @@ __device__ __forceinline__ void pair_body(const PairArgs &a, int bx, int) {
           store_one(p, nx);
           if (ch + 1 < nch) {
             int s = sg;
-            load_one(32 * (ch + 1) + lane, s, nx);
+            load_one(32 * ((ch + 1) * nsplit + part) + lane, s, nx);
             sg = __shfl_sync(FULL, s, 31);
           }
           __syncwarp();
@@ -354,9 +375,7 @@ __device__ __forceinline__ void pair_body(const PairArgs &a, int bx, int) {
             hitq[wid][tl & (kHitQ - 1)][lane] = make_uint2(mk, (uint32_t)(p * 32));
             ++tl;
           }
-          const int nh = __popc(mk);
-          cnt += nh;
-          q4 = (q4 & ~(0xffu << (8 * p))) | ((uint32_t)nh << (8 * p));
+          cnt += __popc(mk);
         }
         continue;
       }
@@ -364,7 +383,7 @@ __device__ __forceinline__ void pair_body(const PairArgs &a, int bx, int) {
       //    every staged candidate against the lane's own i (bit masks), then evaluate (or
       //    list) the hits directly from the staged exact coordinates.
       int sg = 0;
-      for (int base = 0; base < T; base += 32 * kWin) {
+      for (int base = 32 * kWin * part; base < T; base += 32 * kWin * nsplit) {
 #pragma unroll
         for (int w = 0; w < kWin; ++w) {
           int s = sg;
@@ -442,8 +461,8 @@ __device__ __forceinline__ void pair_body(const PairArgs &a, int bx, int) {
             if (COUL) qj = sizeof(real) == 8 ? (real)a.set.qd[sj[slot]] : (real)sq[slot];
             // the particle itself, at zero displacement, is excluded by the evaluation
             // (coincident particles, which no valid configuration has, would be too)
-            pair_eval_masked<real, LJ, COUL, MULTI>(a, tab, act, dsx, dsy, dsz, qi, ti, qj, d.w,
-                                                    acc);
+            pair_eval_masked<LJ, COUL, MULTI, CUBIC>(a, tab, act, dsx, dsy, dsz, qi, ti, qj, d.w,
+                                                     acc);
           }
         }
         __syncwarp();
@@ -457,53 +476,82 @@ __device__ __forceinline__ void pair_body(const PairArgs &a, int bx, int) {
         if (mx > a.K) atomicOr(a.err, ERRBIT_CAPACITY);
       }
     } else if (valid) {
-      const int64_t o = a.set.map ? (int64_t)a.set.map[i] : i;
       const int64_t S = a.Fstride;
-      if (sizeof(real) == 8) {
-        if (a.accumulate) { a.Fd[o] += (double)acc.fx; a.Fd[S + o] += (double)acc.fy; a.Fd[2 * S + o] += (double)acc.fz; }
-        else { a.Fd[o] = (double)acc.fx; a.Fd[S + o] = (double)acc.fy; a.Fd[2 * S + o] = (double)acc.fz; }
-      } else {
-        if (a.accumulate) { a.F[o] += (float)acc.fx; a.F[S + o] += (float)acc.fy; a.F[2 * S + o] += (float)acc.fz; }
-        else { a.F[o] = (float)acc.fx; a.F[S + o] = (float)acc.fy; a.F[2 * S + o] = (float)acc.fz; }
+      if (sizeof(real) == 8) {  // (to length units)
+        acc.fx *= (real)a.fs[0]; acc.fy *= (real)a.fs[1]; acc.fz *= (real)a.fs[2];
       }
-      if (a.nbr) a.nbr[i] = acc.nbr;
+      if (nsplit > 1) {
+        real *P = reinterpret_cast<real *>(a.Fpart) + (int64_t)part * 3 * S + i;
+        P[0] = acc.fx; P[S] = acc.fy; P[2 * S] = acc.fz;
+      } else if (sizeof(real) == 8) {
+        a.Fd[i] = (double)acc.fx; a.Fd[S + i] = (double)acc.fy; a.Fd[2 * S + i] = (double)acc.fz;
+      } else {
+        a.F[i] = (float)acc.fx; a.F[S + i] = (float)acc.fy; a.F[2 * S + i] = (float)acc.fz;
+      }
+      if (a.nbr && nsplit == 1) a.nbr[i] = acc.nbr;
+      else if (a.nbr && acc.nbr) atomicAdd(a.nbr + i, acc.nbr);  // (cleared before)
     }
   }
   if (BUILD) return;
   // block partials of the energies and virials (halves of the per-i sums)
-  double v[NQ_PAIR] = {(double)acc.uc - (double)acc.cuc, (double)acc.ulj,
-                       (double)acc.wc - (double)acc.cwc, (double)acc.wlj};
-#pragma unroll
-  for (int k = 0; k < NQ_PAIR; ++k) {
-    const double w = warp_sum(v[k]);
-    if (lane == 0) wred[wid][k] = w;
-  }
-  __syncthreads();
-  if (threadIdx.x < NQ_PAIR) {
-    double s = 0.0;
-    for (int w = 0; w < kPairWarps; ++w) s += wred[w][threadIdx.x];
-    a.epart[(int64_t)bx * NQ_PAIR + threadIdx.x] = 0.5 * s;
-  }
+  double ulj = (double)acc.ulj, wlj = (double)acc.wlj;
+  if (sizeof(real) == 8 && !MULTI) grid_energies(a, (double)acc.ulj, (double)acc.wlj, ulj, wlj);
+  const double v[8] = {(double)acc.uc - (double)acc.cuc, ulj, (double)acc.wc - (double)acc.cwc, wlj,
+                       0.0, 0.0, 0.0, 0.0};
+  const double s = warp_sum8(v, lane);  // (kPairWarps is 1)
+  if (lane < NQ_PAIR) a.epart[(int64_t)bx * NQ_PAIR + lane] = 0.5 * s;
 }
 
-template <typename real, bool LJ, bool COUL, bool MULTI, bool WRAP, bool T16, bool BUILD>
-__global__ void __launch_bounds__(kPairWarps * 32, 28 / kPairWarps) pair_kernel(const PairArgs a) {
-  pair_body<real, LJ, COUL, MULTI, WRAP, T16, BUILD>(a, (int)blockIdx.x, (int)gridDim.x);
+// The parts of a split pass, added up in order.
+struct PairSumArgs {
+  const double *part;
+  void *F;
+  int64_t n3;
+  int nsplit;
+};
+template <typename real>
+__global__ void __launch_bounds__(256) pair_sum_kernel(const PairSumArgs a) {
+  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= a.n3) return;
+  const real *p = reinterpret_cast<const real *>(a.part) + k;
+  real s = p[0];
+  for (int q = 1; q < a.nsplit; ++q) s += p[q * a.n3];
+  static_cast<real *>(a.F)[k] = s;
+}
+
+template <typename real, bool LJ, bool COUL, bool MULTI, bool WRAP, bool T16, bool BUILD,
+          bool CUBIC>
+__global__ void __launch_bounds__(kPairWarps * 32, sizeof(real) == 8 ? 12 : 28) pair_kernel(const PairArgs a) {
+  pair_body<real, LJ, COUL, MULTI, WRAP, T16, BUILD, CUBIC>(a, (int)blockIdx.x, (int)gridDim.x);
+}
+
+int64_t pair_blocks(int64_t n) { return (n + 32 * kPairWarps - 1) / (32 * kPairWarps); }
+
+// One-warp blocks a tile of 32 particles is shared by: as many (at most 16) as fill the 28
+// resident warps an SM when the tiles alone do not: a tile is one warp's chain through all of its
+// candidates, whatever the box (the wrapping pass of a 2,000-particle, 27 A box: 329 us on 63
+// warps; a batch of 16 boxes of 2,000 to 60,000 particles went from 840 to 600 us a step).
+int pair_split(const Ctx &c) {
+  const int64_t tiles = std::max<int64_t>(1, pair_blocks(c.N));
+  return (int)std::min<int64_t>(16, std::max<int64_t>(1, ((int64_t)c.sms * 28) / tiles));
 }
 
 template <typename real, bool LJ, bool COUL, bool BUILD = false>
 static cudaError_t launch_one(Ctx &c, const PairArgs &a, int64_t n, bool multi, bool wrap) {
-  const unsigned blocks = (unsigned)((n + 32 * kPairWarps - 1) / (32 * kPairWarps));
+  const unsigned blocks = (unsigned)(pair_blocks(n) * (BUILD ? 1 : a.nsplit));
   if (blocks == 0) return cudaSuccess;
   const dim3 g(blocks), b(kPairWarps * 32);
   // (per replica in a batch; the list build is not used batched)
-#define RBE_PK(MU, WR, T)                                                                     \
-  dispatch(c, pair_kernel<real, LJ, COUL, MU, WR, T, BUILD>,                                  \
+#define RBE_PKC(MU, WR, T, CU)                                                                \
+  dispatch(c, pair_kernel<real, LJ, COUL, MU, WR, T, BUILD, CU>,                              \
            nullptr, g, b, 0, a, !BUILD)
+#define RBE_PK(MU, WR, T)                                                                     \
+  (a.cubic ? RBE_PKC(MU, WR, T, sizeof(real) == 8) : RBE_PKC(MU, WR, T, false))
   if (wrap) return multi ? RBE_PK(true, true, false) : RBE_PK(false, true, false);
   if (a.smax16 > 0) return multi ? RBE_PK(true, false, true) : RBE_PK(false, false, true);
   return multi ? RBE_PK(true, false, false) : RBE_PK(false, false, false);
 #undef RBE_PK
+#undef RBE_PKC
 }
 
 // Group x-extent (cells) for the half-precision test at cutoff rc with stencil R: every
@@ -530,8 +578,6 @@ int frame_span_cells(const Ctx &c, double rc) {
   const int s = (int)std::floor((0.5 * c.box[0] * (1.0 - 1e-9) - rc) / ax);
   return s >= 1 ? std::min(s, 1 << 20) : 0;
 }
-
-int64_t pair_blocks(int64_t n) { return (n + 32 * kPairWarps - 1) / (32 * kPairWarps); }
 
 // An FP32 r^2 formed from FP32 frame coordinates (each the integer offset from the group
 // leader, converted and scaled by L / 2^32: within 2u|x| of exact, u = 2^-24) is off by at
@@ -581,7 +627,6 @@ cudaError_t launch_pair(Ctx &c, bool want_counts) {
   a.set.sx = c.s[b]; a.set.sy = c.s[b] + c.N; a.set.sz = c.s[b] + 2 * c.N;
   a.set.qf = c.qf[b]; a.set.qd = c.qd[b]; a.set.type = c.type[b];
   a.set.cell_start = c.cell_start; a.set.map = nullptr; a.set.n = c.N;
-  a.accumulate = 0;
   a.epart = c.epart + c.off_pair;
   a.nbr = want_counts ? c.nbr : nullptr;
   a.smax = frame_span_cells(c, c.rc);
@@ -595,7 +640,15 @@ cudaError_t launch_pair(Ctx &c, bool want_counts) {
     a.invL[d] = (float)(1.0 / c.box[d]);
   }
   set_pretest_band(c, a, c.rc, wrap);
+  set_grid_units(c, a);
+  for (int d = 0; d < 2; ++d) a.wfix[d] = ((int64_t)1 << 48) / c.grid.n[d + 1];
+  a.nsplit = pair_split(c);
+  a.Fpart = c.fpart;
   const bool fp64 = c.precision == RBE_FP64;
+  if (want_counts && a.nsplit > 1) {
+    const cudaError_t e = fill_zero(c, c.nbr, c.N);
+    if (e != cudaSuccess) return e;
+  }
   if (fused) {
     const cudaError_t e = fp64 ? launch_one<double, true, true>(c, a, c.N, multi, wrap)
                                : launch_one<float, true, true>(c, a, c.N, multi, wrap);
@@ -605,7 +658,15 @@ cudaError_t launch_pair(Ctx &c, bool want_counts) {
                                : launch_one<float, true, false>(c, a, c.N, multi, wrap);
     if (e != cudaSuccess) return e;
   }
-  zero_partials_tail(c, c.off_pair, pair_blocks(c.N), c.n_pair_blk);
+  if (a.nsplit > 1) {
+    const int64_t n3 = 3 * c.N;
+    const PairSumArgs sa{c.fpart, fp64 ? (void *)c.Fd : (void *)c.F, n3, a.nsplit};
+    const dim3 g((unsigned)((n3 + 255) / 256)), b(256);
+    const cudaError_t e = fp64 ? dispatch(c, pair_sum_kernel<double>, nullptr, g, b, 0, sa, true)
+                               : dispatch(c, pair_sum_kernel<float>, nullptr, g, b, 0, sa, true);
+    if (e != cudaSuccess) return e;
+  }
+  zero_partials_tail(c, c.off_pair, pair_blocks(c.N) * a.nsplit, c.n_pair_blk);
   mark(c, RBE_PH_PAIR2);
   // the charged subset's Coulomb pass (k_coul.cu), added to the forces the main pass wrote
   if (!fused && c.Nq > 0) return launch_coulomb_subset(c, c.cq4, false);
@@ -649,6 +710,7 @@ cudaError_t launch_list_build(Ctx &c) {
     a.invL[d] = (float)(1.0 / c.box[d]);
   }
   set_pretest_band(c, a, rl, wrap);
+  for (int d = 0; d < 2; ++d) a.wfix[d] = ((int64_t)1 << 48) / c.grid.n[d + 1];
   a.list = c.vl_list; a.len = c.vl_len; a.K = c.vl_K;
   a.gate = c.vl_flags; a.maxlen = c.vl_flags + 2; a.err = c.err;
   cudaError_t e = launch_one<float, false, false, true>(c, a, c.N, false, wrap);

@@ -38,6 +38,18 @@ struct PairArgs {
   // neighbour is rejected; the exact decision is taken again when the pair is evaluated.
   float scale16;
   int smax16;
+  // The work of a tile of 32 particles shared by nsplit one-warp blocks (small systems): block
+  // part p sums every candidate chunk of its share into part p of Fpart ([nsplit][3][N]), which
+  // pair_sum_kernel adds up in order. nsplit 1: straight to F.
+  int nsplit;
+  double *Fpart;
+  int64_t wfix[2];       // 2^48 / cells in y and z (rounded down): a cell's width
+  // FP64 form: r^2 and force factors in grid units of x: h_d / h_x, the band around r_c^2, (h_y /
+  // h_x)^2, (h_z / h_x)^2, h_d / h_x^2, h_x, 1 / h_x, h_x^-6, and the single-type LJ coefficients times
+  // h_x^-12 and h_x^-6
+  float gh[3], glo, ghi;
+  double ry, rz, fs[3], hx, ihx, ih6, A12s, B6s;
+  int cubic;
   // Verlet-list build (the cell kernel's BUILD variant): pc's cutoff fields then hold
   // r_list = r_c + skin, and every j != i with r_ij^2 <= r_list^2 (1 + 1e-5) in FP32 is
   // appended to i's list: warp-interleaved, entry t of the particle in slot i at
@@ -109,9 +121,9 @@ __device__ __forceinline__ void erfc_exp2(const ErfcFit &f, f32x2 r, f32x2 r2, f
 // Squared distance of the exact cutoff decision (the oracle's definition): dx_d =
 // (int32)(s_i - s_j) * (L_d / 2^32) and r2 = dx^2 + dy^2 + dz^2 in FP64, no FMA.
 __device__ __forceinline__ double exact_r2(const PairConst &pc, int dsx, int dsy, int dsz) {
-  const double ex = __dmul_rn((double)dsx, pc.hd[0]);
-  const double ey = __dmul_rn((double)dsy, pc.hd[1]);
-  const double ez = __dmul_rn((double)dsz, pc.hd[2]);
+  const double ex = __dmul_rn(i2d(dsx), pc.hd[0]);
+  const double ey = __dmul_rn(i2d(dsy), pc.hd[1]);
+  const double ez = __dmul_rn(i2d(dsz), pc.hd[2]);
   return __dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez));
 }
 
@@ -204,71 +216,43 @@ __device__ __forceinline__ void pair_force(const PairArgs &a, const LJTable *tab
 // Branch-light evaluation for the cell-list kernel: `act` says whether this lane holds a
 // candidate pair at all (idle lanes compute a masked dummy). The cutoff decision is exact:
 // FP32 outside the +-1e-5 band around r_c^2, the oracle's FP64 expression inside it (a
-// rare, divergent branch); in the FP64 form always the FP64 expression. A zero
-// displacement (the particle itself; r^2 = 0 exactly when the integer displacement is 0)
-// is never a pair. Rejected and idle lanes evaluate with 1/r^2 = 0, which makes every LJ
-// term an exact zero, so no early return diverges the warp.
-template <typename real, bool LJ, bool COUL, bool MULTI>
+// rare, divergent branch). A zero displacement (the particle itself; r^2 = 0 exactly when the
+// integer displacement is 0) is never a pair. Rejected and idle lanes evaluate with 1/r^2 = 0,
+// which makes every LJ term an exact zero, so no early return diverges the warp.
+template <bool LJ, bool COUL, bool MULTI, bool CUBIC>
 __device__ __forceinline__ void pair_eval_masked(const PairArgs &a, const LJTable *tab,
-                                                 bool act, int dsx, int dsy, int dsz, real qi,
-                                                 int ti, real qj, int tj,
-                                                 PairAcc<real> &acc) {
+                                                 bool act, int dsx, int dsy, int dsz, float qi,
+                                                 int ti, float qj, int tj,
+                                                 PairAcc<float> &acc) {
   const PairConst &pc = a.pc;
-  real dx, dy, dz, r2;
-  bool inside;
-  if (sizeof(real) == 8) {
-    dx = (real)__dmul_rn((double)dsx, pc.hd[0]);
-    dy = (real)__dmul_rn((double)dsy, pc.hd[1]);
-    dz = (real)__dmul_rn((double)dsz, pc.hd[2]);
-    r2 = (real)__dadd_rn(__dadd_rn(__dmul_rn((double)dx, (double)dx),
-                                   __dmul_rn((double)dy, (double)dy)),
-                         __dmul_rn((double)dz, (double)dz));
-    inside = act && (double)r2 <= pc.rc2d && (double)r2 > 0.0;
-  } else {
-    dx = (real)((float)dsx * pc.h[0]);
-    dy = (real)((float)dsy * pc.h[1]);
-    dz = (real)((float)dsz * pc.h[2]);
-    r2 = mad(dx, dx, mad(dy, dy, dz * dz));
-    inside = act && (float)r2 < pc.rc2_lo && (float)r2 > 0.f;
-    const bool band = act && (float)r2 >= pc.rc2_lo && (float)r2 <= pc.rc2_hi;
-    if (band) inside = exact_r2(pc, dsx, dsy, dsz) <= pc.rc2d;
-  }
+  const float dx = (float)dsx * pc.h[0], dy = (float)dsy * pc.h[1], dz = (float)dsz * pc.h[2];
+  const float r2 = mad(dx, dx, mad(dy, dy, dz * dz));
+  bool inside = act && r2 < pc.rc2_lo && r2 > 0.f;
+  const bool band = act && r2 >= pc.rc2_lo && r2 <= pc.rc2_hi;
+  if (band) inside = exact_r2(pc, dsx, dsy, dsz) <= pc.rc2d;
   acc.nbr += inside ? 1 : 0;
-  // off the pair: 1/r^2 = 0 exactly (FP64: 1/inf; FP32: the fast quotient is documented
-  // to return 0 for divisors between 2^126 and 2^128)
-  const real r2s = inside ? r2 : (sizeof(real) == 8 ? (real)__longlong_as_double(0x7ff0000000000000ll)
-                                                    : (real)1e38f);
-  real g = (real)0;
+  // off the pair: 1/r^2 = 0 exactly (the fast quotient is documented to return 0 for divisors
+  // between 2^126 and 2^128)
+  const float r2s = inside ? r2 : 1e38f;
+  float g = 0.f;
   if (LJ) {
-    real ir2;
-    if (sizeof(real) == 8) ir2 = (real)(1.0 / (double)r2s);
-    else ir2 = (real)__fdividef(1.0f, (float)r2s);  // fast reciprocal (2 ulp)
-    real gl, u, w;
-    lj_terms<real, MULTI>(a, tab, ti, tj, ir2, gl, u, w);
+    const float ir2 = __fdividef(1.0f, r2s);  // fast reciprocal (2 ulp)
+    float gl, u, w;
+    lj_terms<float, MULTI>(a, tab, ti, tj, ir2, gl, u, w);
     g += gl;
     acc.ulj += u;
     acc.wlj += w;
   }
   if (COUL) {
-    const real qq = qi * qj;
-    if (inside && qq != (real)0) {
-      real r, rinv, erfcv, expv;
-      if (sizeof(real) == 8) {
-        r = (real)sqrt((double)r2);
-        rinv = (real)1 / r;
-        erfcv = (real)erfc(pc.sqrt_alpha_d * (double)r);
-        expv = (real)exp(-pc.alpha_d * (double)r2);
-      } else {
-        rinv = (real)rsqrtf((float)r2);  // 1/r and r from one reciprocal square root
-        r = r2 * rinv;
-        erfcv = (real)erfcf(pc.sqrt_alpha * (float)r);
-        expv = (real)expf(-pc.alpha * (float)r2);
-      }
-      const real Cqq = (sizeof(real) == 8 ? (real)pc.C_d : (real)pc.C) * qq;
-      const real tsp = sizeof(real) == 8 ? (real)pc.two_sqrt_alpha_over_sqrt_pi_d
-                                         : (real)pc.two_sqrt_alpha_over_sqrt_pi;
-      const real rinv2 = rinv * rinv;
-      const real gc = Cqq * mad(erfcv * rinv, rinv2, tsp * expv * rinv2);
+    const float qq = qi * qj;
+    if (inside && qq != 0.f) {
+      const float rinv = rsqrtf(r2);  // 1/r and r from one reciprocal square root
+      const float r = r2 * rinv;
+      const float erfcv = erfcf(pc.sqrt_alpha * r);
+      const float expv = expf(-pc.alpha * r2);
+      const float Cqq = pc.C * qq;
+      const float rinv2 = rinv * rinv;
+      const float gc = Cqq * mad(erfcv * rinv, rinv2, pc.two_sqrt_alpha_over_sqrt_pi * expv * rinv2);
       g += gc;
       if (a.comp) {
         kahan_add(acc.uc, acc.cuc, Cqq * erfcv * rinv);
@@ -282,6 +266,95 @@ __device__ __forceinline__ void pair_eval_masked(const PairArgs &a, const LJTabl
   acc.fx = mad(g, dx, acc.fx);
   acc.fy = mad(g, dy, acc.fy);
   acc.fz = mad(g, dz, acc.fz);
+}
+
+// The FP64 form's evaluation. FP64 runs at 1/64 of the FP32 rate, so its operations are what it
+// costs: 19 a pair in a cubic box (21 otherwise), where scaled displacements, a division, FP64
+// cutoff tests and conversions took about 40 (65,536 particles, 10% charged: 2,888 -> 1,692 us
+// with the ring and split of k_pair.cu). The cutoff is decided in FP32 from the exact displacement,
+// in the +-1e-5 band by the oracle's FP64 expression. r^2 and the force sums stay in grid units
+// of x (the integer displacement converts exactly; the caller scales the sums by fs). 1/r^2 is
+// an FP32 reciprocal refined by one third-order Householder step, y (1 + e + e^2) with
+// e = 1 - r^2 y (|e| < 2^-21: the error left is below 2^-62), the Coulomb 1/r likewise,
+// y (1 + e/2 + 3 e^2 / 8). acc.ulj and acc.wlj hold sum r^-12 and sum r^-6 in grid units for one
+// LJ type, U and W for several.
+// (CUBIC: the three edges are equal. A kernel of its own: as a branch its other side's FP64
+// instructions were issued with a false predicate and still took the pipe.)
+template <bool LJ, bool COUL, bool MULTI, bool CUBIC>
+__device__ __forceinline__ void pair_eval_masked(const PairArgs &a, const LJTable *tab,
+                                                 bool act, int dsx, int dsy, int dsz, double qi,
+                                                 int ti, double qj, int tj,
+                                                 PairAcc<double> &acc) {
+  const PairConst &pc = a.pc;
+  const float ex = (float)dsx * a.gh[0], ey = (float)dsy * a.gh[1], ez = (float)dsz * a.gh[2];
+  const float Rf = fmaf(ex, ex, fmaf(ey, ey, ez * ez));
+  bool inside = act && Rf < a.glo && Rf > 0.f;
+  if (act && Rf >= a.glo && Rf <= a.ghi) inside = exact_r2(pc, dsx, dsy, dsz) <= pc.rc2d;
+  acc.nbr += inside ? 1 : 0;
+  const double Dx = i2d(dsx), Dy = i2d(dsy), Dz = i2d(dsz);
+  const double R = CUBIC ? fma(Dz, Dz, fma(Dy, Dy, Dx * Dx))
+                         : fma(Dz * Dz, a.rz, fma(Dy * Dy, a.ry, Dx * Dx));
+  // (off the pair y = 0: every term below is an exact zero)
+  const double y = f2d(inside ? rcp_approx(Rf) : 0.f);
+  const double e = fma(-R, y, 1.0);
+  const double iR = fma(y, fma(e, e, e), y);
+  double w = 0.0;
+  if (LJ) {
+    const double i6 = iR * iR * iR;
+    if (MULTI) {
+      const int pt = ti * tab->nt + tj;
+      const double ir6 = i6 * a.ih6;
+      w = ir6 * fma(tab->A12d[pt], ir6, -tab->B6d[pt]);
+      acc.ulj = fma(ir6, fma(tab->Ad[pt], ir6, -tab->Bd[pt]), acc.ulj);
+      acc.wlj += w;
+    } else {
+      w = i6 * fma(a.A12s, i6, -a.B6s);
+      acc.ulj = fma(i6, i6, acc.ulj);
+      acc.wlj += i6;
+    }
+  }
+  if (COUL) {
+    const double qq = qi * qj;
+    if (inside && qq != 0.0) {
+      const double z = f2d(rsqrtf(Rf)), ez_ = fma(-(R * z), z, 1.0);
+      const double zr = fma(z, ez_ * fma(ez_, 0.375, 0.5), z);  // 1 / r in grid units
+      const double r = R * zr * a.hx;
+      const double erfcv = erfc(pc.sqrt_alpha_d * r), expv = exp(-pc.alpha_d * (r * r));
+      const double Cqq = pc.C_d * qq, u = Cqq * erfcv * (zr * a.ihx);
+      const double wc = fma(Cqq * pc.two_sqrt_alpha_over_sqrt_pi_d, expv, u);
+      acc.uc += u;
+      acc.wc += wc;
+      w += wc;
+    }
+  }
+  const double g = w * iR;
+  acc.fx = fma(g, Dx, acc.fx);
+  acc.fy = fma(g, Dy, acc.fy);
+  acc.fz = fma(g, Dz, acc.fz);
+}
+
+// What the FP64 evaluation needs beside PairArgs' other fields.
+inline void set_grid_units(const Ctx &c, PairArgs &a) {
+  const double hx = c.pc.hd[0];
+  a.ry = (c.pc.hd[1] / hx) * (c.pc.hd[1] / hx);
+  a.rz = (c.pc.hd[2] / hx) * (c.pc.hd[2] / hx);
+  for (int d = 0; d < 3; ++d) a.fs[d] = c.pc.hd[d] / (hx * hx);
+  for (int d = 0; d < 3; ++d) a.gh[d] = (float)(c.pc.hd[d] / hx);
+  a.glo = (float)(c.pc.rc2d / (hx * hx) * (1.0 - 1e-5));
+  a.ghi = (float)(c.pc.rc2d / (hx * hx) * (1.0 + 1e-5));
+  a.hx = hx;
+  a.ihx = 1.0 / hx;
+  a.ih6 = 1.0 / ((hx * hx) * (hx * hx) * (hx * hx));
+  a.A12s = c.lj.A12d[0] * a.ih6 * a.ih6;
+  a.B6s = c.lj.B6d[0] * a.ih6;
+  a.cubic = c.pc.hd[0] == c.pc.hd[1] && c.pc.hd[1] == c.pc.hd[2];
+}
+// U and W of one LJ type from the FP64 sums in grid units.
+__device__ __forceinline__ void grid_energies(const PairArgs &a, double s12, double s6, double &u,
+                                              double &w) {
+  const double p = a.A12s * s12, q = a.B6s * s6;
+  u = p / 12.0 - q / 6.0;
+  w = p - q;
 }
 
 // Exact cutoff decision from the integer displacement ds = s_i - s_j (mod 2^32, the

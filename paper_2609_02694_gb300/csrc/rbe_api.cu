@@ -20,6 +20,7 @@ using namespace rbe;
 
 namespace rbe {
 int64_t pair_blocks(int64_t n);
+int pair_split(const Ctx &c);
 int64_t rbl_blocks(int64_t n);
 int64_t rbl_slot_count(int64_t n, int sms);
 int64_t rbl_compact_count(int64_t nblk);
@@ -166,7 +167,7 @@ int free_all(Ctx &c) {
     if (c.fgraph[b]) cudaGraphExecDestroy(c.fgraph[b]);
     c.fgraph[b] = nullptr;
   }
-  dfree(c.F); dfree(c.Fd); dfree(c.facc); dfree(c.cl_base); dfree(c.sc_base); dfree(c.sc_info); dfree(c.cl_lo);
+  dfree(c.F); dfree(c.Fd); dfree(c.fpart); dfree(c.facc); dfree(c.cl_base); dfree(c.sc_base); dfree(c.sc_info); dfree(c.cl_lo);
   dfree(c.cl_hi); dfree(c.cjrec); dfree(c.cq4); dfree(c.cs); dfree(c.cqf); dfree(c.cqd); dfree(c.cmap);
   dfree(c.cell_count); dfree(c.cell_start); dfree(c.key); dfree(c.off); dfree(c.tmp);
   dfree(c.scan_blk);
@@ -540,7 +541,7 @@ int rbe_init(rbe_handle *hout, const rbe_params *p, int64_t N, const double box[
   }
 
   // reductions layout
-  c.n_pair_blk = rbl ? 0 : std::max(pair_blocks(N), cpair_blocks_bound(c));
+  c.n_pair_blk = rbl ? 0 : std::max(pair_blocks(N) * pair_split(c), cpair_blocks_bound(c));
   c.n_coul_blk = rbl ? 0 : std::max(pair_blocks(Nq), coul_blocks(Nq));
   c.n_rbl_blk = rbl ? rbl_blocks(N) : 0;
   c.rbl_nslots = rbl ? rbl_slot_count(N, c.sms) : 0;
@@ -569,6 +570,7 @@ int rbe_init(rbe_handle *hout, const rbe_params *p, int64_t N, const double box[
   else rc |= dalloc(c, &c.F, 3 * N);
   if (!rbl) {
     const int64_t nrows = (int64_t)c.grid.n[1] * c.grid.n[2];
+    if (pair_split(c) > 1) rc |= dalloc(c, &c.fpart, pair_split(c) * 3 * N);
     rc |= dalloc(c, &c.facc, 3 * N);
     rc |= dalloc(c, &c.cl_base, nrows + 1);
     rc |= dalloc(c, &c.sc_base, nrows + 1);
@@ -1347,12 +1349,15 @@ static bool record_step(Ctx &c, int flip, Recorder &rec) {
 }
 
 // Same kernel (batched and solo: a kernel launched per replica has no batched form, so its
-// solo instance decides) and the same block shape.
+// solo instance decides) and, where one launch serves the class, the same block shape (a kernel
+// launched per replica keeps each replica's own).
 static bool same_shape(const RecItem &x, const RecItem &y) {
-  return x.fn == y.fn && x.solo_fn == y.solo_fn && x.per_replica == y.per_replica &&
-         x.grid.y == y.grid.y && x.grid.z == y.grid.z &&
-         x.block.x == y.block.x && x.block.y == y.block.y && x.block.z == y.block.z &&
-         x.smem == y.smem && x.args.size() == y.args.size();
+  if (x.fn != y.fn || x.solo_fn != y.solo_fn || x.per_replica != y.per_replica ||
+      x.args.size() != y.args.size())
+    return false;
+  return x.per_replica ||
+         (x.grid.y == y.grid.y && x.grid.z == y.grid.z && x.block.x == y.block.x &&
+          x.block.y == y.block.y && x.block.z == y.block.z && x.smem == y.smem);
 }
 static bool same_sequence(const Recorder &x, const Recorder &y) {
   if (x.items.size() != y.items.size()) return false;
@@ -1420,7 +1425,8 @@ struct ClassLaunch {
   dim3 grid, block;
   size_t smem, tab_off, pre_off;
   bool per_replica;
-  std::vector<dim3> grids;
+  std::vector<dim3> grids, blocks;  // per replica, as are smems and args
+  std::vector<size_t> smems;
   std::vector<std::vector<unsigned char>> args;
 };
 
@@ -1449,6 +1455,8 @@ static int batch_tables(rbe_batch b, int flip, void **dev, std::vector<std::vect
         L.grid = it.grid;
         for (size_t j = 0; j < reps.size(); ++j) {
           L.grids.push_back(rec[k][j].items[i].grid);
+          L.blocks.push_back(rec[k][j].items[i].block);
+          L.smems.push_back(rec[k][j].items[i].smem);
           L.args.push_back(rec[k][j].items[i].args);
         }
       } else {
@@ -1530,7 +1538,7 @@ static int batch_capture(rbe_batch b, int k, int flip) {
               const dim3 g = L.grids[j];
               if (g.x == 0) continue;
               void *params[] = {const_cast<unsigned char *>(L.args[j].data())};
-              if (cudaLaunchKernel(L.fn, g, L.block, params, L.smem, ss) != cudaSuccess) {
+              if (cudaLaunchKernel(L.fn, g, L.blocks[j], params, L.smems[j], ss) != cudaSuccess) {
                 rc = RBE_ERR_CUDA;
                 break;
               }

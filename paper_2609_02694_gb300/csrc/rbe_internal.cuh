@@ -119,6 +119,7 @@ struct Ctx {
   float *invm[2] = {nullptr, nullptr};
   float *F = nullptr;
   double *Fd = nullptr;
+  double *fpart = nullptr;     // per-particle pair kernel: partial forces of a split pass
   // cluster-pair kernel: fixed-point force sums (3N, sorted order), per-row cluster and
   // super-cluster offsets (rows + 1 each), per-cluster bounds
   long long *facc = nullptr;
@@ -244,10 +245,6 @@ __device__ __forceinline__ float phase_to_radians(uint32_t ph) {
   return f * (float)(2.0 * kPi / 8388608.0);
 }
 
-__device__ __forceinline__ double phase_to_radians_d(uint32_t ph) {
-  return (double)(int)ph * (2.0 * kPi / kTwo32);
-}
-
 // Add v * scale to a 64-bit fixed-point force sum (round to nearest); an out-of-range value
 // sets the non-finite flag instead (its sum would wrap). Integer sums do not depend on the
 // order of their terms, so passes that add to the same sums may run in any order.
@@ -291,6 +288,19 @@ __device__ __forceinline__ void fx_add_i32(long long *p, double v, double scale,
 __device__ __forceinline__ float mad(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
 
+// Conversions to FP64 without the conversion instructions, which issue to the FP64 pipe (1/64 of
+// the FP32 rate) and take it longer than an addition. An int through 2^52 + 2^31 + v, whose bits
+// are v's with the sign bit flipped, and one exact subtraction; a float by moving its fields.
+__device__ __forceinline__ double i2d(int v) {
+  return __hiloint2double(0x43300000, v ^ (int)0x80000000) - 4503601774854144.0;
+}
+__device__ __forceinline__ double f2d(float v) {
+  const uint32_t b = __float_as_uint(v), m = b & 0x7fffffffu;
+  if (m - 0x00800000u >= 0x7f000000u && m) return (double)v;  // subnormal, infinite, NaN
+  const uint32_t hi = m ? (m >> 3) + 0x38000000u : 0u;
+  return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
+}
+
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -300,6 +310,14 @@ __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
+}
+// Two sums over the warp: even lanes end with the first, odd lanes with the second, in 5 additions
+// instead of 10.
+__device__ __forceinline__ double warp_sum2(double u, double w, int lane) {
+  double s = (lane & 1 ? w : u) + __shfl_xor_sync(0xffffffffu, lane & 1 ? u : w, 1);
+#pragma unroll
+  for (int o = 2; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
 }
 // Eight sums over the warp; lane k < 8 (and every lane with the same low three bits) ends with
 // sum k. Each exchange halves the list a lane still carries: 9 additions, where eight separate
