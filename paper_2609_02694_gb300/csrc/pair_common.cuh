@@ -3,6 +3,8 @@
 #pragma once
 #include <cuda_fp16.h>
 
+#include <cmath>
+
 #include "f32x2.cuh"
 #include "rbe_internal.cuh"
 
@@ -333,20 +335,32 @@ __device__ __forceinline__ void pair_eval_masked(const PairArgs &a, const LJTabl
   acc.fz = fma(g, Dz, acc.fz);
 }
 
-// What the FP64 evaluation needs beside PairArgs' other fields.
+// What the FP64 evaluation needs beside PairArgs' other fields. The powers of h_x are formed as
+// unevaluated sums of two doubles and divided out with one correction, so that each constant is
+// its true value rounded about once: an error here would be in every pair, sevenfold in the force.
 inline void set_grid_units(const Ctx &c, PairArgs &a) {
   const double hx = c.pc.hd[0];
+  struct DD { double h, l; };
+  auto mul = [](DD x, DD y) {
+    const double p = x.h * y.h;
+    return DD{p, std::fma(x.h, y.h, -p) + (x.h * y.l + x.l * y.h)};
+  };
+  auto div = [](double v, DD y) {
+    const double q = v / y.h;
+    return q + (std::fma(-q, y.h, v) - q * y.l) / y.h;
+  };
+  const DD p1{hx, 0.0}, p2 = mul(p1, p1), p6 = mul(mul(p2, p2), p2), p12 = mul(p6, p6);
   a.ry = (c.pc.hd[1] / hx) * (c.pc.hd[1] / hx);
   a.rz = (c.pc.hd[2] / hx) * (c.pc.hd[2] / hx);
-  for (int d = 0; d < 3; ++d) a.fs[d] = c.pc.hd[d] / (hx * hx);
+  for (int d = 0; d < 3; ++d) a.fs[d] = div(c.pc.hd[d], p2);
   for (int d = 0; d < 3; ++d) a.gh[d] = (float)(c.pc.hd[d] / hx);
   a.glo = (float)(c.pc.rc2d / (hx * hx) * (1.0 - 1e-5));
   a.ghi = (float)(c.pc.rc2d / (hx * hx) * (1.0 + 1e-5));
   a.hx = hx;
   a.ihx = 1.0 / hx;
-  a.ih6 = 1.0 / ((hx * hx) * (hx * hx) * (hx * hx));
-  a.A12s = c.lj.A12d[0] * a.ih6 * a.ih6;
-  a.B6s = c.lj.B6d[0] * a.ih6;
+  a.ih6 = div(1.0, p6);
+  a.A12s = div(c.lj.A12d[0], p12);
+  a.B6s = div(c.lj.B6d[0], p6);
   a.cubic = c.pc.hd[0] == c.pc.hd[1] && c.pc.hd[1] == c.pc.hd[2];
 }
 // U and W of one LJ type from the FP64 sums in grid units.
