@@ -51,10 +51,9 @@ struct GatherArgs {
   const double2 *abd;
   int P, slices;           // the modes shared by `slices` threads a particle
   const int32_t *cmap;
-  float *F;
-  double *Fd;
+  void *fk;                // 3 x Nq forces in charged order (of the form's type), or, with facc,
   int64_t N;
-  long long *facc;         // nullable: add to these 3 x N fixed-point sums instead of F
+  long long *facc;         // nullable: add to these 3 x N fixed-point sums instead
   float fscale;            // (their scale in the FP32 forms,
   double fscale_d;         //  and in the FP64 form)
   int *err;
@@ -301,8 +300,8 @@ __device__ __forceinline__ void gather_body(const GatherArgs &a, int bx, int) {
     else { fx = (float)s[0]; fy = (float)s[1]; fz = (float)s[2]; }
   }
   if (!valid) return;
-  const int64_t p = a.cmap[i];
-  if (a.facc) {  // into the cluster kernel's fixed-point sums (integer atomics)
+  if (a.facc) {
+    const int64_t p = a.cmap[i];  // into the cluster kernel's fixed-point sums (integer atomics)
     if (MODE == 2) {
       const double q = a.cqd[i];
       fx_add(a.facc + p, -q * dx, a.fscale_d, a.err);
@@ -315,20 +314,43 @@ __device__ __forceinline__ void gather_body(const GatherArgs &a, int bx, int) {
       fx_add_i32(a.facc + 2 * N + p, -q * fz, a.fscale, a.err);
     }
   } else if (MODE == 2) {
-    double *__restrict__ Fd = a.Fd;
+    double *__restrict__ fk = static_cast<double *>(a.fk);
     const double q = a.cqd[i];
-    Fd[p] = mad(-q, dx, Fd[p]);
-    Fd[N + p] = mad(-q, dy, Fd[N + p]);
-    Fd[2 * N + p] = mad(-q, dz, Fd[2 * N + p]);
+    fk[i] = -q * dx;
+    fk[Nq + i] = -q * dy;
+    fk[2 * Nq + i] = -q * dz;
   } else {
-    float *__restrict__ F = a.F;
+    float *__restrict__ fk = static_cast<float *>(a.fk);
     const float q = a.cqf[i];
-    F[p] = mad(-q, fx, F[p]);
-    F[N + p] = mad(-q, fy, F[N + p]);
-    F[2 * N + p] = mad(-q, fz, F[2 * N + p]);
+    fk[i] = -q * fx;
+    fk[Nq + i] = -q * fy;
+    fk[2 * Nq + i] = -q * fz;
   }
 }
 RBE_MODE_KERNELS(__launch_bounds__(kGatherThreads), gather_kernel, GatherArgs, gather_body)
+
+// F += the k-space forces of the charged particles (gather_kernel without fixed-point sums), so
+// that the gather can run beside the pass that writes F.
+struct KAddArgs {
+  const void *fk;
+  const int32_t *cmap;
+  void *F;
+  int64_t Nq, N;
+  int fp64;
+};
+__device__ __forceinline__ void kspace_add_body(const KAddArgs &a, int bx, int) {
+  const int64_t i = (int64_t)bx * blockDim.x + threadIdx.x;
+  if (i >= a.Nq) return;
+  const int64_t p = a.cmap[i];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    if (a.fp64)
+      static_cast<double *>(a.F)[d * a.N + p] += static_cast<const double *>(a.fk)[d * a.Nq + i];
+    else
+      static_cast<float *>(a.F)[d * a.N + p] += static_cast<const float *>(a.fk)[d * a.Nq + i];
+  }
+}
+RBE_BATCHED_KERNEL(__launch_bounds__(256), kspace_add_kernel, KAddArgs, kspace_add_body)
 
 template <int MODE>
 static cudaError_t sf_launch(Ctx &c, dim3 grid, size_t shm) {
@@ -361,7 +383,7 @@ cudaError_t launch_kspace_gather(Ctx &c, bool into_facc) {
   const int nper = kGatherThreads / slices;
   const unsigned blocks = (unsigned)((c.Nq + nper - 1) / nper);
   const GatherArgs a{c.cs, c.cqf, c.cqd, c.Nq, c.m, c.kcf, c.kcd, c.abf, c.abd, c.P, slices, c.cmap,
-                     c.F, c.Fd, c.N, into_facc ? c.facc : nullptr, (float)kFixScale32,
+                     c.fk, c.N, into_facc ? c.facc : nullptr, (float)kFixScale32,
                      kFixScale64, c.err};
   // (into the fixed-point sums it runs per replica in a batch, within the pair pass's run)
   if (c.precision == RBE_FP64)
@@ -369,6 +391,14 @@ cudaError_t launch_kspace_gather(Ctx &c, bool into_facc) {
                     0, a, into_facc);
   return dispatch(c, gather_kernel<0>, gather_kernel_b<0>, dim3(blocks), dim3(kGatherThreads), 0,
                   a, into_facc);
+}
+
+cudaError_t launch_kspace_add(Ctx &c) {
+  if (c.Nq == 0) return cudaSuccess;
+  const bool fp64 = c.precision == RBE_FP64;
+  const KAddArgs a{c.fk, c.cmap, fp64 ? (void *)c.Fd : (void *)c.F, c.Nq, c.N, fp64 ? 1 : 0};
+  return dispatch(c, kspace_add_kernel, kspace_add_kernel_b, dim3((unsigned)((c.Nq + 255) / 256)),
+                  dim3(256), 0, a);
 }
 
 }  // namespace rbe

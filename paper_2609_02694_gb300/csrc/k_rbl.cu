@@ -1048,13 +1048,18 @@ __global__ void __launch_bounds__(256) rbl_mean_kernel(const double *__restrict_
   if (threadIdx.x < 3) mean[threadIdx.x] = sh[threadIdx.x][0] / (double)N;
 }
 
+// (fk: the k-space forces when every particle is charged, in the same order; else null)
 template <typename real>
-__global__ void rbl_subtract_kernel(real *__restrict__ F, int64_t N, const double *__restrict__ mean) {
+__global__ void __launch_bounds__(256)
+    rbl_subtract_kernel(real *__restrict__ F, int64_t N, const double *__restrict__ mean,
+                        const real *__restrict__ fk) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
-  F[i] -= (real)mean[0];
-  F[N + i] -= (real)mean[1];
-  F[2 * N + i] -= (real)mean[2];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const real f = F[d * N + i] - (real)mean[d];
+    F[d * N + i] = fk ? f + fk[d * N + i] : f;
+  }
 }
 
 int64_t rbl_blocks(int64_t n) { return (n + 32 * kRblWarps - 1) / (32 * kRblWarps); }
@@ -1191,10 +1196,21 @@ cudaError_t launch_rbl(Ctx &c, bool want_debug) {
                                                              (blocks + ncomp - 1) / ncomp,
                                                              c.rbl_cpart, c.rbl_cpart + ncomp * NQ_PAIR);
   rbl_mean_kernel<<<1, 256, 0, c.stream>>>(c.rbl_cpart + ncomp * NQ_PAIR, ncomp, c.N, c.rbl_mean);
-  const unsigned nb = (unsigned)((c.N + 255) / 256);
-  if (c.precision == RBE_FP64) rbl_subtract_kernel<double><<<nb, 256, 0, c.stream>>>(c.Fd, c.N, c.rbl_mean);
-  else rbl_subtract_kernel<float><<<nb, 256, 0, c.stream>>>(c.F, c.N, c.rbl_mean);
   return cudaGetLastError();
+}
+
+// The mean-force correction, and the k-space forces of the gather.
+cudaError_t launch_rbl_finish(Ctx &c) {
+  const unsigned nb = (unsigned)((c.N + 255) / 256);
+  const bool all = c.Nq == c.N;  // (then charged order is slot order)
+  if (c.precision == RBE_FP64)
+    rbl_subtract_kernel<double><<<nb, 256, 0, c.stream>>>(c.Fd, c.N, c.rbl_mean,
+                                                          all ? (const double *)c.fk : nullptr);
+  else
+    rbl_subtract_kernel<float><<<nb, 256, 0, c.stream>>>(c.F, c.N, c.rbl_mean,
+                                                         all ? (const float *)c.fk : nullptr);
+  const cudaError_t e = cudaGetLastError();
+  return e != cudaSuccess || all ? e : launch_kspace_add(c);
 }
 
 }  // namespace rbe

@@ -167,7 +167,7 @@ int free_all(Ctx &c) {
     if (c.fgraph[b]) cudaGraphExecDestroy(c.fgraph[b]);
     c.fgraph[b] = nullptr;
   }
-  dfree(c.F); dfree(c.Fd); dfree(c.fpart); dfree(c.facc); dfree(c.cl_base); dfree(c.sc_base); dfree(c.sc_info); dfree(c.cl_lo);
+  dfree(c.F); dfree(c.Fd); dfree(c.fpart); dfree(c.fk); dfree(c.facc); dfree(c.cl_base); dfree(c.sc_base); dfree(c.sc_info); dfree(c.cl_lo);
   dfree(c.cl_hi); dfree(c.cjrec); dfree(c.cq4); dfree(c.cs); dfree(c.cqf); dfree(c.cqd); dfree(c.cmap);
   dfree(c.cell_count); dfree(c.cell_start); dfree(c.key); dfree(c.off); dfree(c.tmp);
   dfree(c.scan_blk);
@@ -184,74 +184,100 @@ int free_all(Ctx &c) {
   if (c.aux_stream) cudaStreamDestroy(c.aux_stream);
   c.aux_stream = nullptr;
   if (c.ev_fork) cudaEventDestroy(c.ev_fork);
+  if (c.ev_bin) cudaEventDestroy(c.ev_bin);
   if (c.ev_join) cudaEventDestroy(c.ev_join);
-  c.ev_fork = c.ev_join = nullptr;
+  c.ev_fork = c.ev_bin = c.ev_join = nullptr;
   if (c.scal_host) cudaFreeHost(c.scal_host);
   c.scal_host = nullptr;
   return RBE_OK;
 }
 
-// The cluster kernel's pipeline in two branches of a captured graph: the k-space chain
-// (sampler, structure factor, gather) and the charged subset's Coulomb pass, both into the
-// fixed-point sums, on the auxiliary stream beside the cluster tables and the pair pass; then
-// the fixed-point finish. The sums are integers, so the forces are those of the sequential
-// order bit for bit. The pair pass is issue-bound at three quarters of the issue slots, one
-// warp per block; the other branch's kernels fill the slots and SMs it leaves idle (measured
-// on 2^20 particles: 1.445 -> 1.360 ms a step, against 1.414 with only the k-space chain
-// beside it).
-int cluster_pipeline_forked(Ctx &c, bool debug) {
-  RBE_CUDA_TRY(cudaEventRecord(c.ev_fork, c.stream));
-  RBE_CUDA_TRY(cudaStreamWaitEvent(c.aux_stream, c.ev_fork, 0));
-  const cudaStream_t main_stream = c.stream;
-  c.stream = c.aux_stream;
-  cudaError_t e = launch_sample_k(c);
-  if (e == cudaSuccess) e = launch_structure_factor(c);
-  if (e == cudaSuccess) e = launch_kspace_gather(c, true);
-  const bool fused = c.Nq * 2 > c.N;  // (then the pair pass takes the Coulomb pairs itself)
-  if (e == cudaSuccess && !fused) e = launch_coulomb_subset(c, c.cq4, true);
-  if (e == cudaSuccess) e = cudaEventRecord(c.ev_join, c.aux_stream);
-  c.stream = main_stream;
-  RBE_CUDA_TRY(e);
-  RBE_CUDA_TRY(launch_cluster_tables(c));
-  RBE_CUDA_TRY(launch_cluster_pair(c, fused, c.nt > 1, debug));
-  RBE_CUDA_TRY(cudaStreamWaitEvent(c.stream, c.ev_join, 0));
-  RBE_CUDA_TRY(launch_cluster_finish(c));
+// The real-space pass and what turns it and the k-space forces into F, on c.stream. cp: the
+// cluster kernel (its Coulomb pass runs elsewhere when `coulomb` is false).
+int real_space(Ctx &c, bool cp, bool coulomb, bool debug) {
+  if (c.rbl) RBE_CUDA_TRY(launch_rbl(c, debug));
+  else if (c.vl_on) RBE_CUDA_TRY(launch_list_pair(c, debug));
+  else if (cp && coulomb) RBE_CUDA_TRY(launch_pair_cluster(c, debug));
+  else if (cp) RBE_CUDA_TRY(launch_cluster_pair(c, c.Nq * 2 > c.N, c.nt > 1, debug));
+  else RBE_CUDA_TRY(launch_pair(c, debug));
   return RBE_OK;
 }
-
-// [list check] -> bin + sort -> sample -> structure factor -> [list build] -> real space
-// -> k-space gather (-> the cluster kernel's fixed-point finish)
-int force_pipeline(Ctx &c, bool debug) {
-  mark(c, RBE_PH_BIN);
-  if (c.vl_on) RBE_CUDA_TRY(launch_list_check(c));
-  RBE_CUDA_TRY(launch_bin_sort(c));
-  const bool cp = !c.rbl && !c.vl_on && cpair_usable(c);
-  if (cp && c.Nq > 0 && !c.rec && !c.timing && c.aux_stream) {
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    RBE_CUDA_TRY(cudaStreamIsCapturing(c.stream, &st));
-    if (st == cudaStreamCaptureStatusActive) return cluster_pipeline_forked(c, debug);
-  }
-  mark(c, RBE_PH_SAMPLE);
-  RBE_CUDA_TRY(launch_sample_k(c));
-  mark(c, RBE_PH_SF);
-  RBE_CUDA_TRY(launch_structure_factor(c));
-  mark(c, RBE_PH_LIST);
+int finish_forces(Ctx &c, bool cp) {
+  if (cp) RBE_CUDA_TRY(launch_cluster_finish(c));
+  else if (c.rbl) RBE_CUDA_TRY(launch_rbl_finish(c));
+  else RBE_CUDA_TRY(launch_kspace_add(c));
+  return RBE_OK;
+}
+int lists(Ctx &c, bool cp) {
   if (c.vl_on) {
     RBE_CUDA_TRY(launch_list_build(c));
     RBE_CUDA_TRY(launch_list_commit(c));
   } else if (cp) {
     RBE_CUDA_TRY(launch_cluster_tables(c));  // the cluster-pair kernel's per-step tables
   }
+  return RBE_OK;
+}
+
+// The pipeline in two branches of a captured graph: the sampler, which needs only the step
+// number, beside the binning; then the k-space chain (structure factor, gather) and, with the
+// cluster kernel, the charged subset's Coulomb pass beside the real-space pass; then the pass that
+// forms F. Each branch writes its own arrays (or adds integers to the fixed-point sums), so the
+// forces are those of the sequential order bit for bit. The real-space passes issue in 60 to 75%
+// of their slots; the other branch's kernels fill slots and SMs they leave idle (measured with
+// the cluster kernel on 2^20 particles: 1.445 -> 1.360 ms a step; FORK_FIGURES).
+int force_pipeline_forked(Ctx &c, bool cp, bool debug) {
+  const cudaStream_t main_stream = c.stream;
+  RBE_CUDA_TRY(cudaEventRecord(c.ev_fork, main_stream));
+  RBE_CUDA_TRY(cudaStreamWaitEvent(c.aux_stream, c.ev_fork, 0));
+  c.stream = c.aux_stream;
+  cudaError_t e = launch_sample_k(c);
+  c.stream = main_stream;
+  RBE_CUDA_TRY(e);
+  if (c.vl_on) RBE_CUDA_TRY(launch_list_check(c));
+  RBE_CUDA_TRY(launch_bin_sort(c));
+  RBE_CUDA_TRY(cudaEventRecord(c.ev_bin, main_stream));
+  RBE_CUDA_TRY(cudaStreamWaitEvent(c.aux_stream, c.ev_bin, 0));
+  c.stream = c.aux_stream;
+  e = launch_structure_factor(c);
+  if (e == cudaSuccess) e = launch_kspace_gather(c, cp);
+  // (mostly charged: the pair pass takes the Coulomb pairs itself)
+  if (e == cudaSuccess && cp && c.Nq * 2 <= c.N) e = launch_coulomb_subset(c, c.cq4, true);
+  if (e == cudaSuccess) e = cudaEventRecord(c.ev_join, c.aux_stream);
+  c.stream = main_stream;
+  RBE_CUDA_TRY(e);
+  int rc = lists(c, cp);
+  if (rc == RBE_OK) rc = real_space(c, cp, false, debug);
+  if (rc != RBE_OK) return rc;
+  RBE_CUDA_TRY(cudaStreamWaitEvent(c.stream, c.ev_join, 0));
+  return finish_forces(c, cp);
+}
+
+// [list check] -> bin + sort -> sample -> structure factor -> [list build] -> real space
+// -> k-space gather -> the pass that forms F
+int force_pipeline(Ctx &c, bool debug) {
+  const bool cp = !c.rbl && !c.vl_on && cpair_usable(c);
+  if (c.Nq > 0 && !c.rec && !c.timing && c.aux_stream) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    RBE_CUDA_TRY(cudaStreamIsCapturing(c.stream, &st));
+    if (st == cudaStreamCaptureStatusActive) return force_pipeline_forked(c, cp, debug);
+  }
+  mark(c, RBE_PH_BIN);
+  if (c.vl_on) RBE_CUDA_TRY(launch_list_check(c));
+  RBE_CUDA_TRY(launch_bin_sort(c));
+  mark(c, RBE_PH_SAMPLE);
+  RBE_CUDA_TRY(launch_sample_k(c));
+  mark(c, RBE_PH_SF);
+  RBE_CUDA_TRY(launch_structure_factor(c));
+  mark(c, RBE_PH_LIST);
+  int rc = lists(c, cp);
+  if (rc != RBE_OK) return rc;
   mark(c, RBE_PH_PAIR);
-  if (c.rbl) RBE_CUDA_TRY(launch_rbl(c, debug));
-  else if (c.vl_on) RBE_CUDA_TRY(launch_list_pair(c, debug));
-  else if (cp) RBE_CUDA_TRY(launch_pair_cluster(c, debug));
-  else RBE_CUDA_TRY(launch_pair(c, debug));
+  rc = real_space(c, cp, true, debug);
+  if (rc != RBE_OK) return rc;
   mark(c, RBE_PH_GATHER);
   RBE_CUDA_TRY(launch_kspace_gather(c, cp));
   mark(c, RBE_PH_TAIL);
-  if (cp) RBE_CUDA_TRY(launch_cluster_finish(c));
-  return RBE_OK;
+  return finish_forces(c, cp);
 }
 
 // Kernels one Verlet step launches (memsets excluded).
@@ -267,6 +293,9 @@ int64_t kernels_per_step(const Ctx &c) {
   if (c.vl_on)                           // check, identity copy, build(s), commit
     k += 3 + ((c.Nq * 2 > c.N || c.Nq == 0) ? 1 : 2);
   k += c.Nq > 0 ? 1 : 0;                 // gather
+  if (c.rbl ? c.Nq > 0 && c.Nq < c.N : c.vl_on || !cpair_usable(c))
+    k += c.Nq > 0 ? 1 : 0;               // the k-space forces added to F
+  if (!c.rbl && !c.vl_on && !cpair_usable(c) && pair_split(c) > 1) k += 1;  // parts of the pair pass
   k += 2;                                // kick (+kinetic), totals
   k += (partials_compact_count(c.n_pair_blk) > 0 ? 1 : 0) +  // partials compaction
        (partials_compact_count(c.n_coul_blk) > 0 ? 1 : 0);
@@ -318,6 +347,7 @@ int capture_step_graph(Ctx &c, int parity, cudaGraphExec_t *out, bool forces_onl
   if (!c.cap_stream) RBE_CUDA_TRY(cudaStreamCreateWithFlags(&c.cap_stream, cudaStreamNonBlocking));
   if (!c.aux_stream) RBE_CUDA_TRY(cudaStreamCreateWithFlags(&c.aux_stream, cudaStreamNonBlocking));
   if (!c.ev_fork) RBE_CUDA_TRY(cudaEventCreateWithFlags(&c.ev_fork, cudaEventDisableTiming));
+  if (!c.ev_bin) RBE_CUDA_TRY(cudaEventCreateWithFlags(&c.ev_bin, cudaEventDisableTiming));
   if (!c.ev_join) RBE_CUDA_TRY(cudaEventCreateWithFlags(&c.ev_join, cudaEventDisableTiming));
   const int saved = c.cur;
   cudaStream_t user = c.stream;
@@ -580,6 +610,7 @@ int rbe_init(rbe_handle *hout, const rbe_params *p, int64_t N, const double box[
     if (!fp64) rc |= dalloc(c, &c.cjrec, 8 * cpair_clusters_bound(c));  // 8 slots per cluster
     rc |= dalloc(c, &c.cq4, Nq);
   }
+  rc |= dalloc(c, reinterpret_cast<char **>(&c.fk), 3 * Nq * (fp64 ? 8 : 4));
   rc |= dalloc(c, &c.cs, 3 * Nq);
   rc |= dalloc(c, &c.cqf, Nq);
   if (fp64) rc |= dalloc(c, &c.cqd, Nq);

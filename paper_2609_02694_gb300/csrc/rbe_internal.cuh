@@ -119,6 +119,8 @@ struct Ctx {
   float *invm[2] = {nullptr, nullptr};
   float *F = nullptr;
   double *Fd = nullptr;
+  void *fk = nullptr;          // k-space forces in charged order, 3 Nq of the form's type (unless
+                               // the gather adds to the cluster kernel's fixed-point sums)
   double *fpart = nullptr;     // per-particle pair kernel: partial forces of a split pass
   // cluster-pair kernel: fixed-point force sums (3N, sorted order), per-row cluster and
   // super-cluster offsets (rows + 1 each), per-cluster bounds
@@ -202,7 +204,8 @@ struct Ctx {
   cudaGraphExec_t fgraph[2] = {nullptr, nullptr}; // force evaluations (rbe_forces), the same
   cudaStream_t cap_stream = nullptr;  // internal non-blocking stream used only for capture
   cudaStream_t aux_stream = nullptr;  // second capture stream: the k-space branch of a step
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;  // (fork and join of that branch)
+  cudaEvent_t ev_fork = nullptr, ev_bin = nullptr, ev_join = nullptr;  // (its fork, its wait for
+                                                                      // the binning, its join)
   // profiling: ev[k] is recorded before phase k, ev[RBE_N_PHASE] after the last one
   bool timing = false;
   cudaEvent_t ev[RBE_N_PHASE + 1] = {};
@@ -443,7 +446,8 @@ cudaError_t fill_zero(Ctx &c, void *p, int64_t words);
 cudaError_t launch_sample_k(Ctx &c);
 cudaError_t launch_bin_sort(Ctx &c);
 cudaError_t launch_structure_factor(Ctx &c);
-cudaError_t launch_kspace_gather(Ctx &c, bool into_facc);
+cudaError_t launch_kspace_gather(Ctx &c, bool into_facc);  // to fk, or into the fixed-point sums
+cudaError_t launch_kspace_add(Ctx &c);                     // F += fk
 cudaError_t launch_pair(Ctx &c, bool want_counts);   // per-particle pass, then mark, then Coulomb pass
 // Cluster-pair kernel (k_cpair.cu): whether it applies to the handle's box and tuning, the
 // launch bounds of its super-clusters and clusters, and the launch (tables, pairs, finish).
@@ -459,7 +463,8 @@ cudaError_t launch_pair_cluster(Ctx &c, bool want_counts);
 int64_t coul_blocks(int64_t nq);
 cudaError_t launch_coulomb_subset(Ctx &c, const uint4 *s4, bool into_facc);
 void mark(Ctx &c, int k);  // record the profiling event k (no-op when profiling is off)
-cudaError_t launch_rbl(Ctx &c, bool want_debug);
+cudaError_t launch_rbl(Ctx &c, bool want_debug);  // up to the mean force
+cudaError_t launch_rbl_finish(Ctx &c);             // F -= mean, += the k-space forces
 cudaError_t launch_list_check(Ctx &c);    // rebuild flag from the displacements
 cudaError_t launch_list_build(Ctx &c);    // gated list build(s) at r_c + skin
 cudaError_t launch_list_commit(Ctx &c);   // gated: reference positions, counters
