@@ -296,6 +296,7 @@ struct TotalsArgs {
 // warps: the warp reductions of seven FP64 sums dominate on one SM (FP64 runs at 1/64 of the
 // FP32 rate), and they scale with the warps, the strided sums do not.
 constexpr int kTotalsThreads = 128;
+constexpr int64_t kTotalsDirect = 1024;  // partials of a pass it reads without a compaction
 
 template <typename ACC>
 __device__ __forceinline__ void totals_body(const TotalsArgs &a, int, int) {
@@ -496,16 +497,19 @@ cudaError_t launch_kinetic(Ctx &c) { return kick_impl(c, 0); }
 // Block partials of a pair pass ([nblk][NQ_PAIR]) summed over fixed contiguous ranges in a
 // fixed order into [gridDim.x][NQ_PAIR]: the FP64 adds are spread over many SMs (one SM's
 // FP64 rate is low) before the one-block totals.
-struct CompactArgs {
-  const double *in;
-  int64_t nblk, per;
-  double *out;
+struct CompactArgs {       // two passes' partials: blocks [0, nc0) the first, the rest the second
+  const double *in[2];
+  int64_t nblk[2], per[2];
+  double *out[2];
+  int nc0;
 };
 
 __device__ __forceinline__ void partials_compact_body(const CompactArgs &a, int bx, int) {
-  __shared__ double sh[NQ_PAIR][256];
-  const double *__restrict__ in = a.in;
-  const int64_t nblk = a.nblk, per = a.per;
+  __shared__ double sh[NQ_PAIR][8];
+  const int w = bx >= a.nc0 ? 1 : 0;
+  if (w) bx -= a.nc0;
+  const double *__restrict__ in = a.in[w];
+  const int64_t nblk = a.nblk[w], per = a.per[w];
   const int64_t b0 = (int64_t)bx * per, b1 = min(nblk, b0 + per);
   double acc[NQ_PAIR];
 #pragma unroll
@@ -513,43 +517,48 @@ __device__ __forceinline__ void partials_compact_body(const CompactArgs &a, int 
   for (int64_t b = b0 + threadIdx.x; b < b1; b += blockDim.x)
 #pragma unroll
     for (int k = 0; k < NQ_PAIR; ++k) acc[k] += in[b * NQ_PAIR + k];
-#pragma unroll
-  for (int k = 0; k < NQ_PAIR; ++k) sh[k][threadIdx.x] = acc[k];
+  const int lane = threadIdx.x & 31;
+  const double v[8] = {acc[0], acc[1], acc[2], acc[3], 0.0, 0.0, 0.0, 0.0};
+  const double s = warp_sum8(v, lane);
+  if (lane < NQ_PAIR) sh[lane][threadIdx.x >> 5] = s;
   __syncthreads();
-  for (int st = 128; st > 0; st >>= 1) {
-    if (threadIdx.x < st)
-#pragma unroll
-      for (int k = 0; k < NQ_PAIR; ++k) sh[k][threadIdx.x] += sh[k][threadIdx.x + st];
-    __syncthreads();
+  if (threadIdx.x < NQ_PAIR) {
+    double t = 0.0;
+    for (int k = 0; k < 8; ++k) t += sh[threadIdx.x][k];
+    a.out[w][(int64_t)bx * NQ_PAIR + threadIdx.x] = t;
   }
-  if (threadIdx.x < NQ_PAIR) a.out[(int64_t)bx * NQ_PAIR + threadIdx.x] = sh[threadIdx.x][0];
 }
 RBE_BATCHED_KERNEL(__launch_bounds__(256), partials_compact_kernel, CompactArgs,
                    partials_compact_body)
 
-int64_t partials_compact_count(int64_t nblk) { return std::min<int64_t>(nblk, kCompactMax); }
+// Blocks of the compaction of nblk partials (0: few enough for the totals to read themselves);
+// one for each 256 partials, at most kCompactMax.
+int64_t partials_compact_count(int64_t nblk) {
+  return nblk <= kTotalsDirect ? 0 : std::min<int64_t>((nblk + 255) / 256, kCompactMax);
+}
 
 cudaError_t launch_totals(Ctx &c) {
   TotalsArgs a;
-  // pair and Coulomb-pass partials, compacted first (at most kCompactMax per pass)
-  const int64_t ncp = partials_compact_count(c.n_pair_blk), ncc = partials_compact_count(c.n_coul_blk);
+  // pair and Coulomb-pass partials, compacted first where there are many, by one launch for both
+  const int64_t n[2] = {c.n_pair_blk, c.n_coul_blk};
+  const double *part[2] = {c.epart + c.off_pair, c.epart + c.off_coul};
+  const int64_t nc[2] = {partials_compact_count(n[0]), partials_compact_count(n[1])};
   cudaError_t e;
-  if (ncp > 0) {
-    const CompactArgs ca{c.epart + c.off_pair, c.n_pair_blk, (c.n_pair_blk + ncp - 1) / ncp,
-                         c.ecomp};
-    e = dispatch(c, partials_compact_kernel, partials_compact_kernel_b, dim3((unsigned)ncp),
-                 dim3(256), 0, ca);
+  {  // (recorded without blocks too, so that boxes of any size share a batch's class)
+    CompactArgs ca{};
+    for (int w = 0; w < 2; ++w) {
+      ca.in[w] = part[w];
+      ca.nblk[w] = n[w];
+      ca.per[w] = nc[w] ? (n[w] + nc[w] - 1) / nc[w] : 0;
+      ca.out[w] = c.ecomp + w * kCompactMax * NQ_PAIR;
+    }
+    ca.nc0 = (int)nc[0];
+    e = dispatch(c, partials_compact_kernel, partials_compact_kernel_b,
+                 dim3((unsigned)(nc[0] + nc[1])), dim3(256), 0, ca);
     if (e != cudaSuccess) return e;
   }
-  if (ncc > 0) {
-    const CompactArgs ca{c.epart + c.off_coul, c.n_coul_blk, (c.n_coul_blk + ncc - 1) / ncc,
-                         c.ecomp + kCompactMax * NQ_PAIR};
-    e = dispatch(c, partials_compact_kernel, partials_compact_kernel_b, dim3((unsigned)ncc),
-                 dim3(256), 0, ca);
-    if (e != cudaSuccess) return e;
-  }
-  a.pair = c.ecomp; a.n_pair = ncp;
-  a.coul = c.ecomp + kCompactMax * NQ_PAIR; a.n_coul = ncc;
+  a.pair = nc[0] ? c.ecomp : part[0]; a.n_pair = nc[0] ? nc[0] : n[0];
+  a.coul = nc[1] ? c.ecomp + kCompactMax * NQ_PAIR : part[1]; a.n_coul = nc[1] ? nc[1] : n[1];
   // RBL partials: the compacted ones (rbl_compact_kernel runs after the RBL kernel)
   a.rbl = c.rbl ? c.rbl_cpart : c.epart + c.off_rbl;
   a.n_rbl = c.rbl ? rbl_compact_count(c.n_rbl_blk) : 0;

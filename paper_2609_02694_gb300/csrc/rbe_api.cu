@@ -223,8 +223,9 @@ int lists(Ctx &c, bool cp) {
 // cluster kernel, the charged subset's Coulomb pass beside the real-space pass; then the pass that
 // forms F. Each branch writes its own arrays (or adds integers to the fixed-point sums), so the
 // forces are those of the sequential order bit for bit. The real-space passes issue in 60 to 75%
-// of their slots; the other branch's kernels fill slots and SMs they leave idle (measured with
-// the cluster kernel on 2^20 particles: 1.445 -> 1.360 ms a step; FORK_FIGURES).
+// of their slots; the other branch's kernels fill slots and SMs they leave idle
+// (measured, a step: cluster kernel on 2^20 particles 1.445 -> 1.360 ms; random batch list on
+// 200,000 / 1,400,000 ions 258 -> 225 / 1,226 -> 1,135 us; Verlet list on 100,000 ions 123 -> 100).
 int force_pipeline_forked(Ctx &c, bool cp, bool debug) {
   const cudaStream_t main_stream = c.stream;
   RBE_CUDA_TRY(cudaEventRecord(c.ev_fork, main_stream));
@@ -283,7 +284,7 @@ int force_pipeline(Ctx &c, bool debug) {
 // Kernels one Verlet step launches (memsets excluded).
 int64_t kernels_per_step(const Ctx &c) {
   int64_t k = 1;                         // kick-drift (with the step counter)
-  k += 6;                                // count, 3 scan passes, scatter, rank+permute
+  k += c.scan_nblk > 1 ? 5 : 4;          // count, scan (one or two passes), scatter, rank+permute
   k += 1;                                // sampler
   k += c.Nq > 0 ? 2 : 0;                 // structure factor + combine
   if (c.rbl) k += 4;                     // RBL, compact partials, mean, subtract
@@ -297,8 +298,7 @@ int64_t kernels_per_step(const Ctx &c) {
     k += c.Nq > 0 ? 1 : 0;               // the k-space forces added to F
   if (!c.rbl && !c.vl_on && !cpair_usable(c) && pair_split(c) > 1) k += 1;  // parts of the pair pass
   k += 2;                                // kick (+kinetic), totals
-  k += (partials_compact_count(c.n_pair_blk) > 0 ? 1 : 0) +  // partials compaction
-       (partials_compact_count(c.n_coul_blk) > 0 ? 1 : 0);
+  k += partials_compact_count(c.n_pair_blk) + partials_compact_count(c.n_coul_blk) > 0 ? 1 : 0;
   if (c.nvt) k += 2;                     // thermostat, end-of-step velocity scaling
   return k;
 }
@@ -702,6 +702,7 @@ int rbe_init(rbe_handle *hout, const rbe_params *p, int64_t N, const double box[
       e |= cudaMemcpy(c.T[d], T[d].data(), sizeof(uint64_t) * T[d].size(), cudaMemcpyHostToDevice);
     e |= cudaMemcpy(c.lj_dev, &c.lj, sizeof(LJTable), cudaMemcpyHostToDevice);
     e |= cudaMemset(c.epart, 0, sizeof(double) * c.epart_slots);
+    e |= cudaMemset(c.cell_count, 0, sizeof(int32_t) * 2 * c.grid.ncell);
     e |= cudaMemset(c.emode, 0, sizeof(double) * 2 * c.P);
     e |= cudaMemset(c.err, 0, sizeof(int));
     if (c.facc) e |= cudaMemset(c.facc, 0, sizeof(long long) * 3 * N);
