@@ -6,6 +6,8 @@
 //   ... forces at the new positions ...;  v += (F/m)(dt/2) kappa
 // Every kernel here is a single streaming pass (HBM-bound) except the totals, which sum
 // the per-block partials of all force kernels in a fixed order (latency-bound).
+#include <cmath>
+
 #include "rbe_internal.cuh"
 
 namespace rbe {
@@ -130,53 +132,76 @@ struct KickArgs {
   double *ke_part;
 };
 
+// Particles a block of the kick kernels, four consecutive ones a thread. The kinetic energy's terms
+// are summed in FP64: a thread's four, then the warp's, then the warps' in order, the same in the
+// scalar and the 16-byte kernel, so their partials agree bit for bit. (One particle a thread and
+// a 256-term tree left the pass waiting on memory and barriers: the kinetic energy of 4,000,001
+// particles by the scalar kernel 76 -> 30 us, and the totals over a quarter of the partials
+// 30 -> 14 us.)
+constexpr int kKickThreads = 256;
+
+__device__ __forceinline__ void kick_reduce(const double (&ke)[4], double *out) {
+  __shared__ double sh[kKickThreads / 32];
+  const double s = warp_sum((ke[0] + ke[1]) + (ke[2] + ke[3]));
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int w = 0; w < kKickThreads / 32; ++w) t += sh[w];
+    *out = t;
+  }
+}
+
 template <typename V, typename FT>
 __device__ __forceinline__ void kick_body(const KickArgs<V, FT> &a, int bx, int) {
-  __shared__ double sh[256];
   V *__restrict__ v = a.v;
   const FT *__restrict__ F = a.F;
   const float *__restrict__ invm = a.invm;
   const int64_t N = a.N;
-  const double hdk = a.hdk, inv_kappa = a.inv_kappa;
-  const int do_kick = a.do_kick;
-  const int64_t i = (int64_t)bx * blockDim.x + threadIdx.x;
-  double ke = 0.0;
-  if (i < N) {
-    const V im = (V)invm[i];
+  const int64_t i0 = 4 * ((int64_t)bx * kKickThreads + threadIdx.x);
+  V vv[4][3];
+  float im[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int64_t i = min(i0 + j, N - 1);
+    im[j] = invm[i];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) vv[j][d] = v[d * N + i];
+  }
+  if (a.do_kick) {
+    FT f[4][3];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int d = 0; d < 3; ++d) f[j][d] = F[d * N + min(i0 + j, N - 1)];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        vv[j][d] += (V)f[j][d] * (V)im[j] * (V)a.hdk;
+        if (i0 + j < N) v[d * N + i0 + j] = vv[j][d];
+      }
+  }
+  double ke[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
     V v2 = (V)0;
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      V vv = v[d * N + i];
-      if (do_kick) {
-        vv += (V)F[d * N + i] * im * (V)hdk;
-        v[d * N + i] = vv;
-      }
-      v2 += vv * vv;
-    }
+    for (int d = 0; d < 3; ++d) v2 += vv[j][d] * vv[j][d];
     // 1/2 m v^2 / kappa, m = 1 / (1/m): FP64 in the FP64 form; the FP32 forms form each
     // particle's term in FP32 and sum the terms in FP64
-    if (sizeof(V) == 8) ke = 0.5 * (double)v2 / (double)invm[i] * inv_kappa;
-    else ke = f2d(0.5f * (float)v2 * __frcp_rn(invm[i]) * (float)inv_kappa);
+    if (i0 + j >= N) ke[j] = 0.0;
+    else if (sizeof(V) == 8) ke[j] = 0.5 * (double)v2 / (double)im[j] * a.inv_kappa;
+    else ke[j] = f2d(0.5f * (float)v2 * __frcp_rn(im[j]) * (float)a.inv_kappa);
   }
-  sh[threadIdx.x] = ke;
-  __syncthreads();
-  for (int st = 128; st > 0; st >>= 1) {
-    if (threadIdx.x < st) sh[threadIdx.x] += sh[threadIdx.x + st];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) a.ke_part[bx] = sh[0];
+  kick_reduce(ke, a.ke_part + bx);
 }
-RBE_VF_KERNELS(__launch_bounds__(256), kick_kernel, KickArgs, kick_body)
+RBE_VF_KERNELS(__launch_bounds__(kKickThreads), kick_kernel, KickArgs, kick_body)
 
-// The FP32 forms with N a multiple of 4: blocks of 64 threads over the same 256 particles as
-// kick_body's blocks, four consecutive particles a thread in 16-byte accesses. Each particle's
-// arithmetic, its term's shared-memory slot and the reduction tree are kick_body's, so the
-// kinetic energy partials are the same bit for bit.
+// The FP32 forms with N a multiple of 4: the same in 16-byte accesses.
 __device__ __forceinline__ void kick4_body(const KickArgs<float, float> &a, int bx, int) {
-  __shared__ double sh[256];
   const int64_t N = a.N;
-  const int t = threadIdx.x;
-  const int64_t i = (int64_t)bx * 256 + 4 * t;
+  const int64_t i = 4 * ((int64_t)bx * kKickThreads + threadIdx.x);
   const float hdk = (float)a.hdk, ik = (float)a.inv_kappa;
   double ke[4] = {0.0, 0.0, 0.0, 0.0};
   if (i < N) {  // (all four, N being a multiple of 4)
@@ -204,17 +229,10 @@ __device__ __forceinline__ void kick4_body(const KickArgs<float, float> &a, int 
     ke[2] = f2d(0.5f * v2[2] * __frcp_rn(im.z) * ik);
     ke[3] = f2d(0.5f * v2[3] * __frcp_rn(im.w) * ik);
   }
-#pragma unroll
-  for (int j = 0; j < 4; ++j) sh[4 * t + j] = ke[j];
-  __syncthreads();
-  for (int st = 128; st > 0; st >>= 1) {
-    for (int k = t; k < st; k += 64) sh[k] += sh[k + st];
-    __syncthreads();
-  }
-  if (t == 0) a.ke_part[bx] = sh[0];
+  kick_reduce(ke, a.ke_part + bx);
 }
 using KickArgsF = KickArgs<float, float>;
-RBE_BATCHED_KERNEL(__launch_bounds__(64), kick4_kernel, KickArgsF, kick4_body)
+RBE_BATCHED_KERNEL(__launch_bounds__(kKickThreads), kick4_kernel, KickArgsF, kick4_body)
 
 // Nose-Hoover half steps (chain of one): from 2K = 2 sum(kinetic partials) the end-of-step
 // half (mode 0) gives the velocity scale s_end and the start-of-next-step half gives
@@ -235,6 +253,7 @@ __device__ __forceinline__ void thermostat_body(const ThermoArgs &a, int, int) {
   double *__restrict__ th = a.th;
   const int mode = a.mode;
   double acc = 0.0;
+#pragma unroll 4
   for (int64_t b = threadIdx.x; b < n; b += blockDim.x) acc += ke_part[b];
   sh[threadIdx.x] = acc;
   __syncthreads();
@@ -316,6 +335,7 @@ __device__ __forceinline__ void totals_body(const TotalsArgs &a, int, int) {
     acc[4] += (ACC)a.emode[2 * l];
     acc[5] += (ACC)a.emode[2 * l + 1];
   }
+#pragma unroll 4
   for (int64_t b = threadIdx.x; b < a.n_ke; b += blockDim.x) acc[6] += (ACC)a.ke[b];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   for (int k = 0; k < NV; ++k) {
@@ -391,19 +411,46 @@ __global__ void scatter_state_kernel(const uint32_t *__restrict__ s, const V *__
   }
 }
 
-__global__ void set_positions_kernel(const double *__restrict__ pos, const int32_t *__restrict__ id,
-                                     int64_t N, double Lx, double Ly, double Lz,
-                                     uint32_t *__restrict__ s) {
+// A position's fractional coordinate s = rint(fl(r / L) 2^32) mod 2^32 (fl: rounded to double).
+// For 0 <= r < L it is formed in integers, since FP64 runs at 1/64 of the FP32 rate: with r = M
+// 2^(e - 63) (M the 64-bit left-aligned significand) and K = floor(2^sh / L) in [2^63, 2^64), the
+// high half of M K shifted right by n = sh - 64 - e is r / L in 2^-63 units, short by less than 4.
+// fl moves the quotient by at most 2^10 of those units, so s rounds as in the FP64 expression
+// unless the fraction of s (31 bits) is within 2^12 of one half: those (one in 260,000) and all
+// other positions take that expression. The pass is bound by its 144 MB at 4,000,001 particles (309 us
+// with the FP64 expression throughout, 32 us so; a divide is some 20 FP64 instructions).
+__device__ __forceinline__ uint32_t quantise_f64(double r, double L) {
+  const double f = __dmul_rn(__ddiv_rn(r, L), kTwo32);
+  const double fm = f - kTwo32 * floor(f / kTwo32);  // wrap into [0, 2^32)
+  return (uint32_t)(unsigned long long)__double2ll_rn(fm);
+}
+__device__ __forceinline__ uint32_t quantise_pos(double r, double L, unsigned long long K, int sh) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(r);
+  if (b == 0ull) return 0u;
+  const int e = (int)(b >> 52) - 1023;  // (a negative r: e >= 1025)
+  const int n = sh - 64 - e;
+  if (n < 0 || n > 63 || e < -1000) return quantise_f64(r, L);
+  const unsigned long long M = (b << 11) | 0x8000000000000000ull;
+  const unsigned long long F = __umul64hi(M, K) >> n;  // (2^63 and more: r >= L)
+  const uint32_t frac = (uint32_t)F & 0x7fffffffu;
+  if ((F >> 63) || frac - 0x3ffff000u < 0x2000u) return quantise_f64(r, L);
+  return (uint32_t)(F >> 31) + (frac >> 30);
+}
+
+struct PosScale {
+  double L[3];
+  unsigned long long K[3];
+  int sh[3];
+};
+__global__ void __launch_bounds__(256)
+    set_positions_kernel(const double *__restrict__ pos, const int32_t *__restrict__ id, int64_t N,
+                         const PosScale p, uint32_t *__restrict__ s) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= N) return;
   const int64_t o = (int64_t)id[k] * 3;
-  const double L[3] = {Lx, Ly, Lz};
+  const double r[3] = {pos[o], pos[o + 1], pos[o + 2]};
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const double f = __dmul_rn(__ddiv_rn(pos[o + d], L[d]), kTwo32);
-    const double fm = f - kTwo32 * floor(f / kTwo32);  // wrap into [0, 2^32)
-    s[d * N + k] = (uint32_t)(unsigned long long)__double2ll_rn(fm);
-  }
+  for (int d = 0; d < 3; ++d) s[d * N + k] = quantise_pos(r[d], p.L[d], p.K[d], p.sh[d]);
 }
 
 // Checkpoint load: state given in id order (row-major per particle) into the sorted slots.
@@ -477,7 +524,7 @@ static cudaError_t kick_impl(Ctx &c, int do_kick) {
   const int b = c.cur;
   const double hdk = 0.5 * c.dt * c.kappa;
   if (c.N == 0) return cudaSuccess;
-  const dim3 g(nblk(c.N, 256)), t(256);
+  const dim3 g(nblk(c.N, 4 * kKickThreads)), t(kKickThreads);
   if (c.precision == RBE_FP64) {
     const KickArgs<double, double> a{c.vd[b], c.Fd, c.invm[b], c.N, hdk, 1.0 / c.kappa, do_kick,
                                      c.epart + c.off_ke};
@@ -487,7 +534,7 @@ static cudaError_t kick_impl(Ctx &c, int do_kick) {
                                  c.epart + c.off_ke};
   // (a batch keeps the one-particle kernel: the same results, and replicas of any N share a
   //  class)
-  if (c.N % 4 == 0 && !c.rec) return dispatch(c, kick4_kernel, kick4_kernel_b, g, dim3(64), 0, a);
+  if (c.N % 4 == 0 && !c.rec) return dispatch(c, kick4_kernel, kick4_kernel_b, g, t, 0, a);
   return dispatch(c, kick_kernel<float, float>, kick_kernel_b<float, float>, g, t, 0, a);
 }
 
@@ -574,15 +621,16 @@ cudaError_t launch_totals(Ctx &c) {
                   dim3(kTotalsThreads), 0, a);
 }
 
-cudaError_t launch_scatter_forces(Ctx &c, bool to_double) {
+cudaError_t launch_scatter_forces(Ctx &c, bool to_double, float *outf) {
   const int b = c.cur;
   if (c.N == 0) return cudaSuccess;
+  if (!outf) outf = c.outf;
   if (c.precision == RBE_FP64) {
     if (to_double) scatter_forces_kernel<double, double><<<nblk(c.N, 256), 256, 0, c.stream>>>(c.Fd, c.id[b], c.N, c.outd);
-    else scatter_forces_kernel<double, float><<<nblk(c.N, 256), 256, 0, c.stream>>>(c.Fd, c.id[b], c.N, c.outf);
+    else scatter_forces_kernel<double, float><<<nblk(c.N, 256), 256, 0, c.stream>>>(c.Fd, c.id[b], c.N, outf);
   } else {
     if (to_double) scatter_forces_kernel<float, double><<<nblk(c.N, 256), 256, 0, c.stream>>>(c.F, c.id[b], c.N, c.outd);
-    else scatter_forces_kernel<float, float><<<nblk(c.N, 256), 256, 0, c.stream>>>(c.F, c.id[b], c.N, c.outf);
+    else scatter_forces_kernel<float, float><<<nblk(c.N, 256), 256, 0, c.stream>>>(c.F, c.id[b], c.N, outf);
   }
   return cudaGetLastError();
 }
@@ -599,11 +647,33 @@ cudaError_t launch_scatter_state(Ctx &c, int what) {
   return cudaGetLastError();
 }
 
+// K = floor(2^sh / L) in [2^63, 2^64) by long division of powers of two by L's significand.
+static unsigned long long inverse_bits(double L, int *sh) {
+  int e = 0;
+  const double m = std::frexp(L, &e);                              // L = m 2^e, m in [1/2, 1)
+  const unsigned long long D = (unsigned long long)std::ldexp(m, 53);  // L = D 2^(e - 53)
+  // K = floor(2^k / D), k the largest with K < 2^64: k = 116 (D in [2^52, 2^53)), or 115 for a
+  // power of two (2^116 / 2^52 = 2^64)
+  const int k = D == (1ull << 52) ? 115 : 116;
+  unsigned long long q = 0, r = 0;
+  for (int i = k; i >= 0; --i) {
+    r = 2 * r + (i == k ? 1ull : 0ull);
+    q = 2 * q + (r >= D ? 1ull : 0ull);
+    if (r >= D) r -= D;
+  }
+  *sh = k + e - 53;  // 1 / L = 2^(53 - e) / D
+  return q;
+}
+
 cudaError_t launch_set_positions(Ctx &c) {
   const int b = c.cur;
   if (c.N == 0) return cudaSuccess;
-  set_positions_kernel<<<nblk(c.N, 256), 256, 0, c.stream>>>(c.pos_stage, c.id[b], c.N, c.box[0],
-                                                             c.box[1], c.box[2], c.s[b]);
+  PosScale p;
+  for (int d = 0; d < 3; ++d) {
+    p.L[d] = c.box[d];
+    p.K[d] = inverse_bits(c.box[d], &p.sh[d]);
+  }
+  set_positions_kernel<<<nblk(c.N, 256), 256, 0, c.stream>>>(c.pos_stage, c.id[b], c.N, p, c.s[b]);
   return cudaGetLastError();
 }
 

@@ -575,7 +575,7 @@ int rbe_init(rbe_handle *hout, const rbe_params *p, int64_t N, const double box[
   c.n_coul_blk = rbl ? 0 : std::max(pair_blocks(Nq), coul_blocks(Nq));
   c.n_rbl_blk = rbl ? rbl_blocks(N) : 0;
   c.rbl_nslots = rbl ? rbl_slot_count(N, c.sms) : 0;
-  c.n_ke_blk = (N + 255) / 256;
+  c.n_ke_blk = (N + 1023) / 1024;  // (the kick kernels' blocks)
   c.off_pair = 0;
   c.off_coul = c.off_pair + c.n_pair_blk * NQ_PAIR;
   c.off_rbl = c.off_coul + c.n_coul_blk * NQ_PAIR;
@@ -790,10 +790,21 @@ int rbe_forces(rbe_handle h, uint64_t step, float *F_out, int F_on_device, doubl
   int rc = forces_common(h, step, false);  // no neighbour counts or RBL partners
   if (rc != RBE_OK) return rc;
   if (F_out) {
-    RBE_CUDA_TRY(launch_scatter_forces(c, false));
-    RBE_CUDA_TRY(cudaMemcpyAsync(F_out, c.outf, sizeof(float) * 3 * c.N,
-                                 F_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                                 c.stream));
+    // straight into memory of this device; staged for the host or another device
+    bool direct = false;
+    if (F_on_device && reinterpret_cast<uintptr_t>(F_out) % sizeof(float) == 0) {
+      cudaPointerAttributes at;
+      int dev = -1;
+      direct = cudaPointerGetAttributes(&at, F_out) == cudaSuccess &&
+               at.type == cudaMemoryTypeDevice && cudaGetDevice(&dev) == cudaSuccess &&
+               at.device == dev;
+      if (!direct) cudaGetLastError();
+    }
+    RBE_CUDA_TRY(launch_scatter_forces(c, false, direct ? F_out : nullptr));
+    if (!direct)
+      RBE_CUDA_TRY(cudaMemcpyAsync(F_out, c.outf, sizeof(float) * 3 * c.N,
+                                   F_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
+                                   c.stream));
   }
   if (energies || virial) {
     rc = copy_scalars(c, energies, virial);

@@ -483,7 +483,8 @@ void zero_partials_tail(Ctx &c, int64_t off, int64_t written, int64_t capacity);
 double frame_band(const double X[3], double r, const double box[3], bool wrap);
 cudaError_t launch_set_step(Ctx &c, uint64_t step);
 cudaError_t launch_step_advance(Ctx &c);
-cudaError_t launch_scatter_forces(Ctx &c, bool to_double);
+// Forces in id order, to outf (device; null: c.outf) or c.outd.
+cudaError_t launch_scatter_forces(Ctx &c, bool to_double, float *outf = nullptr);
 cudaError_t launch_scatter_state(Ctx &c, int what);  // 0: positions, 1: velocities, 2: s
 cudaError_t launch_set_positions(Ctx &c);
 // Checkpoint load: positions (uint32) and velocities (double), id order, into the sorted slots.
