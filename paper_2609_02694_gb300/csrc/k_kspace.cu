@@ -14,8 +14,10 @@
 // reduction. Each block writes compensated FP32 partials of its particle tile for a
 // contiguous slice of modes (one thread per mode, particles broadcast from shared memory,
 // no atomics). A combine kernel then sums the partials in FP64 in a fixed order, so the
-// result is reproducible run to run. Both passes are bound by the SFU (one sincos per
-// particle and mode) and FP32/INT issue.
+// result is reproducible run to run. In the FP32 forms both passes are bound by FMA and issue slots
+// (three integer multiply-adds, a sine and a cosine, five to nine further operations a particle
+// and mode), so they take two phases a step, on packed pairs where those are not the slower form.
+#include "f32x2.cuh"
 #include "rbe_internal.cuh"
 
 namespace rbe {
@@ -27,6 +29,7 @@ struct SfArgs {
   int64_t Nq;
   const int4 *m;
   int P, tile;
+  int slices;  // tiles a block (P <= 256; otherwise 1 and blockIdx.y counts the modes' blocks)
   double *part;
 };
 struct CombineArgs {
@@ -101,28 +104,62 @@ __device__ __forceinline__ void sincos_phase(uint32_t ph, double &sn, double &co
   co = __hiloint2double(__double2hiint(b) ^ (int)(((q + 1u) & 2u) << 30), __double2loint(b));
 }
 
+// A phase plus a bias, which rides on the multiply-adds.
+__device__ __forceinline__ uint32_t phase_add(int4 m, uint32_t x, uint32_t y, uint32_t z,
+                                              uint32_t bias) {
+  return (uint32_t)m.x * x + ((uint32_t)m.y * y + ((uint32_t)m.z * z + bias));
+}
+// The angles of two phases with kTurnBias added: the values of phase_to_radians, the exponent of
+// 2^23 set by the shift.
+constexpr uint32_t kTurnBias = 0x80000100u;
+__device__ __forceinline__ f32x2 turns_to_radians(uint32_t pa, uint32_t pb) {
+  const f32x2 f = pk(__uint_as_float(__funnelshift_r(pa, 150u, 9)),  // 2^23 + (p >> 9)
+                     __uint_as_float(__funnelshift_r(pb, 150u, 9)));
+  return mul2(add2(f, pk(-12582912.0f)), pk((float)(2.0 * kPi / 8388608.0)));
+}
+// The angles of two phases with kHalfBias added, from the middle of their half turn: 2^-24 turns,
+// twice as fine; bit 31 tells the second half turn, where sine and cosine change sign.
+constexpr uint32_t kHalfBias = 0x40000080u;
+__device__ __forceinline__ f32x2 half_turns_to_radians(uint32_t pa, uint32_t pb) {
+  const f32x2 f = pk(__uint_as_float(((pa >> 8) & 0x7fffffu) | 0x4b000000u),
+                     __uint_as_float(((pb >> 8) & 0x7fffffu) | 0x4b000000u));
+  return mul2(add2(f, pk(-12582912.0f)), pk((float)(kPi / 8388608.0)));
+}
+
 // MODE: 0 = FP32 with Kahan-compensated per-thread sums, 1 = plain FP32, 2 = FP64.
+// MODE 0 compensates the sum of two particles' terms at once. That alone would leave rho 0.5% less
+// exact (2.77e-7 against 64 bits for 200,000 ions); the finer phases more than make up for it
+// (1.98e-7). 1,400,000 ions, P = 200: 198 us with one particle a step and every term compensated
+// by itself, 184 on full warps (see sf_launch), 172 so.
 template <int MODE>
 __device__ __forceinline__ void sf_body(const SfArgs &a, int bx, int) {
-  extern __shared__ uint4 sh[];
+  extern __shared__ uint4 smem[];  // tile particles (an even number) a slice
+  uint4 *sh = smem;
   const uint32_t *__restrict__ cs = a.cs;
   const float *__restrict__ cqf = a.cqf;
   const double *__restrict__ cqd = a.cqd;
   const int64_t Nq = a.Nq;
   const int P = a.P, tile = a.tile;
-  const int64_t p0 = (int64_t)bx * tile;
-  const int np = (int)min((int64_t)tile, Nq - p0);
+  const int64_t b0 = (int64_t)bx * a.slices * tile;
+  const int nb = (int)min((int64_t)tile * a.slices, Nq - b0);
   double *shq = reinterpret_cast<double *>(sh + tile);
-  for (int k = threadIdx.x; k < np; k += blockDim.x) {
-    sh[k] = make_uint4(cs[p0 + k], cs[Nq + p0 + k], cs[2 * Nq + p0 + k],
-                       __float_as_uint(cqf[p0 + k]));
-    if (MODE == 2) shq[k] = cqd[p0 + k];
+  for (int k = threadIdx.x; k < nb; k += blockDim.x) {
+    sh[k] = make_uint4(cs[b0 + k], cs[Nq + b0 + k], cs[2 * Nq + b0 + k],
+                       __float_as_uint(cqf[b0 + k]));
+    if (MODE == 2) shq[k] = cqd[b0 + k];
   }
+  if (MODE != 2 && (nb & 1) && threadIdx.x == 0) sh[nb] = make_uint4(0u, 0u, 0u, 0u);  // no charge
   __syncthreads();
-  const int l = blockIdx.y * blockDim.x + threadIdx.x;
-  if (l >= P) return;
+  int l = blockIdx.y * blockDim.x + threadIdx.x, slice = 0;
+  if (MODE != 2 && a.slices > 1) {
+    slice = l / P;
+    l -= slice * P;
+    sh += slice * tile;
+  }
+  const int np = min(tile, nb - slice * tile);
+  if (l >= P || slice >= a.slices || np <= 0) return;
   const int4 mm = a.m[l];
-  double *out = a.part + ((int64_t)bx * P + l) * 2;
+  double *out = a.part + (((int64_t)bx * a.slices + slice) * P + l) * 2;
   if (MODE == 2) {
     double re = 0.0, im = 0.0;
     for (int k = 0; k < np; ++k) {
@@ -135,31 +172,43 @@ __device__ __forceinline__ void sf_body(const SfArgs &a, int bx, int) {
     out[0] = re;
     out[1] = im;
   } else {
-    float re = 0.f, im = 0.f, cre = 0.f, cim = 0.f;
-    for (int k = 0; k < np; ++k) {
-      const uint4 e = sh[k];
-      float sn, co;
-      __sincosf(phase_to_radians(phase_u32(mm, e.x, e.y, e.z)), &sn, &co);
-      const float q = __uint_as_float(e.w);
-      if (MODE == 0) {  // Kahan summation
-        const float yr = fmaf(q, co, -cre);
-        const float tr = re + yr;
-        cre = (tr - re) - yr;
-        re = tr;
-        const float yi = fmaf(q, sn, -cim);
-        const float ti = im + yi;
-        cim = (ti - im) - yi;
-        im = ti;
-      } else {
-        re = fmaf(q, co, re);
-        im = fmaf(q, sn, im);
+    f32x2 sum = pk(0.f), low = pk(0.f);  // (Re, Im) and what their additions dropped
+    const f32x2 m1 = pk(-1.f);
+    if (MODE == 0) {
+#pragma unroll 2
+      for (int k = 0; k < np; k += 2) {
+        const uint4 e = sh[k], g = sh[k + 1];
+        const uint32_t pa = phase_add(mm, e.x, e.y, e.z, kHalfBias),
+                       pb = phase_add(mm, g.x, g.y, g.z, kHalfBias);
+        const f32x2 w = half_turns_to_radians(pa, pb);
+        f32x2 ea, eb;
+        __sincosf(w.x, &ea.y, &ea.x);
+        __sincosf(w.y, &eb.y, &eb.x);
+        // the second half turn's sign, on the charge
+        const f32x2 qa = pk(__uint_as_float(e.w ^ (pa & 0x80000000u))),
+                    qb = pk(__uint_as_float(g.w ^ (pb & 0x80000000u)));
+        // Kahan summation of the pair's terms
+        const f32x2 y = fma2(qb, eb, fma2(qa, ea, low)), t = add2(sum, y);
+        low = fma2(fma2(sum, m1, t), m1, y);
+        sum = t;
+      }
+    } else {
+#pragma unroll 8
+      for (int k = 0; k < np; k += 2) {
+        const uint4 e = sh[k], g = sh[k + 1];
+        const f32x2 w = turns_to_radians(phase_add(mm, e.x, e.y, e.z, kTurnBias),
+                                         phase_add(mm, g.x, g.y, g.z, kTurnBias));
+        f32x2 ea, eb;
+        __sincosf(w.x, &ea.y, &ea.x);
+        __sincosf(w.y, &eb.y, &eb.x);
+        sum = fma2(pk(__uint_as_float(g.w)), eb, fma2(pk(__uint_as_float(e.w)), ea, sum));
       }
     }
-    out[0] = f2d(re) - f2d(cre);
-    out[1] = f2d(im) - f2d(cim);
+    out[0] = f2d(sum.x) + f2d(low.x);
+    out[1] = f2d(sum.y) + f2d(low.y);
   }
 }
-RBE_MODE_KERNELS(__launch_bounds__(256), sf_kernel, SfArgs, sf_body)
+RBE_MODE_KERNELS(__launch_bounds__(MODE == 2 ? 256 : 1024), sf_kernel, SfArgs, sf_body)
 
 // One block per mode: sum the block partials in a fixed order, then derive the per-mode
 // energy, virial and the gather coefficients (c Im rho, c Re rho).
@@ -224,6 +273,9 @@ constexpr int kGatherChunk = 256;
 template <int MODE> struct GatherReal { using type = float; };
 template <> struct GatherReal<2> { using type = double; };
 
+// FP32 forms: a thread takes the modes in pairs, whose data lie side by side in shared memory (two
+// 16-byte loads a mode instead of three): 1,400,000 charged, P = 200: 176 -> 156 us; 400,000, P = 500:
+// 137 -> 121 us.
 template <int MODE>
 __device__ __forceinline__ void gather_body(const GatherArgs &a, int bx, int) {
   const uint32_t *__restrict__ cs = a.cs;
@@ -234,9 +286,8 @@ __device__ __forceinline__ void gather_body(const GatherArgs &a, int bx, int) {
   const double4_16a *__restrict__ kcd = a.kcd;
   const float2 *__restrict__ abf = a.abf;
   const double2 *__restrict__ abd = a.abd;
-  __shared__ int4 sm[kGatherChunk];
-  __shared__ float4 skf[kGatherChunk];
-  __shared__ float2 sabf[kGatherChunk];
+  __shared__ int4 sm[MODE == 2 ? kGatherChunk : 1];
+  __shared__ float4 skp[MODE == 2 ? 1 : kGatherChunk * 2];  // 4 a pair of modes
   __shared__ double4_16a skd[MODE == 2 ? kGatherChunk : 1];
   __shared__ double2 sabd[MODE == 2 ? kGatherChunk : 1];
   const int nper = kGatherThreads / a.slices;  // particles a block (a multiple of 32)
@@ -245,23 +296,38 @@ __device__ __forceinline__ void gather_body(const GatherArgs &a, int bx, int) {
   const bool valid = i < Nq;
   const uint32_t sx = valid ? cs[i] : 0u, sy = valid ? cs[Nq + i] : 0u,
                  sz = valid ? cs[2 * Nq + i] : 0u;
-  float fx = 0.f, fy = 0.f, fz = 0.f;
+  f32x2 gx = pk(0.f), gy = pk(0.f), gz = pk(0.f);  // over the even and the odd modes
   double dx = 0.0, dy = 0.0, dz = 0.0;
   for (int l0 = 0; l0 < P; l0 += kGatherChunk) {
     const int nl = min(kGatherChunk, P - l0);
     __syncthreads();
-    for (int t = threadIdx.x; t < nl; t += blockDim.x) {
-      sm[t] = m[l0 + t];
-      if (MODE == 2) {
+    if (MODE == 2) {
+      for (int t = threadIdx.x; t < nl; t += blockDim.x) {
+        sm[t] = m[l0 + t];
         skd[t] = kcd[l0 + t];
         sabd[t] = abd[l0 + t];
-      } else {
-        skf[t] = kcf[l0 + t];
-        sabf[t] = abf[l0 + t];
+      }
+    } else {  // a pair of modes: (m.x, m.y) (m.z, A) (B, kx) (ky, kz) of both, side by side
+      for (int h = threadIdx.x; 2 * h < nl; h += blockDim.x) {
+        const int ta = l0 + 2 * h;
+        const bool two = 2 * h + 1 < nl;
+        const int4 ma = m[ta], mb = two ? m[ta + 1] : make_int4(0, 0, 0, 0);
+        const float4 ka = kcf[ta], kb = two ? kcf[ta + 1] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float2 ca = abf[ta], cb = two ? abf[ta + 1] : make_float2(0.f, 0.f);
+        float2 *o = reinterpret_cast<float2 *>(skp) + 8 * h;
+        o[0] = pk(__int_as_float(ma.x), __int_as_float(mb.x));
+        o[1] = pk(__int_as_float(ma.y), __int_as_float(mb.y));
+        o[2] = pk(__int_as_float(ma.z), __int_as_float(mb.z));
+        o[3] = pk(ca.x, cb.x);
+        o[4] = pk(-ca.y, -cb.y);
+        o[5] = pk(ka.x, kb.x);
+        o[6] = pk(ka.y, kb.y);
+        o[7] = pk(ka.z, kb.z);
       }
     }
     __syncthreads();
-    const int t0 = nl * slice / a.slices, t1 = nl * (slice + 1) / a.slices;
+    const int nt = MODE == 2 ? nl : (nl + 1) / 2;
+    const int t0 = nt * slice / a.slices, t1 = nt * (slice + 1) / a.slices;
     if (MODE == 2) {
       for (int t = t0; t < t1; ++t) {
         double sn, co;
@@ -272,16 +338,24 @@ __device__ __forceinline__ void gather_body(const GatherArgs &a, int bx, int) {
         dz = mad(g, skd[t].z, dz);
       }
     } else {
+#pragma unroll 2
       for (int t = t0; t < t1; ++t) {
-        float sn, co;
-        __sincosf(phase_to_radians(phase_u32(sm[t], sx, sy, sz)), &sn, &co);
-        const float g = mad(sabf[t].x, co, -(sabf[t].y * sn));
-        fx = fmaf(g, skf[t].x, fx);
-        fy = fmaf(g, skf[t].y, fy);
-        fz = fmaf(g, skf[t].z, fz);
+        const float4 u = skp[4 * t], v = skp[4 * t + 1], b = skp[4 * t + 2], k = skp[4 * t + 3];
+        const int4 ma = make_int4(__float_as_int(u.x), __float_as_int(u.z), __float_as_int(v.x), 0);
+        const int4 mb = make_int4(__float_as_int(u.y), __float_as_int(u.w), __float_as_int(v.y), 0);
+        const f32x2 w = turns_to_radians(phase_add(ma, sx, sy, sz, kTurnBias),
+                                         phase_add(mb, sx, sy, sz, kTurnBias));
+        f32x2 sn, co;
+        __sincosf(w.x, &sn.x, &co.x);
+        __sincosf(w.y, &sn.y, &co.y);
+        const f32x2 g = fma2(pk(v.z, v.w), co, mul2(pk(b.x, b.y), sn));
+        gx = fma2(g, pk(b.z, b.w), gx);
+        gy = fma2(g, pk(k.x, k.y), gy);
+        gz = fma2(g, pk(k.z, k.w), gz);
       }
     }
   }
+  float fx = gx.x + gx.y, fy = gy.x + gy.y, fz = gz.x + gz.y;
   if (a.slices > 1) {  // the slices' sums, added up in order
     using real = typename GatherReal<MODE>::type;
     __shared__ real part[3][kGatherThreads];
@@ -327,7 +401,7 @@ __device__ __forceinline__ void gather_body(const GatherArgs &a, int bx, int) {
     fk[2 * Nq + i] = -q * fz;
   }
 }
-RBE_MODE_KERNELS(__launch_bounds__(kGatherThreads), gather_kernel, GatherArgs, gather_body)
+RBE_MODE_KERNELS(__launch_bounds__(kGatherThreads, 1), gather_kernel, GatherArgs, gather_body)
 
 // F += the k-space forces of the charged particles (gather_kernel without fixed-point sums), so
 // that the gather can run beside the pass that writes F.
@@ -354,8 +428,19 @@ RBE_BATCHED_KERNEL(__launch_bounds__(256), kspace_add_kernel, KAddArgs, kspace_a
 
 template <int MODE>
 static cudaError_t sf_launch(Ctx &c, dim3 grid, size_t shm) {
-  const SfArgs a{c.cs, c.cqf, c.cqd, c.Nq, c.m, c.P, c.sf_tile, c.sf_part};
-  cudaError_t e = dispatch(c, sf_kernel<MODE>, sf_kernel_b<MODE>, grid, dim3(c.sf_mb), shm, a);
+  // Of P = 200 modes' seven warps one has 8 of its 32 lanes at work. Where the tiles give every SM
+  // four tiles, a block takes up to four tiles and lays its threads over modes and tiles
+  // (P = 200: 25 full warps for four).
+  int k = 1;
+  if (MODE != 2 && c.P <= 256 && c.sf_nblk_p >= 4 * c.sms) {
+    auto full = [&](int n) { return (double)(c.P * n) / ((c.P * n + 31) / 32); };
+    for (int n = 2; n <= 4; ++n)
+      if (n * shm <= 48 * 1024 && full(n) > 1.01 * full(k)) k = n;
+  }
+  const SfArgs a{c.cs, c.cqf, c.cqd, c.Nq, c.m, c.P, c.sf_tile, k, c.sf_part};
+  const dim3 block((unsigned)(k > 1 ? (k * c.P + 31) / 32 * 32 : c.sf_mb));
+  grid.x = (grid.x + k - 1) / k;
+  cudaError_t e = dispatch(c, sf_kernel<MODE>, sf_kernel_b<MODE>, grid, block, k * shm, a);
   if (e != cudaSuccess) return e;
   const CombineArgs b{c.sf_part, c.sf_nblk_p, c.P, c.kcd, c.alpha, c.rho, c.abf, c.abd, c.emode};
   return dispatch(c, sf_combine_kernel<MODE>, sf_combine_kernel_b<MODE>, dim3(c.P), dim3(128),

@@ -563,8 +563,10 @@ int rbe_init(rbe_handle *hout, const rbe_params *p, int64_t N, const double box[
   c.sf_nblk_m = (c.P + c.sf_mb - 1) / c.sf_mb;
   {
     const int64_t target_blocks = (int64_t)c.sms * 8;
-    int64_t tile = Nq * c.sf_nblk_m / std::max<int64_t>(1, target_blocks);
-    tile = std::max<int64_t>(32, std::min<int64_t>(512, ((tile + 31) / 32) * 32));
+    // (tiles of at most 512, in as many whole waves as that takes)
+    const int64_t want = Nq * c.sf_nblk_m;
+    const int64_t waves = std::max<int64_t>(1, (want + 512 * target_blocks - 1) / (512 * target_blocks));
+    const int64_t tile = std::max<int64_t>(32, ((want / (waves * target_blocks) + 31) / 32) * 32);
     c.sf_tile = (int)tile;
     c.sf_nblk_p = (int)std::max<int64_t>(1, (Nq + tile - 1) / tile);
     c.sf_part_blocks = std::max<int64_t>(1, (Nq + 31) / 32);  // room for the smallest tile
