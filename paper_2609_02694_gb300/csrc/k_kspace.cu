@@ -428,11 +428,13 @@ RBE_BATCHED_KERNEL(__launch_bounds__(256), kspace_add_kernel, KAddArgs, kspace_a
 
 template <int MODE>
 static cudaError_t sf_launch(Ctx &c, dim3 grid, size_t shm) {
-  // Of P = 200 modes' seven warps one has 8 of its 32 lanes at work. Where the tiles give every SM
-  // four tiles, a block takes up to four tiles and lays its threads over modes and tiles
-  // (P = 200: 25 full warps for four).
+  // Of P = 200 modes' seven warps one has 8 of its 32 lanes at work. Where the tiles are long and
+  // give every SM four, a block takes up to four of them and lays its threads over modes and tiles
+  // (P = 200: 25 full warps for four; 1,400,000 charged: a step 1,105 -> 1,086 us). Shorter ones keep
+  // small blocks, which find room beside those of the other graph branch (100,000 charged, Verlet
+  // list: a step 87 us, 114 with blocks of four tiles).
   int k = 1;
-  if (MODE != 2 && c.P <= 256 && c.sf_nblk_p >= 4 * c.sms) {
+  if (MODE != 2 && c.P <= 256 && c.sf_tile >= 256 && c.sf_nblk_p >= 4 * c.sms) {
     auto full = [&](int n) { return (double)(c.P * n) / ((c.P * n + 31) / 32); };
     for (int n = 2; n <= 4; ++n)
       if (n * shm <= 48 * 1024 && full(n) > 1.01 * full(k)) k = n;

@@ -21,6 +21,17 @@ def rel_l2(a, b):
 @pytest.mark.parametrize("N,nq,P", [(500, 3, 1), (500, 5, 2), (2000, 65, 255), (2000, 97, 257),
                                     (30001, 30001, 131)])
 def test_odd_particles_and_modes(orc, precision, tol, N, nq, P):
+    run(orc, precision, tol, N, nq, P, None)
+
+
+@pytest.mark.parametrize("precision,tol", [("fp32_comp", 2e-6), ("fp32", 2e-5)])
+@pytest.mark.parametrize("N,P,tile", [(170001, 200, 256), (160003, 57, 256), (312001, 33, 512)])
+def test_tiles_shared_by_a_block(orc, precision, tol, N, P, tile):
+    """Long tiles in numbers that do not fill the last block's."""
+    run(orc, precision, tol, N, N, P, tile)
+
+
+def run(orc, precision, tol, N, nq, P, tile):
     build.build()
     sy = synth.make_system(N, density=0.02, frac_charged=0.0, seed=31)
     rng = np.random.default_rng(7)
@@ -30,11 +41,15 @@ def test_odd_particles_and_modes(orc, precision, tol, N, nq, P):
     r_core, r_s, p, seed, step = 2.7, 5.0, 4, 3, 2
     with binding.from_system(sy, P=P, alpha=ALPHA, r_c=r_s, r_core=r_core, p_rbl=p, seed=seed,
                              precision=precision) as h:
+        if tile:
+            h.set_tuning("sf_tile", tile)
         F, _, _ = h.forces_f64(step)
         rho, m = h.rho()
         _, S = h.sample_k(step)
+    assert rel_l2(rho, orc.rho(sy.s, sy.q, sy.box, m)) < tol
+    if tile:
+        return
     ref = orc.rbl(sy.s, sy.q, sy.types, sy.box, ALPHA, r_core, r_s, p, seed, step, 0, C, sy.eps,
                   sy.sig)
     Fk, _, _ = orc.rbe_kspace(sy.s, sy.q, sy.box, ALPHA, C, m, S)
-    assert rel_l2(rho, orc.rho(sy.s, sy.q, sy.box, m)) < tol
     assert rel_l2(F, ref["F"] + Fk) < 1e-5
