@@ -414,9 +414,10 @@ __device__ __forceinline__ void bin_identity_body(const PermuteArgs &a, int bx, 
 }
 RBE_BATCHED_KERNEL(__launch_bounds__(256), bin_identity_kernel, PermuteArgs, bin_identity_body)
 
-cudaError_t launch_bin_sort(Ctx &c) {
+// Cell counts and starts, from the current positions (all that the cluster rows need).
+cudaError_t launch_bin_count(Ctx &c) {
   const int64_t N = c.N, nc = c.grid.ncell;
-  const int b0 = c.cur, b1 = 1 - c.cur;
+  const int b0 = c.cur;
   const int32_t *gate = c.vl_on ? c.vl_flags : nullptr;  // list mode: sort only on a build
   cudaError_t e = cudaSuccess;  // (the counts are clear: at first, and after each scan)
   if (N > 0) {
@@ -438,9 +439,16 @@ cudaError_t launch_bin_sort(Ctx &c) {
                dim3(kScanThreads), 0, sa);
   if (e != cudaSuccess) return e;
   // (no blocks for a one-block scan; recorded all the same, so that boxes of any size share a class)
-  e = dispatch(c, scan_add_kernel, scan_add_kernel_b, dim3(nblk > 1 ? (unsigned)nblk : 0u, 2),
-               dim3(kScanThreads), 0, sa);
-  if (e != cudaSuccess) return e;
+  return dispatch(c, scan_add_kernel, scan_add_kernel_b, dim3(nblk > 1 ? (unsigned)nblk : 0u, 2),
+                  dim3(kScanThreads), 0, sa);
+}
+
+// The particles moved to their cells' ranges, in order, in the other buffers (which become current).
+cudaError_t launch_bin_place(Ctx &c) {
+  const int64_t N = c.N, nc = c.grid.ncell;
+  const int b0 = c.cur, b1 = 1 - c.cur;
+  const int32_t *gate = c.vl_on ? c.vl_flags : nullptr;
+  cudaError_t e;
   if (N > 0) {
     const ScatterArgs xa{N, c.key, c.off, c.cell_start, c.tmp, gate};
     if (N % 4 == 0 && !c.rec)

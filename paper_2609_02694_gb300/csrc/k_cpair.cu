@@ -1325,13 +1325,15 @@ bool cpair_usable(const Ctx &c) {
   return c.box[0] - 2.0 * c.rc > 2.0 * c.box[0] / c.grid.n[0];
 }
 
-cudaError_t launch_cluster_tables(Ctx &c) {
+cudaError_t launch_cluster_rows(Ctx &c) {
+  const RowsArgs ra{c.cell_start, c.grid.n[0], c.grid.n[1] * c.grid.n[2], cpair_nc(c), c.cl_base,
+                    c.sc_base};
+  return dispatch(c, cluster_rows_kernel, cluster_rows_kernel_b, dim3(1), dim3(1024), 0, ra);
+}
+
+cudaError_t launch_cluster_bounds(Ctx &c) {
   const int b = c.cur;
   const int nrows = c.grid.n[1] * c.grid.n[2];
-  const RowsArgs ra{c.cell_start, c.grid.n[0], nrows, cpair_nc(c), c.cl_base, c.sc_base};
-  cudaError_t e = dispatch(c, cluster_rows_kernel, cluster_rows_kernel_b, dim3(1), dim3(1024), 0,
-                           ra);
-  if (e != cudaSuccess) return e;
   const int64_t ccap = cpair_clusters_bound(c);
   const BoundsArgs ba{c.s[b], c.s[b] + c.N, c.s[b] + 2 * c.N, c.qf[b], c.cell_start, c.grid.n[0],
                       nrows, c.cl_base, ccap, c.cl_lo, c.cl_hi, c.cjrec, c.pc.h[1], c.pc.h[2],
@@ -1340,7 +1342,7 @@ cudaError_t launch_cluster_tables(Ctx &c) {
                   dim3((unsigned)((kClSize * ccap + 255) / 256)), dim3(256), 0, ba);
 }
 
-// The pair pass itself (the tables of launch_cluster_tables must be current); its forces stay
+// The pair pass itself (the tables of the two passes above must be current); its forces stay
 // in the fixed-point sums, which the Coulomb pass and the k-space gather add to before
 // launch_cluster_finish converts them.
 cudaError_t launch_cluster_pair(Ctx &c, bool coul, bool multi, bool want_counts) {

@@ -584,26 +584,30 @@ int64_t partials_compact_count(int64_t nblk) {
   return nblk <= kTotalsDirect ? 0 : std::min<int64_t>((nblk + 255) / 256, kCompactMax);
 }
 
-cudaError_t launch_totals(Ctx &c) {
-  TotalsArgs a;
-  // pair and Coulomb-pass partials, compacted first where there are many, by one launch for both
+// Pair and Coulomb-pass partials, compacted where there are many, by one launch for both (recorded
+// without blocks too, so that boxes of any size share a batch's class).
+cudaError_t launch_totals_compact(Ctx &c) {
   const int64_t n[2] = {c.n_pair_blk, c.n_coul_blk};
   const double *part[2] = {c.epart + c.off_pair, c.epart + c.off_coul};
   const int64_t nc[2] = {partials_compact_count(n[0]), partials_compact_count(n[1])};
-  cudaError_t e;
-  {  // (recorded without blocks too, so that boxes of any size share a batch's class)
-    CompactArgs ca{};
-    for (int w = 0; w < 2; ++w) {
-      ca.in[w] = part[w];
-      ca.nblk[w] = n[w];
-      ca.per[w] = nc[w] ? (n[w] + nc[w] - 1) / nc[w] : 0;
-      ca.out[w] = c.ecomp + w * kCompactMax * NQ_PAIR;
-    }
-    ca.nc0 = (int)nc[0];
-    e = dispatch(c, partials_compact_kernel, partials_compact_kernel_b,
-                 dim3((unsigned)(nc[0] + nc[1])), dim3(256), 0, ca);
-    if (e != cudaSuccess) return e;
+  CompactArgs ca{};
+  for (int w = 0; w < 2; ++w) {
+    ca.in[w] = part[w];
+    ca.nblk[w] = n[w];
+    ca.per[w] = nc[w] ? (n[w] + nc[w] - 1) / nc[w] : 0;
+    ca.out[w] = c.ecomp + w * kCompactMax * NQ_PAIR;
   }
+  ca.nc0 = (int)nc[0];
+  return dispatch(c, partials_compact_kernel, partials_compact_kernel_b,
+                  dim3((unsigned)(nc[0] + nc[1])), dim3(256), 0, ca);
+}
+
+// The totals; the pair passes' partials must be compacted.
+cudaError_t launch_totals(Ctx &c) {
+  TotalsArgs a;
+  const int64_t n[2] = {c.n_pair_blk, c.n_coul_blk};
+  const double *part[2] = {c.epart + c.off_pair, c.epart + c.off_coul};
+  const int64_t nc[2] = {partials_compact_count(n[0]), partials_compact_count(n[1])};
   a.pair = nc[0] ? c.ecomp : part[0]; a.n_pair = nc[0] ? nc[0] : n[0];
   a.coul = nc[1] ? c.ecomp + kCompactMax * NQ_PAIR : part[1]; a.n_coul = nc[1] ? nc[1] : n[1];
   // RBL partials: the compacted ones (rbl_compact_kernel runs after the RBL kernel)

@@ -184,9 +184,8 @@ int free_all(Ctx &c) {
   if (c.aux_stream) cudaStreamDestroy(c.aux_stream);
   c.aux_stream = nullptr;
   if (c.ev_fork) cudaEventDestroy(c.ev_fork);
-  if (c.ev_bin) cudaEventDestroy(c.ev_bin);
   if (c.ev_join) cudaEventDestroy(c.ev_join);
-  c.ev_fork = c.ev_bin = c.ev_join = nullptr;
+  c.ev_fork = c.ev_join = nullptr;
   if (c.scal_host) cudaFreeHost(c.scal_host);
   c.scal_host = nullptr;
   return RBE_OK;
@@ -208,68 +207,113 @@ int finish_forces(Ctx &c, bool cp) {
   else RBE_CUDA_TRY(launch_kspace_add(c));
   return RBE_OK;
 }
+// (cluster kernel: the rows' offsets are current already)
 int lists(Ctx &c, bool cp) {
   if (c.vl_on) {
     RBE_CUDA_TRY(launch_list_build(c));
     RBE_CUDA_TRY(launch_list_commit(c));
   } else if (cp) {
-    RBE_CUDA_TRY(launch_cluster_tables(c));  // the cluster-pair kernel's per-step tables
+    RBE_CUDA_TRY(launch_cluster_bounds(c));
   }
   return RBE_OK;
 }
 
-// The pipeline in two branches of a captured graph: the sampler, which needs only the step
-// number, beside the binning; then the k-space chain (structure factor, gather) and, with the
-// cluster kernel, the charged subset's Coulomb pass beside the real-space pass; then the pass that
-// forms F. Each branch writes its own arrays (or adds integers to the fixed-point sums), so the
-// forces are those of the sequential order bit for bit. The real-space passes issue in 60 to 75%
-// of their slots; the other branch's kernels fill slots and SMs they leave idle
-// (measured, a step: cluster kernel on 2^20 particles 1.445 -> 1.360 ms; random batch list on
-// 200,000 / 1,400,000 ions 258 -> 225 / 1,226 -> 1,135 us; Verlet list on 100,000 ions 123 -> 100).
-int force_pipeline_forked(Ctx &c, bool cp, bool debug) {
+// Capture on the graph's second branch: what `to` launches next waits for `from`'s last node.
+int join(Ctx &c, cudaStream_t from, cudaStream_t to) {
+  RBE_CUDA_TRY(cudaEventRecord(c.ev_fork, from));
+  RBE_CUDA_TRY(cudaStreamWaitEvent(to, c.ev_fork, 0));
+  return RBE_OK;
+}
+template <class F> int on_branch(Ctx &c, F launches) {
   const cudaStream_t main_stream = c.stream;
-  RBE_CUDA_TRY(cudaEventRecord(c.ev_fork, main_stream));
-  RBE_CUDA_TRY(cudaStreamWaitEvent(c.aux_stream, c.ev_fork, 0));
   c.stream = c.aux_stream;
-  cudaError_t e = launch_sample_k(c);
+  const cudaError_t e = launches();
   c.stream = main_stream;
   RBE_CUDA_TRY(e);
-  if (c.vl_on) RBE_CUDA_TRY(launch_list_check(c));
-  RBE_CUDA_TRY(launch_bin_sort(c));
-  RBE_CUDA_TRY(cudaEventRecord(c.ev_bin, main_stream));
-  RBE_CUDA_TRY(cudaStreamWaitEvent(c.aux_stream, c.ev_bin, 0));
-  c.stream = c.aux_stream;
-  e = launch_structure_factor(c);
-  if (e == cudaSuccess) e = launch_kspace_gather(c, cp);
-  // (mostly charged: the pair pass takes the Coulomb pairs itself)
-  if (e == cudaSuccess && cp && c.Nq * 2 <= c.N) e = launch_coulomb_subset(c, c.cq4, true);
-  if (e == cudaSuccess) e = cudaEventRecord(c.ev_join, c.aux_stream);
-  c.stream = main_stream;
-  RBE_CUDA_TRY(e);
-  int rc = lists(c, cp);
-  if (rc == RBE_OK) rc = real_space(c, cp, false, debug);
+  return RBE_OK;
+}
+
+// The second branch's stream and events.
+int make_branch(Ctx &c) {
+  if (!c.aux_stream) RBE_CUDA_TRY(cudaStreamCreateWithFlags(&c.aux_stream, cudaStreamNonBlocking));
+  if (!c.ev_fork) RBE_CUDA_TRY(cudaEventCreateWithFlags(&c.ev_fork, cudaEventDisableTiming));
+  if (!c.ev_join) RBE_CUDA_TRY(cudaEventCreateWithFlags(&c.ev_join, cudaEventDisableTiming));
+  return RBE_OK;
+}
+
+// What a captured step or evaluation does after the drift, in two branches of the graph. Beside the
+// binning runs the sampler, which needs only the step number, and once the cells are counted the
+// cluster rows; beside the real-space pass the k-space chain (structure factor, gather), with the
+// cluster kernel the charged subset's Coulomb pass, and an evaluation's kinetic energy; beside the
+// pass that forms F the sums over the real-space pass's partials (an evaluation's totals too). Each
+// branch writes its own arrays (or adds integers to the fixed-point sums), so the results are those
+// of the sequential order bit for bit. The real-space passes issue in 60 to 75% of their slots; the
+// other branch's kernels fill slots and SMs they leave idle, and in a small box take launches off
+// the longer branch (measured, a step: cluster kernel on 2^20 particles 1.445 -> 1.360 ms; random
+// batch list on 200,000 / 1,400,000 ions 258 -> 225 / 1,226 -> 1,135 us; Verlet list on 100,000 ions
+// 123 -> 100; rows, sums and kinetic energy moved over: 3,000 charged particles 78 -> 74, an evaluation 79 -> 73).
+int pipeline_forked(Ctx &c, bool forces_only) {
+  const bool cp = !c.rbl && !c.vl_on && cpair_usable(c);
+  const cudaStream_t main_stream = c.stream, aux = c.aux_stream;
+  int rc = join(c, main_stream, aux);
+  if (rc == RBE_OK) rc = on_branch(c, [&] { return launch_sample_k(c); });
   if (rc != RBE_OK) return rc;
-  RBE_CUDA_TRY(cudaStreamWaitEvent(c.stream, c.ev_join, 0));
-  return finish_forces(c, cp);
+  if (c.vl_on) RBE_CUDA_TRY(launch_list_check(c));
+  RBE_CUDA_TRY(launch_bin_count(c));
+  if (cp) {
+    rc = join(c, main_stream, aux);
+    if (rc == RBE_OK) rc = on_branch(c, [&] { return launch_cluster_rows(c); });
+    if (rc != RBE_OK) return rc;
+  }
+  RBE_CUDA_TRY(launch_bin_place(c));
+  if (cp) rc = join(c, aux, main_stream);
+  if (rc == RBE_OK) rc = join(c, main_stream, aux);
+  if (rc == RBE_OK)
+    rc = on_branch(c, [&] {
+      cudaError_t e = launch_structure_factor(c);
+      if (e == cudaSuccess) e = launch_kspace_gather(c, cp);
+      // (mostly charged: the pair pass takes the Coulomb pairs itself)
+      if (e == cudaSuccess && cp && c.Nq * 2 <= c.N) e = launch_coulomb_subset(c, c.cq4, true);
+      if (e == cudaSuccess && forces_only) e = launch_kinetic(c);
+      return e == cudaSuccess ? cudaEventRecord(c.ev_join, aux) : e;
+    });
+  if (rc == RBE_OK) rc = lists(c, cp);
+  if (rc == RBE_OK) rc = real_space(c, cp, false, false);
+  if (rc == RBE_OK) rc = join(c, main_stream, aux);
+  const bool totals_aside = forces_only && !c.rbl;  // (the random batch list's need its last pass)
+  if (rc == RBE_OK)
+    rc = on_branch(c, [&] {
+      cudaError_t e = launch_totals_compact(c);
+      return e == cudaSuccess && totals_aside ? launch_totals(c) : e;
+    });
+  if (rc != RBE_OK) return rc;
+  RBE_CUDA_TRY(cudaStreamWaitEvent(main_stream, c.ev_join, 0));
+  rc = finish_forces(c, cp);
+  if (rc != RBE_OK) return rc;
+  if (!forces_only) {
+    RBE_CUDA_TRY(launch_kick(c));
+    if (c.nvt) RBE_CUDA_TRY(launch_thermostat(c, 0));
+  }
+  rc = join(c, aux, main_stream);
+  if (rc != RBE_OK) return rc;
+  if (!totals_aside) RBE_CUDA_TRY(launch_totals(c));
+  return RBE_OK;
 }
 
 // [list check] -> bin + sort -> sample -> structure factor -> [list build] -> real space
 // -> k-space gather -> the pass that forms F
 int force_pipeline(Ctx &c, bool debug) {
   const bool cp = !c.rbl && !c.vl_on && cpair_usable(c);
-  if (c.Nq > 0 && !c.rec && !c.timing && c.aux_stream) {
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    RBE_CUDA_TRY(cudaStreamIsCapturing(c.stream, &st));
-    if (st == cudaStreamCaptureStatusActive) return force_pipeline_forked(c, cp, debug);
-  }
   mark(c, RBE_PH_BIN);
   if (c.vl_on) RBE_CUDA_TRY(launch_list_check(c));
-  RBE_CUDA_TRY(launch_bin_sort(c));
+  RBE_CUDA_TRY(launch_bin_count(c));
+  RBE_CUDA_TRY(launch_bin_place(c));
   mark(c, RBE_PH_SAMPLE);
   RBE_CUDA_TRY(launch_sample_k(c));
   mark(c, RBE_PH_SF);
   RBE_CUDA_TRY(launch_structure_factor(c));
   mark(c, RBE_PH_LIST);
+  if (cp) RBE_CUDA_TRY(launch_cluster_rows(c));
   int rc = lists(c, cp);
   if (rc != RBE_OK) return rc;
   mark(c, RBE_PH_PAIR);
@@ -345,10 +389,7 @@ int copy_scalars(Ctx &c, double *energies, double *virial) {
 // c.stream.
 int capture_step_graph(Ctx &c, int parity, cudaGraphExec_t *out, bool forces_only = false) {
   if (!c.cap_stream) RBE_CUDA_TRY(cudaStreamCreateWithFlags(&c.cap_stream, cudaStreamNonBlocking));
-  if (!c.aux_stream) RBE_CUDA_TRY(cudaStreamCreateWithFlags(&c.aux_stream, cudaStreamNonBlocking));
-  if (!c.ev_fork) RBE_CUDA_TRY(cudaEventCreateWithFlags(&c.ev_fork, cudaEventDisableTiming));
-  if (!c.ev_bin) RBE_CUDA_TRY(cudaEventCreateWithFlags(&c.ev_bin, cudaEventDisableTiming));
-  if (!c.ev_join) RBE_CUDA_TRY(cudaEventCreateWithFlags(&c.ev_join, cudaEventDisableTiming));
+  if (int rc = make_branch(c); rc != RBE_OK) return rc;
   const int saved = c.cur;
   cudaStream_t user = c.stream;
   c.cur = parity;
@@ -362,21 +403,22 @@ int capture_step_graph(Ctx &c, int parity, cudaGraphExec_t *out, bool forces_onl
   }
   int rc = RBE_OK;
   do {
-    if (forces_only) {  // (the step number is set on the device before each launch)
-      rc = force_pipeline(c, false);
-      if (rc != RBE_OK) break;
-      if (launch_kinetic(c) != cudaSuccess) { rc = RBE_ERR_CUDA; break; }
-      if (launch_totals(c) != cudaSuccess) { rc = RBE_ERR_CUDA; break; }
+    // (an evaluation's step number is set on the device before each launch)
+    if (!forces_only) {
+      mark(c, RBE_PH_KICK_DRIFT);
+      if (launch_kick_drift(c) != cudaSuccess) { rc = RBE_ERR_CUDA; break; }  // + step counter
+    }
+    if (c.Nq > 0 && !c.timing) {  // (per-phase times are taken of one branch)
+      rc = pipeline_forked(c, forces_only);
       break;
     }
-    mark(c, RBE_PH_KICK_DRIFT);
-    if (launch_kick_drift(c) != cudaSuccess) { rc = RBE_ERR_CUDA; break; }  // + step counter
     rc = force_pipeline(c, false);
     if (rc != RBE_OK) break;
-    if (launch_kick(c) != cudaSuccess) { rc = RBE_ERR_CUDA; break; }
-    if (c.nvt && launch_thermostat(c, 0) != cudaSuccess) { rc = RBE_ERR_CUDA; break; }
+    if ((forces_only ? launch_kinetic(c) : launch_kick(c)) != cudaSuccess) { rc = RBE_ERR_CUDA; break; }
+    if (!forces_only && c.nvt && launch_thermostat(c, 0) != cudaSuccess) { rc = RBE_ERR_CUDA; break; }
+    if (launch_totals_compact(c) != cudaSuccess) { rc = RBE_ERR_CUDA; break; }
     if (launch_totals(c) != cudaSuccess) { rc = RBE_ERR_CUDA; break; }
-    mark(c, RBE_N_PHASE);
+    if (!forces_only) mark(c, RBE_N_PHASE);
   } while (0);
   cudaError_t e = cudaStreamEndCapture(c.stream, &g);
   c.cur = saved;
@@ -779,6 +821,7 @@ static int forces_common(rbe_handle h, uint64_t step, bool debug) {
   int rc = force_pipeline(c, debug);
   if (rc != RBE_OK) return rc;
   RBE_CUDA_TRY(launch_kinetic(c));
+  RBE_CUDA_TRY(launch_totals_compact(c));
   RBE_CUDA_TRY(launch_totals(c));
   mark(c, RBE_N_PHASE);
   c.have_forces = (step == c.step);
@@ -1347,13 +1390,16 @@ static int batch_free(rbe_batch b) {
   return RBE_OK;
 }
 
-// One Verlet step of replica c on c.stream (the sequence rbe_step captures).
+// One Verlet step of replica c on c.stream (the sequence rbe_step captures, in two branches where
+// it is captured and not recorded).
 static int step_sequence(Ctx &c) {
   if (launch_kick_drift(c) != cudaSuccess) return RBE_ERR_CUDA;  // + step counter
+  if (!c.rec && c.aux_stream && c.Nq > 0 && !c.timing) return pipeline_forked(c, false);
   int rc = force_pipeline(c, false);
   if (rc != RBE_OK) return rc;
   if (launch_kick(c) != cudaSuccess) return RBE_ERR_CUDA;
   if (c.nvt && launch_thermostat(c, 0) != cudaSuccess) return RBE_ERR_CUDA;
+  if (launch_totals_compact(c) != cudaSuccess) return RBE_ERR_CUDA;
   if (launch_totals(c) != cudaSuccess) return RBE_ERR_CUDA;
   return RBE_OK;
 }
@@ -1558,6 +1604,9 @@ static int batch_capture(rbe_batch b, int k, int flip) {
     saved_cur[r] = b->h[r]->cur;
     saved_stream[r] = b->h[r]->stream;
   }
+  for (int r : b->solo)
+    if (rc == RBE_OK) rc = make_branch(*b->h[r]);
+  if (rc != RBE_OK) return rc;
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal);
   if (e == cudaSuccess) {

@@ -203,9 +203,9 @@ struct Ctx {
   cudaGraphExec_t graph[2] = {nullptr, nullptr};  // one per starting buffer parity
   cudaGraphExec_t fgraph[2] = {nullptr, nullptr}; // force evaluations (rbe_forces), the same
   cudaStream_t cap_stream = nullptr;  // internal non-blocking stream used only for capture
-  cudaStream_t aux_stream = nullptr;  // second capture stream: the k-space branch of a step
-  cudaEvent_t ev_fork = nullptr, ev_bin = nullptr, ev_join = nullptr;  // (its fork, its wait for
-                                                                      // the binning, its join)
+  cudaStream_t aux_stream = nullptr;  // second capture stream: a step's other branch
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;  // edges between the branches; the end of the
+                                                     // k-space chain
   // profiling: ev[k] is recorded before phase k, ev[RBE_N_PHASE] after the last one
   bool timing = false;
   cudaEvent_t ev[RBE_N_PHASE + 1] = {};
@@ -444,7 +444,8 @@ cudaError_t fill_zero(Ctx &c, void *p, int64_t words);
 // Launchers (each in its own translation unit). All return cudaGetLastError().
 
 cudaError_t launch_sample_k(Ctx &c);
-cudaError_t launch_bin_sort(Ctx &c);
+cudaError_t launch_bin_count(Ctx &c);
+cudaError_t launch_bin_place(Ctx &c);
 cudaError_t launch_structure_factor(Ctx &c);
 cudaError_t launch_kspace_gather(Ctx &c, bool into_facc);  // to fk, or into the fixed-point sums
 cudaError_t launch_kspace_add(Ctx &c);                     // F += fk
@@ -454,7 +455,8 @@ cudaError_t launch_pair(Ctx &c, bool want_counts);   // per-particle pass, then 
 bool cpair_usable(const Ctx &c);
 int64_t cpair_blocks_bound(const Ctx &c);
 int64_t cpair_clusters_bound(const Ctx &c);
-cudaError_t launch_cluster_tables(Ctx &c);  // per-row offsets and per-cluster bounds
+cudaError_t launch_cluster_rows(Ctx &c);    // per-row offsets (after the cell starts)
+cudaError_t launch_cluster_bounds(Ctx &c);  // per-cluster bounds and records
 cudaError_t launch_cluster_pair(Ctx &c, bool coul, bool multi, bool want_counts);
 cudaError_t launch_cluster_finish(Ctx &c);
 cudaError_t launch_pair_cluster(Ctx &c, bool want_counts);
@@ -473,6 +475,7 @@ cudaError_t launch_kick_drift(Ctx &c);  // also advances the device step counter
 cudaError_t launch_kick(Ctx &c);
 cudaError_t launch_kinetic(Ctx &c);
 cudaError_t launch_thermostat(Ctx &c, int mode);  // 0: end + next start half, 1: start half only
+cudaError_t launch_totals_compact(Ctx &c);  // the pair passes' partials, where there are many
 cudaError_t launch_totals(Ctx &c);
 int64_t partials_compact_count(int64_t nblk);
 // The totals sum every slot of a pass's partial range: a pass whose grid writes fewer slots
