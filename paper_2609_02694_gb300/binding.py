@@ -248,9 +248,9 @@ class RBE:
         return s.value
 
     def state(self):
-        pos = np.zeros((self.N, 3), np.float64)
-        vel = np.zeros((self.N, 3), np.float64)
-        s = np.zeros((self.N, 3), np.uint32)
+        pos = np.empty((self.N, 3), np.float64)
+        vel = np.empty((self.N, 3), np.float64)
+        s = np.empty((self.N, 3), np.uint32)
         _check(lib().rbe_get_state(self._h, pos.ctypes.data, vel.ctypes.data, s.ctypes.data),
                "rbe_get_state")
         return pos, vel, s

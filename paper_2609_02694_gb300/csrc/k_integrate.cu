@@ -377,10 +377,14 @@ __global__ void __launch_bounds__(kTotalsThreads)
   totals_body<ACC>(t[q.r], q.bx, q.nbx);
 }
 
+// Results in particle order, in device or pinned host memory; err_out (nullable): the error flags,
+// for the host that waits for the results.
 template <typename FT, typename OT>
 __global__ void scatter_forces_kernel(const FT *__restrict__ F, const int32_t *__restrict__ id,
-                                      int64_t N, OT *__restrict__ out) {
+                                      int64_t N, OT *__restrict__ out, const int *err,
+                                      int *err_out) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k == 0 && err_out) *err_out = *err;
   if (k >= N) return;
   const int64_t o = (int64_t)id[k] * 3;
   out[o] = (OT)F[k];
@@ -390,24 +394,28 @@ __global__ void scatter_forces_kernel(const FT *__restrict__ F, const int32_t *_
 
 template <typename V>
 __global__ void scatter_state_kernel(const uint32_t *__restrict__ s, const V *__restrict__ v,
-                                     const int32_t *__restrict__ id, int64_t N, int what,
-                                     double hx, double hy, double hz, double *__restrict__ outd,
-                                     uint32_t *__restrict__ outu) {
+                                     const int32_t *__restrict__ id, int64_t N, double hx,
+                                     double hy, double hz, double *pos, double *vel, uint32_t *frac,
+                                     const int *err, int *err_out) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k == 0 && err_out) *err_out = *err;
   if (k >= N) return;
   const int64_t o = (int64_t)id[k] * 3;
-  if (what == 0) {
-    outd[o] = (double)s[k] * hx;
-    outd[o + 1] = (double)s[N + k] * hy;
-    outd[o + 2] = (double)s[2 * N + k] * hz;
-  } else if (what == 1) {
-    outd[o] = (double)v[k];
-    outd[o + 1] = (double)v[N + k];
-    outd[o + 2] = (double)v[2 * N + k];
-  } else {
-    outu[o] = s[k];
-    outu[o + 1] = s[N + k];
-    outu[o + 2] = s[2 * N + k];
+  const uint32_t x = s[k], y = s[N + k], z = s[2 * N + k];
+  if (pos) {
+    pos[o] = (double)x * hx;
+    pos[o + 1] = (double)y * hy;
+    pos[o + 2] = (double)z * hz;
+  }
+  if (vel) {
+    vel[o] = (double)v[k];
+    vel[o + 1] = (double)v[N + k];
+    vel[o + 2] = (double)v[2 * N + k];
+  }
+  if (frac) {
+    frac[o] = x;
+    frac[o + 1] = y;
+    frac[o + 2] = z;
   }
 }
 
@@ -625,29 +633,31 @@ cudaError_t launch_totals(Ctx &c) {
                   dim3(kTotalsThreads), 0, a);
 }
 
-cudaError_t launch_scatter_forces(Ctx &c, bool to_double, float *outf) {
+cudaError_t launch_scatter_forces(Ctx &c, bool to_double, float *outf, int *err_out) {
   const int b = c.cur;
   if (c.N == 0) return cudaSuccess;
   if (!outf) outf = c.outf;
+  const unsigned g = nblk(c.N, 256);
+  const int32_t *id = c.id[b];
   if (c.precision == RBE_FP64) {
-    if (to_double) scatter_forces_kernel<double, double><<<nblk(c.N, 256), 256, 0, c.stream>>>(c.Fd, c.id[b], c.N, c.outd);
-    else scatter_forces_kernel<double, float><<<nblk(c.N, 256), 256, 0, c.stream>>>(c.Fd, c.id[b], c.N, outf);
+    if (to_double) scatter_forces_kernel<double, double><<<g, 256, 0, c.stream>>>(c.Fd, id, c.N, c.outd, c.err, err_out);
+    else scatter_forces_kernel<double, float><<<g, 256, 0, c.stream>>>(c.Fd, id, c.N, outf, c.err, err_out);
   } else {
-    if (to_double) scatter_forces_kernel<float, double><<<nblk(c.N, 256), 256, 0, c.stream>>>(c.F, c.id[b], c.N, c.outd);
-    else scatter_forces_kernel<float, float><<<nblk(c.N, 256), 256, 0, c.stream>>>(c.F, c.id[b], c.N, outf);
+    if (to_double) scatter_forces_kernel<float, double><<<g, 256, 0, c.stream>>>(c.F, id, c.N, c.outd, c.err, err_out);
+    else scatter_forces_kernel<float, float><<<g, 256, 0, c.stream>>>(c.F, id, c.N, outf, c.err, err_out);
   }
   return cudaGetLastError();
 }
 
-cudaError_t launch_scatter_state(Ctx &c, int what) {
+cudaError_t launch_scatter_state(Ctx &c, double *pos, double *vel, uint32_t *frac, int *err_out) {
   const int b = c.cur;
   if (c.N == 0) return cudaSuccess;
   const double hx = c.box[0] / kTwo32, hy = c.box[1] / kTwo32, hz = c.box[2] / kTwo32;
-  uint32_t *outu = reinterpret_cast<uint32_t *>(c.outf);
+  const unsigned g = nblk(c.N, 256);
   if (c.precision == RBE_FP64)
-    scatter_state_kernel<double><<<nblk(c.N, 256), 256, 0, c.stream>>>(c.s[b], c.vd[b], c.id[b], c.N, what, hx, hy, hz, c.outd, outu);
+    scatter_state_kernel<double><<<g, 256, 0, c.stream>>>(c.s[b], c.vd[b], c.id[b], c.N, hx, hy, hz, pos, vel, frac, c.err, err_out);
   else
-    scatter_state_kernel<float><<<nblk(c.N, 256), 256, 0, c.stream>>>(c.s[b], c.vf[b], c.id[b], c.N, what, hx, hy, hz, c.outd, outu);
+    scatter_state_kernel<float><<<g, 256, 0, c.stream>>>(c.s[b], c.vf[b], c.id[b], c.N, hx, hy, hz, pos, vel, frac, c.err, err_out);
   return cudaGetLastError();
 }
 
@@ -669,7 +679,7 @@ static unsigned long long inverse_bits(double L, int *sh) {
   return q;
 }
 
-cudaError_t launch_set_positions(Ctx &c) {
+cudaError_t launch_set_positions(Ctx &c, const double *pos) {
   const int b = c.cur;
   if (c.N == 0) return cudaSuccess;
   PosScale p;
@@ -677,7 +687,7 @@ cudaError_t launch_set_positions(Ctx &c) {
     p.L[d] = c.box[d];
     p.K[d] = inverse_bits(c.box[d], &p.sh[d]);
   }
-  set_positions_kernel<<<nblk(c.N, 256), 256, 0, c.stream>>>(c.pos_stage, c.id[b], c.N, p, c.s[b]);
+  set_positions_kernel<<<nblk(c.N, 256), 256, 0, c.stream>>>(pos, c.id[b], c.N, p, c.s[b]);
   return cudaGetLastError();
 }
 

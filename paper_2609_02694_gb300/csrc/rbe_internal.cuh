@@ -162,7 +162,8 @@ struct Ctx {
   int64_t off_pair = 0, off_coul = 0, off_rbl = 0, off_ke = 0, n_pair_blk = 0,
           n_coul_blk = 0, n_rbl_blk = 0, n_ke_blk = 0;
   double *scal = nullptr;    // device scalars (see integrate kernels)
-  double *scal_host = nullptr;  // pinned
+  double *scal_host = nullptr;  // pinned: the scalars, and behind them
+  int *flags_host = nullptr;    // the error flags
   uint64_t *step_dev = nullptr;
   uint64_t step = 0;
   int *err = nullptr;
@@ -487,9 +488,12 @@ double frame_band(const double X[3], double r, const double box[3], bool wrap);
 cudaError_t launch_set_step(Ctx &c, uint64_t step);
 cudaError_t launch_step_advance(Ctx &c);
 // Forces in id order, to outf (device; null: c.outf) or c.outd.
-cudaError_t launch_scatter_forces(Ctx &c, bool to_double, float *outf = nullptr);
-cudaError_t launch_scatter_state(Ctx &c, int what);  // 0: positions, 1: velocities, 2: s
-cudaError_t launch_set_positions(Ctx &c);
+// (outf, nullable: where to, of memory this device writes; else the device staging array)
+cudaError_t launch_scatter_forces(Ctx &c, bool to_double, float *outf = nullptr,
+                                  int *err_out = nullptr);
+// (each destination nullable)
+cudaError_t launch_scatter_state(Ctx &c, double *pos, double *vel, uint32_t *frac, int *err_out);
+cudaError_t launch_set_positions(Ctx &c, const double *pos);  // (memory this device reads)
 // Checkpoint load: positions (uint32) and velocities (double), id order, into the sorted slots.
 cudaError_t launch_gather_state(Ctx &c, const uint32_t *s_id, const double *v_id);
 cudaError_t launch_scatter_int(Ctx &c, const int32_t *src_sorted, int32_t *dst_id, int width);
