@@ -511,12 +511,9 @@ __global__ void __launch_bounds__(kRblWarps * 32, 16) rbl64_kernel(const RblArgs
       if (a.nshell) a.nshell[i] = nsh;
     }
   }
-  double v[NQ_PAIR + 3] = {en[0], en[1], en[2], en[3], (double)fx, (double)fy, (double)fz};
-#pragma unroll
-  for (int k = 0; k < NQ_PAIR + 3; ++k) {
-    const double s = warp_sum(v[k]);
-    if (lane == 0) wred[wid][k] = s;
-  }
+  const double v[8] = {en[0], en[1], en[2], en[3], (double)fx, (double)fy, (double)fz, 0.0};
+  const double vs = warp_sum8(v, lane);
+  if (lane < NQ_PAIR + 3) wred[wid][lane] = vs;
   __syncthreads();
   if (threadIdx.x < NQ_PAIR + 3) {
     double s = 0.0;

@@ -281,24 +281,26 @@ int pipeline_forked(Ctx &c, bool forces_only) {
   if (rc == RBE_OK) rc = lists(c, cp);
   if (rc == RBE_OK) rc = real_space(c, cp, false, false);
   if (rc == RBE_OK) rc = join(c, main_stream, aux);
-  const bool totals_aside = forces_only && !c.rbl;  // (the random batch list's need its last pass)
+  const int parts = forces_only ? 3 : 1;  // (a step's kinetic energy comes last, on this branch)
   if (rc == RBE_OK)
     rc = on_branch(c, [&] {
       cudaError_t e = launch_totals_compact(c);
-      return e == cudaSuccess && totals_aside ? launch_totals(c) : e;
+      // (the random batch list's totals need its last pass)
+      return e == cudaSuccess && !c.rbl ? launch_totals(c, parts) : e;
     });
   if (rc != RBE_OK) return rc;
   RBE_CUDA_TRY(cudaStreamWaitEvent(main_stream, c.ev_join, 0));
   rc = finish_forces(c, cp);
+  if (rc == RBE_OK && c.rbl) {
+    rc = join(c, main_stream, aux);
+    if (rc == RBE_OK) rc = on_branch(c, [&] { return launch_totals(c, parts); });
+  }
   if (rc != RBE_OK) return rc;
   if (!forces_only) {
     RBE_CUDA_TRY(launch_kick(c));
-    if (c.nvt) RBE_CUDA_TRY(launch_thermostat(c, 0));
+    RBE_CUDA_TRY(c.nvt ? launch_thermostat(c, 0) : launch_totals(c, 2));
   }
-  rc = join(c, aux, main_stream);
-  if (rc != RBE_OK) return rc;
-  if (!totals_aside) RBE_CUDA_TRY(launch_totals(c));
-  return RBE_OK;
+  return join(c, aux, main_stream);
 }
 
 // [list check] -> bin + sort -> sample -> structure factor -> [list build] -> real space
@@ -345,6 +347,7 @@ int64_t kernels_per_step(const Ctx &c) {
   k += 2;                                // kick (+kinetic), totals
   k += partials_compact_count(c.n_pair_blk) + partials_compact_count(c.n_coul_blk) > 0 ? 1 : 0;
   if (c.nvt) k += 2;                     // thermostat, end-of-step velocity scaling
+  else if (c.Nq > 0 && !c.timing) k += 1;  // the kinetic energy apart from the other totals
   return k;
 }
 

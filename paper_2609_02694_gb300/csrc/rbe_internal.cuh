@@ -323,22 +323,36 @@ __device__ __forceinline__ double warp_sum2(double u, double w, int lane) {
   for (int o = 2; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   return s;
 }
+// Four sums over the warp; lane k < 4 (and every lane with the same low two bits) ends with sum k,
+// in 6 additions instead of 20.
+__device__ __forceinline__ double warp_sum4(const double (&v)[4], int lane) {
+  double w[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const double keep = lane & 1 ? v[2 * k + 1] : v[2 * k], send = lane & 1 ? v[2 * k] : v[2 * k + 1];
+    w[k] = keep + __shfl_xor_sync(0xffffffffu, send, 1);
+  }
+  double s = (lane & 2 ? w[1] : w[0]) + __shfl_xor_sync(0xffffffffu, lane & 2 ? w[0] : w[1], 2);
+#pragma unroll
+  for (int o = 4; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
 // Eight sums over the warp; lane k < 8 (and every lane with the same low three bits) ends with
 // sum k. Each exchange halves the list a lane still carries: 9 additions, where eight separate
 // reductions take 40 (FP64 runs at 1/64 of the FP32 rate).
-__device__ __forceinline__ double warp_sum8(const double (&v)[8], int lane) {
-  double w[4], u[2];
+template <typename T> __device__ __forceinline__ T warp_sum8(const T (&v)[8], int lane) {
+  T w[4], u[2];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    const double keep = lane & 1 ? v[2 * k + 1] : v[2 * k], send = lane & 1 ? v[2 * k] : v[2 * k + 1];
+    const T keep = lane & 1 ? v[2 * k + 1] : v[2 * k], send = lane & 1 ? v[2 * k] : v[2 * k + 1];
     w[k] = keep + __shfl_xor_sync(0xffffffffu, send, 1);
   }
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
-    const double keep = lane & 2 ? w[2 * k + 1] : w[2 * k], send = lane & 2 ? w[2 * k] : w[2 * k + 1];
+    const T keep = lane & 2 ? w[2 * k + 1] : w[2 * k], send = lane & 2 ? w[2 * k] : w[2 * k + 1];
     u[k] = keep + __shfl_xor_sync(0xffffffffu, send, 2);
   }
-  double s = (lane & 4 ? u[1] : u[0]) + __shfl_xor_sync(0xffffffffu, lane & 4 ? u[0] : u[1], 4);
+  T s = (lane & 4 ? u[1] : u[0]) + __shfl_xor_sync(0xffffffffu, lane & 4 ? u[0] : u[1], 4);
   s += __shfl_xor_sync(0xffffffffu, s, 8);
   s += __shfl_xor_sync(0xffffffffu, s, 16);
   return s;
@@ -477,7 +491,9 @@ cudaError_t launch_kick(Ctx &c);
 cudaError_t launch_kinetic(Ctx &c);
 cudaError_t launch_thermostat(Ctx &c, int mode);  // 0: end + next start half, 1: start half only
 cudaError_t launch_totals_compact(Ctx &c);  // the pair passes' partials, where there are many
-cudaError_t launch_totals(Ctx &c);
+// Totals of the evaluation: the energies and virials (part 1), the kinetic energy (part 2; a
+// thermostat's step sets it itself) or both.
+cudaError_t launch_totals(Ctx &c, int parts = 3);
 int64_t partials_compact_count(int64_t nblk);
 // The totals sum every slot of a pass's partial range: a pass whose grid writes fewer slots
 // than the range holds clears the rest (another kernel may have filled them before).
