@@ -50,6 +50,7 @@ struct CoulArgs {
   float fscale;               //   F is not written), their scale (FP32 forms)
   double fscale_d;            //   (FP64 form)
   int *err;                   //   (a sum out of range sets ERRBIT_NONFINITE)
+  ErfcFit fit;
 };
 
 int64_t coul_blocks(int64_t nq) { return (nq + kCoulWarps - 1) / kCoulWarps; }
@@ -58,9 +59,10 @@ template <typename real>
 __device__ __forceinline__ void coul_body(const CoulArgs a, int bx, int) {
   constexpr bool F64 = sizeof(real) == 8;
   constexpr unsigned FULL = 0xffffffffu;
-  __shared__ int4 buf[kCoulWarps][kCoulBuf];  // hits: integer displacement, charge bits or index
-  __shared__ int32_t seg_beg[kCoulWarps][2 * kCoulMaxRows];
-  __shared__ int32_t seg_pre[kCoulWarps][2 * kCoulMaxRows + 1];
+  // hits: displacement and charge (FP32 forms), or integer displacement and index
+  __shared__ int4 buf[kCoulWarps][kCoulBuf];
+  __shared__ int32_t seg_off[kCoulWarps][2 * kCoulMaxRows];
+  __shared__ int32_t seg_pre[kCoulWarps][2 * kCoulMaxRows];
   __shared__ double wred[kCoulWarps][2];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const PairConst &pc = a.pc;
@@ -80,7 +82,7 @@ __device__ __forceinline__ void coul_body(const CoulArgs a, int bx, int) {
     const float fyc = (float)pi.y * ((float)n1 * 2.3283064365386963e-10f);
     const float fzc = (float)pi.z * ((float)n2 * 2.3283064365386963e-10f);
     const float wy = pc.h[1] * (4294967296.0f / (float)n1), wz = pc.h[2] * (4294967296.0f / (float)n2);
-    int carry = 0;
+    int carry = 0, nseg = 0;
     for (int rb = 0; rb < nrows; rb += 32) {
       const int t = rb + lane;
       int b0 = 0, l0 = 0, b1 = 0, l1 = 0;
@@ -101,19 +103,20 @@ __device__ __forceinline__ void coul_body(const CoulArgs a, int bx, int) {
           rzw += rzw < 0 ? n2 : 0;
           rzw -= rzw >= n2 ? n2 : 0;
           const int64_t rowbase = (int64_t)n0 * (ryw + (int64_t)n1 * rzw);
-          // x-cells within reach (unwrapped floor division by the cell width)
-          const int64_t reach = (int64_t)(sqrtf(rx2) * (1.0f + 1e-5f) / pc.h[0]) + 4;
-          const int64_t c0 = (((int64_t)pi.x - reach) * n0) >> 32;
-          const int64_t c1 = (((int64_t)pi.x + reach) * n0) >> 32;
-          int sa0, sb0, sa1 = 0, sb1 = -1;
-          if (c1 - c0 + 1 >= n0) { sa0 = 0; sb0 = n0 - 1; }
-          else if (c0 < 0) { sa0 = (int)(c0 + n0); sb0 = n0 - 1; sa1 = 0; sb1 = (int)c1; }
-          else if (c1 >= n0) { sa0 = (int)c0; sb0 = n0 - 1; sa1 = 0; sb1 = (int)(c1 - n0); }
-          else { sa0 = (int)c0; sb0 = (int)c1; }
+          // x-cells within reach: one run, or two where the reach passes an end of the box
+          const uint32_t reach = (uint32_t)(sqrtf(rx2) * (1.0f + 1e-5f) / pc.h[0]) + 4u;
+          const uint32_t xl = pi.x - reach, xr = pi.x + reach;
+          const bool wl = xl > pi.x, wr = xr < pi.x;
+          int sa0 = cell_of(xl, n0), sb0 = cell_of(xr, n0), sb1 = -1;
+          if (wl || wr) {
+            if ((wl && wr) || sb0 + 1 >= sa0) sa0 = 0;  // (the whole row)
+            else sb1 = sb0;                             // and from the row's start
+            sb0 = n0 - 1;
+          }
           b0 = a.cell_start[rowbase + sa0];
           l0 = a.cell_start[rowbase + sb0 + 1] - b0;
-          if (sb1 >= sa1) {
-            b1 = a.cell_start[rowbase + sa1];
+          if (sb1 >= 0) {
+            b1 = a.cell_start[rowbase];
             l1 = a.cell_start[rowbase + sb1 + 1] - b1;
           }
         }
@@ -125,82 +128,89 @@ __device__ __forceinline__ void coul_body(const CoulArgs a, int bx, int) {
         const int v = __shfl_up_sync(FULL, incl, o);
         if (lane >= o) incl += v;
       }
+      // the runs that hold candidates, in order: offset in the list, and first particle minus it
       const int excl = carry + incl - tot;
-      if (t < nrows) {
-        seg_beg[wid][2 * t] = b0;
-        seg_pre[wid][2 * t] = excl;
-        seg_beg[wid][2 * t + 1] = b1;
-        seg_pre[wid][2 * t + 1] = excl + l0;
+      const unsigned m0 = __ballot_sync(FULL, l0 > 0), m1 = __ballot_sync(FULL, l1 > 0);
+      const unsigned below = (1u << lane) - 1u;
+      int k = nseg + __popc(m0 & below) + __popc(m1 & below);
+      if (l0 > 0) {
+        seg_pre[wid][k] = excl;
+        seg_off[wid][k++] = b0 - excl;
       }
+      if (l1 > 0) {
+        seg_pre[wid][k] = excl + l0;
+        seg_off[wid][k] = b1 - excl - l0;
+      }
+      nseg += __popc(m0) + __popc(m1);
       carry += __shfl_sync(FULL, incl, 31);
     }
-    if (lane == 0) seg_pre[wid][2 * nrows] = carry;
     __syncwarp();
     const int T = carry;
-    // evaluate buffered hits [0, n) (one per lane)
-    auto evaluate = [&](int n) {
-      if (lane < n) {
-        const int4 e = buf[wid][lane];
-        real dx, dy, dz, r2, qj;
-        if (F64) {
-          dx = (real)(i2d(e.x) * pc.hd[0]);
-          dy = (real)(i2d(e.y) * pc.hd[1]);
-          dz = (real)(i2d(e.z) * pc.hd[2]);
-          r2 = mad(dx, dx, mad(dy, dy, dz * dz));
-          qj = (real)a.qd[e.w];
-        } else {
-          dx = (real)((float)e.x * pc.h[0]);
-          dy = (real)((float)e.y * pc.h[1]);
-          dz = (real)((float)e.z * pc.h[2]);
-          r2 = mad(dx, dx, mad(dy, dy, dz * dz));
-          qj = (real)__int_as_float(e.w);
-        }
-        real r, rinv, erfcv, expv;
-        if (F64) {
-          // 1/r from an FP32 start by one third-order Householder step (as in the pair kernel)
-          const float ex = (float)e.x * pc.h[0], ey = (float)e.y * pc.h[1], ez = (float)e.z * pc.h[2];
-          const double z = f2d(rsqrtf(fmaf(ex, ex, fmaf(ey, ey, ez * ez))));
-          const double c = fma(-((double)r2 * z), z, 1.0);
-          rinv = (real)fma(z, c * fma(c, 0.375, 0.5), z);
-          r = r2 * rinv;
-          erfcv = (real)erfc(pc.sqrt_alpha_d * (double)r);
-          expv = (real)exp(-pc.alpha_d * (double)r2);
-        } else {
-          rinv = (real)rsqrtf((float)r2);
-          r = r2 * rinv;
-          erfcv = (real)erfcf(pc.sqrt_alpha * (float)r);
-          expv = (real)expf(-pc.alpha * (float)r2);
-        }
-        const real Cqq = (F64 ? (real)pc.C_d : (real)pc.C) * qi * qj;
-        const real tsp = F64 ? (real)pc.two_sqrt_alpha_over_sqrt_pi_d
-                             : (real)pc.two_sqrt_alpha_over_sqrt_pi;
-        const real rinv2 = rinv * rinv;
-        const real gc = Cqq * mad(erfcv * rinv, rinv2, tsp * expv * rinv2);
-        fx = mad(gc, dx, fx); fy = mad(gc, dy, fy); fz = mad(gc, dz, fz);
-        if (a.comp) {
-          kahan_add(uc, cuc, Cqq * erfcv * rinv);
-          kahan_add(wc, cwc, gc * r2);
-        } else {
-          uc = mad(Cqq * erfcv, rinv, uc);
-          wc = mad(gc, r2, wc);
-        }
+    // Buffered hits [0, n), one per lane, in the FP32 forms.
+    auto evaluate32 = [&](int n) {
+      if (lane >= n) return;
+      const int4 e = buf[wid][lane];
+      const float dx = __int_as_float(e.x), dy = __int_as_float(e.y), dz = __int_as_float(e.z);
+      const float r2 = mad(dx, dx, mad(dy, dy, dz * dz)), rinv = rsqrtf(r2), r = r2 * rinv;
+      float er, ex;
+      if (a.fit.ok) {
+        erfc_exp1(a.fit, r, r2, er, ex);
+      } else {
+        er = erfcf(pc.sqrt_alpha * r);
+        ex = expf(-pc.alpha * r2);
+      }
+      const float Cqq = pc.C * (float)qi * __int_as_float(e.w), rinv2 = rinv * rinv;
+      const float gc = Cqq * mad(er * rinv, rinv2, pc.two_sqrt_alpha_over_sqrt_pi * ex * rinv2);
+      fx = mad((real)gc, (real)dx, fx); fy = mad((real)gc, (real)dy, fy); fz = mad((real)gc, (real)dz, fz);
+      if (a.comp) {
+        kahan_add(uc, cuc, (real)(Cqq * er * rinv));
+        kahan_add(wc, cwc, (real)(gc * r2));
+      } else {
+        uc = mad((real)(Cqq * er), (real)rinv, uc);
+        wc = mad((real)gc, (real)r2, wc);
       }
     };
-    int nb = 0;  // buffered hits (warp-uniform)
-    const int nseg = 2 * nrows;
+    // FP64 form: one per lane.
+    auto evaluate64 = [&](int n) {
+      if (lane < n) {
+        const int4 e = buf[wid][lane];
+        const double dx = i2d(e.x) * pc.hd[0], dy = i2d(e.y) * pc.hd[1], dz = i2d(e.z) * pc.hd[2];
+        const double r2 = mad(dx, dx, mad(dy, dy, dz * dz));
+        // 1/r from an FP32 start by one third-order Householder step (as in the pair kernel)
+        const float ex = (float)e.x * pc.h[0], ey = (float)e.y * pc.h[1], ez = (float)e.z * pc.h[2];
+        const double z = f2d(rsqrtf(fmaf(ex, ex, fmaf(ey, ey, ez * ez))));
+        const double c = fma(-(r2 * z), z, 1.0);
+        const double rinv = fma(z, c * fma(c, 0.375, 0.5), z), r = r2 * rinv;
+        const double erfcv = erfc(pc.sqrt_alpha_d * r), expv = exp(-pc.alpha_d * r2);
+        const double Cqq = pc.C_d * (double)qi * a.qd[e.w], rinv2 = rinv * rinv;
+        const double gc =
+            Cqq * mad(erfcv * rinv, rinv2, pc.two_sqrt_alpha_over_sqrt_pi_d * expv * rinv2);
+        fx = mad((real)gc, (real)dx, fx); fy = mad((real)gc, (real)dy, fy); fz = mad((real)gc, (real)dz, fz);
+        uc = mad((real)(Cqq * erfcv), (real)rinv, uc);
+        wc = mad((real)gc, (real)r2, wc);
+      }
+    };
+    auto evaluate = [&](int n) {
+      if constexpr (F64) evaluate64(n); else evaluate32(n);
+    };
+    int nb = 0;      // buffered hits (warp-uniform)
+    int before = 0;  // runs that start before the 32 candidates
     for (int base = 0; base < T; base += 32) {
       const int cc = base + lane;
       bool hit = false;
       int4 rec = make_int4(0, 0, 0, 0);
+      // a bit for each run that starts among these candidates; cc's run is the last one at or
+      // before it
+      unsigned starts = 0u;
+      for (int k = lane; k < nseg; k += 32) {
+        const unsigned d = (unsigned)(seg_pre[wid][k] - base);
+        starts |= d < 32u ? 1u << d : 0u;
+      }
+      starts = __reduce_or_sync(FULL, starts);
+      const int run = before + __popc(starts & (0xffffffffu >> (31 - lane))) - 1;
+      before += __popc(starts);
       if (cc < T) {
-        // candidate cc's run: the last of the (possibly empty) runs starting at or before cc,
-        // by a binary search over the run offsets (the same steps on every lane)
-        int s = 0, hi = nseg;
-        while (hi - s > 1) {
-          const int mid = (s + hi) >> 1;
-          if (seg_pre[wid][mid] <= cc) s = mid; else hi = mid;
-        }
-        const int64_t j = seg_beg[wid][s] + (cc - seg_pre[wid][s]);
+        const int64_t j = cc + seg_off[wid][run];
         if (j != i) {
           const uint4 pj = a.s4[j];
           const int dsx = (int)(pi.x - pj.x), dsy = (int)(pi.y - pj.y), dsz = (int)(pi.z - pj.z);
@@ -209,7 +219,8 @@ __device__ __forceinline__ void coul_body(const CoulArgs a, int bx, int) {
           const float r2 = mad(ex, ex, mad(ey, ey, ez * ez));
           hit = r2 < pc.rc2_lo;
           if (r2 >= pc.rc2_lo && r2 <= pc.rc2_hi) hit = exact_r2(pc, dsx, dsy, dsz) <= pc.rc2d;
-          rec = make_int4(dsx, dsy, dsz, F64 ? (int)j : (int)pj.w);
+          rec = F64 ? make_int4(dsx, dsy, dsz, (int)j)
+                    : make_int4(__float_as_int(ex), __float_as_int(ey), __float_as_int(ez), (int)pj.w);
         }
       }
       const unsigned hm = __ballot_sync(FULL, hit);
@@ -257,11 +268,14 @@ __device__ __forceinline__ void coul_body(const CoulArgs a, int bx, int) {
   }
 }
 
-// (16 blocks of 4 warps in the FP32 forms: the whole SM's 64 warps; the pass is bound by the
-// latency of each warp's dependent loads, so occupancy is what hides it; 8 in the FP64 form,
-// whose registers would spill)
+// (12 blocks of 4 warps in the FP32 forms, 40 registers without spills; 16 run as fast with spills,
+// 10 slower: the pass is bound by issue and by the latency of each warp's dependent loads. Two hits
+// a lane as a packed pair took 48 registers and 154 us where one takes 121. 104,858 charged of
+// 2^20: 135 us with a binary search for a candidate's run and erfcf and expf, 122 so; 400,000 of
+// 4,000,001: 481 -> 433. 8 in the
+// FP64 form, whose registers would spill.)
 template <typename real>
-__global__ void __launch_bounds__(kCoulWarps * 32, sizeof(real) == 8 ? 8 : 16)
+__global__ void __launch_bounds__(kCoulWarps * 32, sizeof(real) == 8 ? 8 : 12)
     coul_kernel(const CoulArgs a) {
   coul_body<real>(a, (int)blockIdx.x, (int)gridDim.x);
 }
@@ -285,6 +299,7 @@ cudaError_t launch_coulomb_subset(Ctx &c, const uint4 *s4, bool into_facc) {
   a.fscale = (float)kFixScale32;
   a.fscale_d = kFixScale64;
   a.err = c.err;
+  a.fit = c.fit;
   const dim3 g((unsigned)c.n_coul_blk), b(kCoulWarps * 32);  // every slot of the partial range
   // (per replica in a batch, like the other pair kernels)
   if (c.precision == RBE_FP64)

@@ -120,6 +120,17 @@ __device__ __forceinline__ void erfc_exp2(const ErfcFit &f, f32x2 r, f32x2 r2, f
   er = mul2(ex, p);
 }
 
+// One value of each.
+__device__ __forceinline__ void erfc_exp1(const ErfcFit &f, float r, float r2, float &er, float &ex) {
+  const float t = fmaf(r, f.ts, -1.f);
+  float p = f.c[kErfcDeg];
+#pragma unroll
+  for (int k = kErfcDeg - 1; k >= 0; --k) p = fmaf(p, t, f.c[k]);
+  const float arg = r2 * f.ea, d = fmaf(r2, -f.ea_lo, fmaf(r2, -f.ea, arg)), e = ex2_approx(-arg);
+  ex = fmaf(e, d * 0.693147181f, e);
+  er = ex * p;
+}
+
 // Squared distance of the exact cutoff decision (the oracle's definition): dx_d =
 // (int32)(s_i - s_j) * (L_d / 2^32) and r2 = dx^2 + dy^2 + dz^2 in FP64, no FMA.
 __device__ __forceinline__ double exact_r2(const PairConst &pc, int dsx, int dsy, int dsz) {
