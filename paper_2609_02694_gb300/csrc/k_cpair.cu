@@ -112,6 +112,7 @@ struct FinishArgs {
   int64_t n3;
   float sh, sl;
   double inv_scale;
+  int per;                 // sums a block (a multiple of 512, at most 512 kFinishPairs)
 };
 
 // One block: clusters and super-clusters of every row, as exclusive prefix sums.
@@ -233,8 +234,12 @@ RBE_BATCHED_KERNEL(__launch_bounds__(256), cluster_bounds_kernel, BoundsArgs, cl
 // 64-bit sum converts as its two 32-bit halves (a 64-bit integer conversion is slow here):
 // v = hi 2^32 + lo with hi signed and lo unsigned; FP32 forms take the FP32 factors
 // sh = 2^32 / scale and sl = 1 / scale (no FP64 work per element), the FP64 form the FP64 ones.
-// Four sums a thread in 16-byte accesses (one 8-byte sum a thread left most of the pass
-// waiting on memory latency).
+// The pass waits on the latency of loads from sums that atomics have just written, so a thread has up
+// to eight 16-byte loads in flight: 12,000,003 sums, 512 / 1,024 / 2,048 / 4,096 a block: 159 / 115 / 67 /
+// 46 us, an 8-byte pair of floats a store; cold 120 -> 32 (it moves 240 MB). Fewer a block in a small box, to spread over the SMs.
+constexpr int kFinishPairs = 8;  // pairs of sums a thread, at most
+template <typename real> struct Pair2 { using type = float2; };
+template <> struct Pair2<double> { using type = double2; };
 template <typename real>
 __device__ __forceinline__ real fx_value(long long v, const FinishArgs &a) {
   const int hi = (int)(v >> 32);
@@ -245,30 +250,33 @@ __device__ __forceinline__ real fx_value(long long v, const FinishArgs &a) {
 
 template <typename real>
 __device__ __forceinline__ void cpair_finalize_body(const FinishArgs &a, int bx, int) {
-  const int64_t k0 = 4 * ((int64_t)bx * blockDim.x + threadIdx.x);
-  const int64_t n3 = a.n3;
-  if (k0 >= n3) return;
-  long long *__restrict__ facc = a.facc;
-  real *__restrict__ F = static_cast<real *>(a.F);
-  if (k0 + 4 <= n3) {  // facc and F start 256-byte aligned, k0 is a multiple of 4
-    const longlong2 u = *reinterpret_cast<const longlong2 *>(facc + k0);
-    const longlong2 w = *reinterpret_cast<const longlong2 *>(facc + k0 + 2);
-    *reinterpret_cast<longlong2 *>(facc + k0) = make_longlong2(0, 0);
-    *reinterpret_cast<longlong2 *>(facc + k0 + 2) = make_longlong2(0, 0);
-    const real f0 = fx_value<real>(u.x, a), f1 = fx_value<real>(u.y, a);
-    const real f2 = fx_value<real>(w.x, a), f3 = fx_value<real>(w.y, a);
-    if (sizeof(real) == 4) {
-      *reinterpret_cast<float4 *>(F + k0) = make_float4((float)f0, (float)f1, (float)f2, (float)f3);
-    } else {
-      *reinterpret_cast<double2 *>(F + k0) = make_double2((double)f0, (double)f1);
-      *reinterpret_cast<double2 *>(F + k0 + 2) = make_double2((double)f2, (double)f3);
+  using real2 = typename Pair2<real>::type;
+  // (facc and F start 256-byte aligned and b0 is even: pairs)
+  const int64_t b0 = (int64_t)bx * a.per, b1 = min(b0 + a.per, a.n3);
+  const int np = (int)((b1 - b0) >> 1);
+  longlong2 *p = reinterpret_cast<longlong2 *>(a.facc + b0);
+  real2 *f = reinterpret_cast<real2 *>(static_cast<real *>(a.F) + b0);
+  longlong2 v[kFinishPairs];
+#pragma unroll
+  for (int k = 0; k < kFinishPairs; ++k) {
+    const int t = threadIdx.x + 256 * k;
+    if (t < np) v[k] = p[t];
+  }
+#pragma unroll
+  for (int k = 0; k < kFinishPairs; ++k) {
+    const int t = threadIdx.x + 256 * k;
+    if (t < np) {
+      p[t] = make_longlong2(0, 0);
+      real2 o;
+      o.x = fx_value<real>(v[k].x, a);
+      o.y = fx_value<real>(v[k].y, a);
+      f[t] = o;
     }
-  } else {
-    for (int64_t k = k0; k < n3; ++k) {
-      const long long v = facc[k];
-      facc[k] = 0;
-      F[k] = fx_value<real>(v, a);
-    }
+  }
+  if (((b1 - b0) & 1) && threadIdx.x == 0) {  // the last sum of an odd number
+    const long long w = a.facc[b1 - 1];
+    a.facc[b1 - 1] = 0;
+    static_cast<real *>(a.F)[b1 - 1] = fx_value<real>(w, a);
   }
 }
 template <typename real>
@@ -1436,14 +1444,16 @@ cudaError_t launch_cluster_finish(Ctx &c) {
   const int64_t n3 = 3 * c.N;
   // (per replica in a batch too: it joins the pair kernel, the Coulomb pass and the gather in
   // one run of per-replica launches, one fork and join per step)
-  const dim3 fg((unsigned)(((n3 + 3) / 4 + 255) / 256)), fb(256);
+  const int per = (int)std::min<int64_t>(
+      512 * kFinishPairs, std::max<int64_t>(512, n3 / ((int64_t)4 * c.sms) / 512 * 512));
+  const dim3 fg((unsigned)((n3 + per - 1) / per)), fb(256);
   if (fp64) {
-    const FinishArgs f{c.facc, c.Fd, n3, 0.f, 0.f, 1.0 / kFixScale64};
+    const FinishArgs f{c.facc, c.Fd, n3, 0.f, 0.f, 1.0 / kFixScale64, per};
     return dispatch(c, cpair_finalize_kernel<double>, cpair_finalize_kernel_b<double>, fg, fb, 0, f,
                     true);
   }
   const FinishArgs f{c.facc, c.F, n3, (float)(4294967296.0 / kFixScale32),
-                     (float)(1.0 / kFixScale32), 0.0};
+                     (float)(1.0 / kFixScale32), 0.0, per};
   return dispatch(c, cpair_finalize_kernel<float>, cpair_finalize_kernel_b<float>, fg, fb, 0, f,
                   true);
 }

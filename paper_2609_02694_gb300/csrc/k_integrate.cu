@@ -327,18 +327,20 @@ __device__ __forceinline__ void totals_body(const TotalsArgs &a, int, int) {
   ACC acc[NV];
   for (int k = 0; k < NV; ++k) acc[k] = (ACC)0;
   const double *srcs[3] = {a.pair, a.coul, a.rbl};
-  const int64_t ns[3] = {a.n_pair, a.n_coul, a.n_rbl};
-  for (int r = 0; r < 3 && a.parts & 1; ++r) {
+  const bool en = a.parts & 1, kin = a.parts & 2;
+  const int64_t ns[3] = {en ? a.n_pair : 0, en ? a.n_coul : 0, en ? a.n_rbl : 0};
+  const int64_t n_ke = kin ? a.n_ke : 0;
+  for (int r = 0; r < 3; ++r) {
 #pragma unroll 4
     for (int64_t b = threadIdx.x; b < ns[r]; b += blockDim.x)
       for (int k = 0; k < NQ_PAIR; ++k) acc[k] += (ACC)srcs[r][b * NQ_PAIR + k];
   }
-  for (int l = threadIdx.x; l < a.P && a.parts & 1; l += blockDim.x) {
+  for (int l = threadIdx.x; l < (en ? a.P : 0); l += blockDim.x) {
     acc[4] += (ACC)a.emode[2 * l];
     acc[5] += (ACC)a.emode[2 * l + 1];
   }
 #pragma unroll 4
-  for (int64_t b = threadIdx.x; b < a.n_ke && a.parts & 2; b += blockDim.x) acc[6] += (ACC)a.ke[b];
+  for (int64_t b = threadIdx.x; b < n_ke; b += blockDim.x) acc[6] += (ACC)a.ke[b];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const ACC v = warp_sum8(acc, lane);
   if (lane < NV) sh[lane][wid] = v;
@@ -353,8 +355,8 @@ __device__ __forceinline__ void totals_body(const TotalsArgs &a, int, int) {
     const double ur = (double)sh[Q_UREAL][0], ul = (double)sh[Q_ULJ][0];
     const double wr = (double)sh[Q_WREAL][0], wl = (double)sh[Q_WLJ][0];
     const double uk = (double)sh[4][0], wk = (double)sh[5][0];
-    if (a.parts & 2) a.scal[S_KE] = a.ke_override ? *a.ke_override : (double)sh[6][0];
-    if (!(a.parts & 1)) return;
+    if (kin) a.scal[S_KE] = a.ke_override ? *a.ke_override : (double)sh[6][0];
+    if (!en) return;
     a.scal[S_UREAL] = ur;
     a.scal[S_ULJ] = ul;
     a.scal[S_UK] = uk;
