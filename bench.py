@@ -492,7 +492,7 @@ def run_ours(args):
                                     "events in the graph; the headline ran without them"},
             "roofline": {"bound": "alu",
                          "kernel": ("list_pair_kernel (Verlet-list LJ)" if skin > 0
-                                    else "cpair_kernel (cluster pairs, LJ)"
+                                    else "cpair32_kernel (cluster pairs, LJ)"
                                     if tuned.get("pair_cluster")
                                     else "pair_kernel (cell-list LJ)"),
                          "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
