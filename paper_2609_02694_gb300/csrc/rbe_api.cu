@@ -389,9 +389,11 @@ bool reaches(const void *p, size_t bytes, size_t align, cudaMemoryType type) {
   return ok;
 }
 
-int copy_scalars(Ctx &c, double *energies, double *virial) {
-  RBE_CUDA_TRY(cudaMemcpyAsync(c.scal_host, c.scal, sizeof(double) * S_COUNT,
-                               cudaMemcpyDeviceToHost, c.stream));
+// there: the stream's work brings the scalars to the host
+int copy_scalars(Ctx &c, double *energies, double *virial, bool there = false) {
+  if (!there)
+    RBE_CUDA_TRY(cudaMemcpyAsync(c.scal_host, c.scal, sizeof(double) * S_COUNT,
+                                 cudaMemcpyDeviceToHost, c.stream));
   RBE_CUDA_TRY(cudaStreamSynchronize(c.stream));
   const double *s = c.scal_host;
   if (energies) {
@@ -876,7 +878,8 @@ int rbe_forces(rbe_handle h, uint64_t step, float *F_out, int F_on_device, doubl
     const bool direct = F_on_device ? reaches(F_out, bytes, 4, cudaMemoryTypeDevice)
                                     : c.N <= kPinnedN && reaches(F_out, bytes, 4, cudaMemoryTypeHost);
     RBE_CUDA_TRY(launch_scatter_forces(c, false, direct ? F_out : nullptr,
-                                       host || scalars ? c.flags_host : nullptr));
+                                       host || scalars ? c.flags_host : nullptr,
+                                       scalars ? c.scal_host : nullptr));
     if (!direct)
       RBE_CUDA_TRY(cudaMemcpyAsync(F_out, c.outf, bytes,
                                    F_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
@@ -886,7 +889,7 @@ int rbe_forces(rbe_handle h, uint64_t step, float *F_out, int F_on_device, doubl
   if (!F_out || c.N == 0)
     RBE_CUDA_TRY(cudaMemcpyAsync(c.flags_host, c.err, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
   if (scalars) {
-    rc = copy_scalars(c, energies, virial);
+    rc = copy_scalars(c, energies, virial, F_out && c.N > 0);
     if (rc != RBE_OK) return rc;
   } else {
     RBE_CUDA_TRY(cudaStreamSynchronize(c.stream));

@@ -506,7 +506,7 @@ cudaError_t launch_step_advance(Ctx &c);
 // Forces in id order, to outf (device; null: c.outf) or c.outd.
 // (outf, nullable: where to, of memory this device writes; else the device staging array)
 cudaError_t launch_scatter_forces(Ctx &c, bool to_double, float *outf = nullptr,
-                                  int *err_out = nullptr);
+                                  int *err_out = nullptr, double *scal_out = nullptr);
 // (each destination nullable)
 cudaError_t launch_scatter_state(Ctx &c, double *pos, double *vel, uint32_t *frac, int *err_out);
 cudaError_t launch_set_positions(Ctx &c, const double *pos);  // (memory this device reads)
