@@ -824,7 +824,9 @@ __global__ void __launch_bounds__(32, EAGER ? 18 : 20) rbl32_kernel(const RblArg
       for (int w = 0; w < 2; ++w) {
         const int c = base + 32 * w + lane;
         int s = sg, dxj = 0, dyj = 0, dzj = 0, tj = 0;
-        nx[w] = ny[w] = nz[w] = 3e17f;  // past the last candidate: beyond every member's reach
+        // past the last candidate: beyond every member's reach, or, where differences are folded
+        // into the box, anywhere (dropped below)
+        nx[w] = ny[w] = nz[w] = 3e17f;
         float qj = 0.f;
         if (c < T) {
           s = run_of(c, sg);
@@ -872,8 +874,11 @@ __global__ void __launch_bounds__(32, EAGER ? 18 : 20) rbl32_kernel(const RblArg
       c0 = __brev(c0); c1 = __brev(c1); s0 = __brev(s0); s1 = __brev(s1);
       s0 &= ~c0;
       s1 &= ~c1;
+      // (WRAP: those of the window's slots that hold a candidate; a far coordinate folds to any
+      // value, to 0 where L divides it. The same in the other variant costs 5%.)
+      const int held = WRAP ? min(64, T - base) : 64;
       if (in && (bc <= a.rc_half || bs <= a.rs_half)) {  // rare: the exact decision
-        for (int c = 0; c < 64; ++c) {
+        for (int c = 0; c < held; ++c) {
           const f32x2 rp = pair_r2(c & 31);
           const float r2 = c < 32 ? rp.x : rp.y;
           if (!(fabsf(r2 - a.rc_mid) <= a.rc_half || fabsf(r2 - a.rs_mid) <= a.rs_half)) continue;
@@ -887,6 +892,12 @@ __global__ void __launch_bounds__(32, EAGER ? 18 : 20) rbl32_kernel(const RblArg
           mc = isc ? mc | b : mc & ~b;
           ms = iss ? ms | b : ms & ~b;
         }
+      }
+      if (WRAP && held < 64) {
+        const uint32_t h0 = held < 32 ? (1u << held) - 1u : 0xffffffffu;
+        const uint32_t h1 = held > 32 ? (1u << (held - 32)) - 1u : 0u;
+        c0 &= h0; s0 &= h0;
+        c1 &= h1; s1 &= h1;
       }
       if (!in) c0 = c1 = s0 = s1 = 0u;
       const int ks = self - base;  // the particle itself (r = 0) is no pair
