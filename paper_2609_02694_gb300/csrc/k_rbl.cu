@@ -554,7 +554,7 @@ constexpr int kRblMaxWin = kRblMaxChunks / 2;
 
 struct RblAcc2 {
   f32x2 fx, fy, fz;
-  f32x2 u0, u1;            // one type: sum r^-12, sum r^-6; several: sum 12 A r^-12, sum -6 B r^-6
+  f32x2 u0, u1;            // one type: the virial and sum r^-6; several: sum 12 A r^-12, sum -6 B r^-6
   f32x2 uc, wc, cuc, cwc;  // Coulomb energy and virial (Kahan compensations)
 };
 
@@ -585,8 +585,10 @@ __device__ __forceinline__ void rbl_eval2(const RblArgs &a, bool a0, bool a1, in
     acc.u0 = fma2(mul2(A, ir6), ir6, acc.u0);
     acc.u1 = fma2(B, ir6, acc.u1);
   } else {
-    g = mul2(mul2(ir6, ir2), fma2(pk(a.pa.ljA12), ir6, pk(-a.pa.ljB6)));
-    acc.u0 = fma2(ir6, ir6, acc.u0);
+    // (no r^-12 without its coefficient: it leaves FP32's range in small units of length)
+    const f32x2 t = fma2(pk(a.pa.ljA12), ir6, pk(-a.pa.ljB6));
+    g = mul2(mul2(ir6, ir2), t);
+    acc.u0 = fma2(ir6, t, acc.u0);
     acc.u1 = add2(acc.u1, ir6);
   }
   if (COUL) {
@@ -976,8 +978,9 @@ __global__ void __launch_bounds__(32, EAGER ? 18 : 20) rbl32_kernel(const RblArg
       ulj = fmaf(u0, 1.f / 12.f, u1 * (1.f / 6.f));
       wlj = u0 + u1;
     } else {
-      ulj = fmaf(a.pa.ljA, u0, -(a.pa.ljB * u1));
-      wlj = fmaf(a.pa.ljA12, u0, -(a.pa.ljB6 * u1));
+      // u0 = 12 A s12 - 6 B s6 and u1 = s6, so A s12 - B s6 = (u0 - 6 B s6) / 12
+      ulj = fmaf(-a.pa.ljB6, u1, u0) * (1.f / 12.f);
+      wlj = u0;
     }
     if (COUL) {  // core + w shell with the compensations, as an unevaluated FP32 sum
       auto total = [&](const f32x2 &cs, const f32x2 &cc, const f32x2 &ss, const f32x2 &sc, float &h,

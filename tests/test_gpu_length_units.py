@@ -2,7 +2,9 @@
 
 Forces and energies are those of the oracle in the same units, within the bounds that hold in
 Angstrom: 1e-5 for the forces, 2e-6 for the energies. The scales: 30 and 60 (r_c^-14 leaves the
-normal FP32 numbers in between) and 100 (picometres; 2^32 times 48 eps sigma^12 is no FP32 number).
+normal FP32 numbers in between), 100 (picometres; 2^32 times 48 eps sigma^12 is no FP32 number)
+and, for the random batch list, whose forces are no fixed-point sums, 7 / 30000 (r^-12 of close
+pairs is no FP32 number; eps is raised so that 48 eps sigma^12 is a normal one).
 """
 import numpy as np
 import pytest
@@ -43,3 +45,25 @@ def test_cells(orc, precision, u, cluster):
     assert np.array_equal(nbr, ref["nbr"])
     assert rel_l2(F, ref["F"]) < 1e-5
     assert E["lj"] == pytest.approx(ref["U_lj"], rel=2e-6)
+
+
+@pytest.mark.parametrize("precision", ["fp32_comp", "fp32"])
+@pytest.mark.parametrize("u,eps", [(1.0, 0.1), (30.0, 0.1), (100.0, 0.1), (7.0 / 30000, 1e5)])
+@pytest.mark.parametrize("eager", [0, 1])
+def test_random_batch_list(orc, precision, u, eps, eager):
+    sy, alpha, C = scaled(6001, u, eps)
+    r_core, r_s, p, seed, step = 4.0 * u, 8.0 * u, 10, 3, 6
+    with binding.from_system(sy, P=8, alpha=alpha, r_c=r_s, r_core=r_core, p_rbl=p, seed=seed,
+                             coulomb_C=C, precision=precision) as h:
+        h.set_tuning("rbl_eager", eager)
+        F, E, W = h.forces_f64(step)
+        pa = h.rbl_partners()
+        m, S = h.sample_k(step)
+    ref = orc.rbl(sy.s, sy.q, sy.types, sy.box, alpha, r_core, r_s, p, seed, step, 0, C, sy.eps,
+                  sy.sig)
+    assert np.array_equal(pa, ref["partners"])
+    Fk, _, _ = orc.rbe_kspace(sy.s, sy.q, sy.box, alpha, C, m, S)
+    assert rel_l2(F, ref["F"] + Fk) < 1e-5
+    assert abs(E["lj"] - ref["U_lj"]) < 2e-6 * (abs(ref["U_lj"]) + abs(ref["U_real"]))
+    assert E["lj"] == pytest.approx(ref["U_lj"], rel=2e-5)
+    assert W["lj"] == pytest.approx(ref["W_lj"], rel=2e-5)
