@@ -331,7 +331,8 @@ int force_pipeline(Ctx &c, bool debug) {
 // Kernels one Verlet step launches (memsets excluded).
 int64_t kernels_per_step(const Ctx &c) {
   int64_t k = 1;                         // kick-drift (with the step counter)
-  k += c.scan_nblk > 1 ? 5 : 4;          // count, scan (one or two passes), scatter, rank+permute
+  // count, scan (one to three passes), scatter, rank+permute
+  k += c.scan_nblk > kScanDirect ? 6 : (c.scan_nblk > 1 ? 5 : 4);
   k += 1;                                // sampler
   k += c.Nq > 0 ? 2 : 0;                 // structure factor + combine
   if (c.rbl) k += 4;                     // RBL, compact partials, mean, subtract

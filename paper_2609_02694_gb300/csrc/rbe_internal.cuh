@@ -30,6 +30,7 @@ enum : int { ERRBIT_SAMPLER = 1, ERRBIT_NONFINITE = 2, ERRBIT_CAPACITY = 4 };
 
 // Partial-sum slots (doubles per block) of the energy / virial reductions.
 enum : int { Q_UREAL = 0, Q_ULJ = 1, Q_WREAL = 2, Q_WLJ = 3, NQ_PAIR = 4 };
+constexpr int64_t kScanDirect = 1 << 14;  // blocks of the cell scan that add up the totals before them
 constexpr int kCompactMax = 256;  // compacted partials per pair pass before the totals
 // Fixed-point scales of the cluster kernel's force sums (64-bit integers): 2^32 in the FP32
 // forms, 2^40 in the FP64 form.
