@@ -167,7 +167,7 @@ int free_all(Ctx &c) {
     if (c.fgraph[b]) cudaGraphExecDestroy(c.fgraph[b]);
     c.fgraph[b] = nullptr;
   }
-  dfree(c.F); dfree(c.Fd); dfree(c.fpart); dfree(c.fk); dfree(c.facc); dfree(c.cl_base); dfree(c.sc_base); dfree(c.sc_info); dfree(c.cl_lo);
+  dfree(c.F); dfree(c.Fd); dfree(c.fpart); dfree(c.facc); dfree(c.cl_base); dfree(c.sc_base); dfree(c.sc_info); dfree(c.cl_lo);
   dfree(c.cl_hi); dfree(c.cjrec); dfree(c.cq4); dfree(c.cs); dfree(c.cqf); dfree(c.cqd); dfree(c.cmap);
   dfree(c.cell_count); dfree(c.cell_start); dfree(c.key); dfree(c.off); dfree(c.tmp);
   dfree(c.scan_blk);
@@ -686,7 +686,6 @@ int rbe_init(rbe_handle *hout, const rbe_params *p, int64_t N, const double box[
     if (!fp64) rc |= dalloc(c, &c.cjrec, 8 * cpair_clusters_bound(c));  // 8 slots per cluster
     rc |= dalloc(c, &c.cq4, Nq);
   }
-  rc |= dalloc(c, reinterpret_cast<char **>(&c.fk), 3 * Nq * (fp64 ? 8 : 4));
   rc |= dalloc(c, &c.cs, 3 * Nq);
   rc |= dalloc(c, &c.cqf, Nq);
   if (fp64) rc |= dalloc(c, &c.cqd, Nq);
@@ -739,7 +738,7 @@ int rbe_init(rbe_handle *hout, const rbe_params *p, int64_t N, const double box[
     return RBE_ERR_OOM;
   }
   c.flags_host = reinterpret_cast<int *>(c.scal_host + S_COUNT);
-  c.cell_start += 0;
+  c.fk = c.outd;
   c.ccell_start = c.cell_start + (c.grid.ncell + 1);
   c.ccell_count = c.cell_count + c.grid.ncell;
 

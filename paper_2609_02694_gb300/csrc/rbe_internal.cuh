@@ -120,8 +120,10 @@ struct Ctx {
   float *invm[2] = {nullptr, nullptr};
   float *F = nullptr;
   double *Fd = nullptr;
-  void *fk = nullptr;          // k-space forces in charged order, 3 Nq of the form's type (unless
-                               // the gather adds to the cluster kernel's fixed-point sums)
+  // k-space forces in charged order, 3 Nq of the form's type (unless the gather adds to the cluster
+  // kernel's fixed-point sums). They live within one evaluation, so they take the front of outd,
+  // which only calls that wait for their results fill: 12 or 24 bytes a charged particle less.
+  void *fk = nullptr;
   double *fpart = nullptr;     // per-particle pair kernel: partial forces of a split pass
   // cluster-pair kernel: fixed-point force sums (3N, sorted order), per-row cluster and
   // super-cluster offsets (rows + 1 each), per-cluster bounds
