@@ -253,12 +253,26 @@ int make_branch(Ctx &c) {
 // the longer branch (measured, a step: cluster kernel on 2^20 particles 1.445 -> 1.360 ms; random
 // batch list on 200,000 / 1,400,000 ions 258 -> 225 / 1,226 -> 1,135 us; Verlet list on 100,000 ions
 // 123 -> 100; rows, sums and kinetic energy moved over: 3,000 charged particles 78 -> 74, an evaluation 79 -> 73).
+//
+// late: the chain, with the sampler at its head, is let go together with the real-space pass, not
+// before it. The passes of one-warp blocks (all but the cluster kernel) fill the GPU about once or
+// less; blocks of the chain that sit on the SMs first, set up for little shared memory, keep the
+// pass's blocks off them, and these crowd on the SMs left over, for their whole run. A step with the
+// chain first / with the sampler as its head start / in one branch, us: random batch list, FP64, on
+// 5,000 charged particles 5,148 / 2,230 / 2,315, 30,001 (10% charged) 2,044 / 1,129 / 1,148, FP32 on
+// 10,001 charged 364 / 252 / 266; per-particle kernel, FP32, 90,000 charged 821 / 650 / 673; Verlet
+// list, FP64, 30,001 charged 5,809 / 4,662 / 4,856. (The FP32 Verlet list takes no shared memory and
+// waits on memory: the chain first is best, 100,000 charged particles 5% below one branch.)
 int pipeline_forked(Ctx &c, bool forces_only) {
   const bool cp = !c.rbl && !c.vl_on && cpair_usable(c);
+  const bool late = !cp && (!c.vl_on || c.precision == RBE_FP64);
   const cudaStream_t main_stream = c.stream, aux = c.aux_stream;
-  int rc = join(c, main_stream, aux);
-  if (rc == RBE_OK) rc = on_branch(c, [&] { return launch_sample_k(c); });
-  if (rc != RBE_OK) return rc;
+  int rc = RBE_OK;
+  if (!late) {
+    rc = join(c, main_stream, aux);
+    if (rc == RBE_OK) rc = on_branch(c, [&] { return launch_sample_k(c); });
+    if (rc != RBE_OK) return rc;
+  }
   if (c.vl_on) RBE_CUDA_TRY(launch_list_check(c));
   RBE_CUDA_TRY(launch_bin_count(c));
   if (cp) {
@@ -268,18 +282,21 @@ int pipeline_forked(Ctx &c, bool forces_only) {
   }
   RBE_CUDA_TRY(launch_bin_place(c));
   if (cp) rc = join(c, aux, main_stream);
+  if (late && rc == RBE_OK) rc = lists(c, cp);
   if (rc == RBE_OK) rc = join(c, main_stream, aux);
+  if (late && rc == RBE_OK) rc = real_space(c, cp, false, false);
   if (rc == RBE_OK)
     rc = on_branch(c, [&] {
-      cudaError_t e = launch_structure_factor(c);
+      cudaError_t e = late ? launch_sample_k(c) : cudaSuccess;
+      if (e == cudaSuccess) e = launch_structure_factor(c);
       if (e == cudaSuccess) e = launch_kspace_gather(c, cp);
       // (mostly charged: the pair pass takes the Coulomb pairs itself)
       if (e == cudaSuccess && cp && c.Nq * 2 <= c.N) e = launch_coulomb_subset(c, c.cq4, true);
       if (e == cudaSuccess && forces_only) e = launch_kinetic(c);
       return e == cudaSuccess ? cudaEventRecord(c.ev_join, aux) : e;
     });
-  if (rc == RBE_OK) rc = lists(c, cp);
-  if (rc == RBE_OK) rc = real_space(c, cp, false, false);
+  if (!late && rc == RBE_OK) rc = lists(c, cp);
+  if (!late && rc == RBE_OK) rc = real_space(c, cp, false, false);
   if (rc == RBE_OK) rc = join(c, main_stream, aux);
   const int parts = forces_only ? 3 : 1;  // (a step's kinetic energy comes last, on this branch)
   if (rc == RBE_OK)
