@@ -572,7 +572,9 @@ __device__ __forceinline__ void rbl_eval2(const RblArgs &a, bool a0, bool a1, in
   const f32x2 dy = mul2(pk((float)d0.y, (float)d1.y), pk(pc.h[1]));
   const f32x2 dz = mul2(pk((float)d0.z, (float)d1.z), pk(pc.h[2]));
   f32x2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
-  r2 = pk(a0 ? r2.x : 1.f, a1 ? r2.y : 1.f);
+  // (an idle half stands at r_s: within the erfc fit's range in any unit of length, so that its
+  // terms are finite before they are dropped)
+  r2 = pk(a0 ? r2.x : a.rs_mid, a1 ? r2.y : a.rs_mid);
   const f32x2 on = pk(a0 ? 1.f : 0.f, a1 ? 1.f : 0.f);
   const f32x2 ir2 = mul2(pk(rcp_approx(r2.x), rcp_approx(r2.y)), on);
   const f32x2 ir6 = mul2(mul2(ir2, ir2), ir2);

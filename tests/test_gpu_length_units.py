@@ -67,3 +67,28 @@ def test_random_batch_list(orc, precision, u, eps, eager):
     assert abs(E["lj"] - ref["U_lj"]) < 2e-6 * (abs(ref["U_lj"]) + abs(ref["U_real"]))
     assert E["lj"] == pytest.approx(ref["U_lj"], rel=2e-5)
     assert W["lj"] == pytest.approx(ref["W_lj"], rel=2e-5)
+
+
+@pytest.mark.parametrize("precision", ["fp32_comp", "fp32"])
+@pytest.mark.parametrize("frac", [0.1, 1.0])
+@pytest.mark.parametrize("eager", [0, 1])
+def test_random_batch_list_idle_halves(orc, precision, frac, eager):
+    """r_s far below 1 (8e-4): a lane's odd pair leaves half of a packed pair idle, and what that
+    half computes must not reach the sums."""
+    u, eps, N = 1e-4, 1e5, 4202
+    sy = synth.make_system(N, density=0.1, seed=14, frac_charged=frac, eps=eps)
+    sy.box, sy.sig = sy.box * u, sy.sig * u
+    alpha, C = synth.ALPHA / u ** 2, synth.COULOMB_C * u * (eps / 0.1)
+    r_core, r_s, p, seed, step = 4.0 * u, 8.0 * u, 7, 3, 6
+    with binding.from_system(sy, P=8, alpha=alpha, r_c=r_s, r_core=r_core, p_rbl=p, seed=seed,
+                             coulomb_C=C, precision=precision) as h:
+        h.set_tuning("rbl_eager", eager)
+        F, E, W = h.forces_f64(step)
+        m, S = h.sample_k(step)
+    ref = orc.rbl(sy.s, sy.q, sy.types, sy.box, alpha, r_core, r_s, p, seed, step, 0, C, sy.eps,
+                  sy.sig)
+    Fk, _, _ = orc.rbe_kspace(sy.s, sy.q, sy.box, alpha, C, m, S)
+    assert rel_l2(F, ref["F"] + Fk) < 1e-5
+    scale = abs(ref["U_lj"]) + abs(ref["U_real"])
+    assert abs(E["lj"] - ref["U_lj"]) < 2e-6 * scale
+    assert abs(E["real"] - ref["U_real"]) < 2e-6 * scale
