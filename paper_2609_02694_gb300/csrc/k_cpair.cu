@@ -463,7 +463,7 @@ template <bool COUL, bool MULTI>
 __device__ __forceinline__ float cp_band_terms(const ClusterArgs &a, float r2, float qi, float qj,
                                                float2 lj, CpAcc2 &acc) {
   const float ir2 = rcp_approx(r2), ir6 = ir2 * ir2 * ir2, t = fmaf(lj.x, ir6, lj.y);
-  float g = ir6 * ir2 * t;
+  float g = MULTI ? ir6 * t * ir2 : ir6 * ir2 * t;
   acc.u0 = add2(acc.u0, pk(MULTI ? lj.x * ir6 * ir6 : ir6 * t, 0.f));
   acc.u1 = add2(acc.u1, pk(MULTI ? lj.y * ir6 : ir6, 0.f));
   if (COUL) {
@@ -741,7 +741,7 @@ __device__ __forceinline__ void cpair32_body(const ClusterArgs &a, int bx, int n
             if (MULTI) {
               const float2 t0 = stab[ti * nt + tj0], t1 = stab[ti * nt + tj1];
               const f32x2 A = pk(t0.x, t1.x), B = pk(t0.y, t1.y);
-              g = mul2(mul2(ir6, ir2), fma2(A, ir6, B));
+              g = mul2(mul2(ir6, fma2(A, ir6, B)), ir2);  // (r^-8 alone leaves FP32 sooner)
               acc.u0 = fma2(mul2(A, ir6), ir6, acc.u0);
               acc.u1 = fma2(B, ir6, acc.u1);
             } else {

@@ -583,14 +583,14 @@ __device__ __forceinline__ void rbl_eval2(const RblArgs &a, bool a0, bool a1, in
     const LJTable *tab = a.pa.table;
     const int p0 = ti * tab->nt + t0, p1 = ti * tab->nt + t1;
     const f32x2 A = pk(tab->A12[p0], tab->A12[p1]), B = pk(-tab->B6[p0], -tab->B6[p1]);
-    g = mul2(mul2(ir6, ir2), fma2(A, ir6, B));
+    g = mul2(mul2(ir6, fma2(A, ir6, B)), ir2);
     acc.u0 = fma2(mul2(A, ir6), ir6, acc.u0);
     acc.u1 = fma2(B, ir6, acc.u1);
   } else {
-    // (no r^-12 without its coefficient: it leaves FP32's range in small units of length)
-    const f32x2 t = fma2(pk(a.pa.ljA12), ir6, pk(-a.pa.ljB6));
-    g = mul2(mul2(ir6, ir2), t);
-    acc.u0 = fma2(ir6, t, acc.u0);
+    // (no r^-12 or r^-8 without the coefficients: they leave FP32's range in small units of length)
+    const f32x2 w = mul2(ir6, fma2(pk(a.pa.ljA12), ir6, pk(-a.pa.ljB6)));
+    g = mul2(w, ir2);
+    acc.u0 = add2(acc.u0, w);
     acc.u1 = add2(acc.u1, ir6);
   }
   if (COUL) {

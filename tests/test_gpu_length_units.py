@@ -92,3 +92,31 @@ def test_random_batch_list_idle_halves(orc, precision, frac, eager):
     scale = abs(ref["U_lj"]) + abs(ref["U_real"])
     assert abs(E["lj"] - ref["U_lj"]) < 2e-6 * scale
     assert abs(E["real"] - ref["U_real"]) < 2e-6 * scale
+
+
+@pytest.mark.parametrize("precision", ["fp32_comp", "fp32"])
+@pytest.mark.parametrize("traversal,two", [("rbl", 0), ("rbl", 1), ("cells", 1)])
+def test_charges_alone(orc, precision, traversal, two):
+    """No Lennard-Jones part (eps 0), neighbours some 4e-6 apart: r^-6 is an FP32 number, r^-8 is
+    not, and neither may reach the forces."""
+    u, N, seed, step = 2e-6, 4202, 3, 6
+    sy = synth.make_system(N, density=0.1, seed=14, all_charged=True, eps=0.0)
+    sy.box, sy.sig = sy.box * u, sy.sig * u
+    if two:
+        sy.types = (np.arange(N) % 3 == 0).astype(np.int32)
+        sy.eps, sy.sig = np.zeros(4), np.array([3.0, 2.8, 2.8, 2.6]) * u
+    alpha, C, r_s, r_core = synth.ALPHA / u ** 2, synth.COULOMB_C * u ** 2, 8.0 * u, 4.0 * u
+    kw = dict(r_core=r_core, p_rbl=7) if traversal == "rbl" else {}
+    with binding.from_system(sy, P=8, alpha=alpha, r_c=r_s, seed=seed, coulomb_C=C,
+                             precision=precision, **kw) as h:
+        F, E, W = h.forces_f64(step)
+        m, S = h.sample_k(step)
+    if traversal == "rbl":
+        ref = orc.rbl(sy.s, sy.q, sy.types, sy.box, alpha, r_core, r_s, 7, seed, step, 0, C, sy.eps,
+                      sy.sig)
+        F0 = ref["F"] + orc.rbe_kspace(sy.s, sy.q, sy.box, alpha, C, m, S)[0]
+    else:
+        ref = orc.total_forces(sy.s, sy.q, sy.types, sy.box, alpha, r_s, C, sy.eps, sy.sig, m, S)
+        F0 = ref["F"]
+    assert rel_l2(F, F0) < 1e-5
+    assert E["lj"] == 0.0 and E["real"] == pytest.approx(ref["U_real"], rel=1e-5)
