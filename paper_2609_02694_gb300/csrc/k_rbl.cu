@@ -981,7 +981,7 @@ __global__ void __launch_bounds__(32, EAGER ? 18 : 20) rbl32_kernel(const RblArg
       wlj = u0 + u1;
     } else {
       // u0 = 12 A s12 - 6 B s6 and u1 = s6, so A s12 - B s6 = (u0 - 6 B s6) / 12
-      ulj = fmaf(-a.pa.ljB6, u1, u0) * (1.f / 12.f);
+      ulj = fmaf(-a.pa.ljB6, u1, u0) / 12.f;
       wlj = u0;
     }
     if (COUL) {  // core + w shell with the compensations, as an unevaluated FP32 sum
