@@ -112,7 +112,7 @@ __device__ __forceinline__ PairAcc<double> rbl_pair_eval(const RblArgs &a, const
   PairAcc<double> t;
   t.fx = t.fy = t.fz = t.ulj = t.wlj = t.uc = t.wc = t.cuc = t.cwc = 0.0;
   t.nbr = 0;
-  pair_force_v<double, true, COUL, MULTI>(a.pa, tab, dx * on, dy * on, dz * on, r2s, qi, ti,
+  pair_force_v<COUL, MULTI>(a.pa, tab, dx * on, dy * on, dz * on, r2s, qi, ti,
                                           act ? qj : 0.0, tj, t);
   return t;
 }

@@ -161,69 +161,33 @@ __device__ __forceinline__ void lj_terms(const PairArgs &a, const LJTable *tab, 
   u = ir6 * mad(A, ir6, -B);
 }
 
-// Pair force, energies and virial of one pair that is inside the cutoff (Eqs. F_i,
-// G_short, LJ), added to acc.
-template <typename real, bool LJ, bool COUL, bool MULTI>
-__device__ __forceinline__ void pair_force_v(const PairArgs &a, const LJTable *tab, real dx,
-                                             real dy, real dz, real r2, real qi, int ti,
-                                             real qj, int tj, PairAcc<real> &acc) {
+// Pair force, energies and virial of one pair that is inside the cutoff (Eqs. F_i, G_short, LJ),
+// added to acc: the FP64 form's random batch list.
+template <bool COUL, bool MULTI>
+__device__ __forceinline__ void pair_force_v(const PairArgs &a, const LJTable *tab, double dx,
+                                             double dy, double dz, double r2, double qi, int ti,
+                                             double qj, int tj, PairAcc<double> &acc) {
   const PairConst &pc = a.pc;
-  real g = (real)0;
-  if (LJ) {
-    real ir2;
-    if (sizeof(real) == 8) ir2 = (real)(1.0 / (double)r2);
-    else ir2 = (real)__fdividef(1.0f, (float)r2);  // fast reciprocal (2 ulp)
-    real gl, u, w;
-    lj_terms<real, MULTI>(a, tab, ti, tj, ir2, gl, u, w);
-    g += gl;
-    acc.ulj += u;
-    acc.wlj += w;
-  }
+  double g, u, w;
+  lj_terms<double, MULTI>(a, tab, ti, tj, 1.0 / r2, g, u, w);
+  acc.ulj += u;
+  acc.wlj += w;
   if (COUL) {
-    const real qq = qi * qj;
-    if (qq != (real)0) {
-      real r, rinv, erfcv, expv;
-      if (sizeof(real) == 8) {
-        r = (real)sqrt((double)r2);
-        rinv = (real)1 / r;
-        erfcv = (real)erfc(pc.sqrt_alpha_d * (double)r);
-        expv = (real)exp(-pc.alpha_d * (double)r2);
-      } else {
-        rinv = (real)rsqrtf((float)r2);  // 1/r and r from one reciprocal square root
-        r = r2 * rinv;
-        erfcv = (real)erfcf(pc.sqrt_alpha * (float)r);
-        expv = (real)expf(-pc.alpha * (float)r2);
-      }
-      const real Cqq = (sizeof(real) == 8 ? (real)pc.C_d : (real)pc.C) * qq;
-      const real tsp = sizeof(real) == 8 ? (real)pc.two_sqrt_alpha_over_sqrt_pi_d
-                                         : (real)pc.two_sqrt_alpha_over_sqrt_pi;
-      const real rinv2 = rinv * rinv;
-      const real gc = Cqq * mad(erfcv * rinv, rinv2, tsp * expv * rinv2);
+    const double qq = qi * qj;
+    if (qq != 0.0) {
+      const double r = sqrt(r2), rinv = 1.0 / r;
+      const double erfcv = erfc(pc.sqrt_alpha_d * r), expv = exp(-pc.alpha_d * r2);
+      const double Cqq = pc.C_d * qq, rinv2 = rinv * rinv;
+      const double gc =
+          Cqq * mad(erfcv * rinv, rinv2, pc.two_sqrt_alpha_over_sqrt_pi_d * expv * rinv2);
       g += gc;
-      // erfc-Coulomb pair energies of both signs cancel heavily: compensate the sums
-      if (a.comp) {
-        kahan_add(acc.uc, acc.cuc, Cqq * erfcv * rinv);
-        kahan_add(acc.wc, acc.cwc, gc * r2);
-      } else {
-        acc.uc = mad(Cqq * erfcv, rinv, acc.uc);
-        acc.wc = mad(gc, r2, acc.wc);
-      }
+      acc.uc = mad(Cqq * erfcv, rinv, acc.uc);
+      acc.wc = mad(gc, r2, acc.wc);
     }
   }
   acc.fx = mad(g, dx, acc.fx);
   acc.fy = mad(g, dy, acc.fy);
   acc.fz = mad(g, dz, acc.fz);
-}
-
-// Same, with the charge and type of j read from the set.
-template <typename real, bool LJ, bool COUL, bool MULTI>
-__device__ __forceinline__ void pair_force(const PairArgs &a, const LJTable *tab, real dx,
-                                           real dy, real dz, real r2, real qi, int ti,
-                                           int64_t j, PairAcc<real> &acc) {
-  real qj = (real)0;
-  if (COUL) qj = sizeof(real) == 8 ? (real)a.set.qd[j] : (real)a.set.qf[j];
-  const int tj = MULTI ? a.set.type[j] : 0;
-  pair_force_v<real, LJ, COUL, MULTI>(a, tab, dx, dy, dz, r2, qi, ti, qj, tj, acc);
 }
 
 // Branch-light evaluation for the cell-list kernel: `act` says whether this lane holds a
@@ -380,68 +344,6 @@ __device__ __forceinline__ void grid_energies(const PairArgs &a, double s12, dou
   const double p = a.A12s * s12, q = a.B6s * s6;
   u = p / 12.0 - q / 6.0;
   w = p - q;
-}
-
-// Exact cutoff decision from the integer displacement ds = s_i - s_j (mod 2^32, the
-// minimum image), then the pair force. FP32 decides outside the +-1e-5 band around r_c^2;
-// inside it (and always in the FP64 form) the oracle's FP64 expression decides.
-template <typename real, bool LJ, bool COUL, bool MULTI>
-__device__ __forceinline__ void pair_body_ds(const PairArgs &a, const LJTable *tab, int dsx,
-                                             int dsy, int dsz, real qi, int ti, real qj,
-                                             int tj, PairAcc<real> &acc) {
-  const PairConst &pc = a.pc;
-  real dx, dy, dz, r2;
-  if (sizeof(real) == 8) {
-    dx = (real)__dmul_rn((double)dsx, pc.hd[0]);
-    dy = (real)__dmul_rn((double)dsy, pc.hd[1]);
-    dz = (real)__dmul_rn((double)dsz, pc.hd[2]);
-    r2 = (real)__dadd_rn(__dadd_rn(__dmul_rn((double)dx, (double)dx),
-                                   __dmul_rn((double)dy, (double)dy)),
-                         __dmul_rn((double)dz, (double)dz));
-    if (!((double)r2 <= pc.rc2d)) return;
-  } else {
-    dx = (real)((float)dsx * pc.h[0]);
-    dy = (real)((float)dsy * pc.h[1]);
-    dz = (real)((float)dsz * pc.h[2]);
-    r2 = mad(dx, dx, mad(dy, dy, dz * dz));
-    if ((float)r2 > pc.rc2_hi) return;
-    if ((float)r2 >= pc.rc2_lo && !(exact_r2(pc, dsx, dsy, dsz) <= pc.rc2d)) return;
-  }
-  acc.nbr += 1;
-  pair_force_v<real, LJ, COUL, MULTI>(a, tab, dx, dy, dz, r2, qi, ti, qj, tj, acc);
-}
-
-
-// Exact cutoff decision at r_c followed by the pair force (cell-list real space).
-template <typename real, bool LJ, bool COUL, bool MULTI>
-__device__ __forceinline__ void pair_body(const PairArgs &a, const LJTable *tab, uint32_t sxi,
-                                          uint32_t syi, uint32_t szi, real qi, int ti,
-                                          int64_t j, PairAcc<real> &acc) {
-  const PairConst &pc = a.pc;
-  const int dsx = (int)(sxi - a.set.sx[j]);
-  const int dsy = (int)(syi - a.set.sy[j]);
-  const int dsz = (int)(szi - a.set.sz[j]);
-  real dx, dy, dz, r2;
-  if (sizeof(real) == 8) {
-    dx = (real)__dmul_rn((double)dsx, pc.hd[0]);
-    dy = (real)__dmul_rn((double)dsy, pc.hd[1]);
-    dz = (real)__dmul_rn((double)dsz, pc.hd[2]);
-    r2 = (real)__dadd_rn(__dadd_rn(__dmul_rn((double)dx, (double)dx),
-                                   __dmul_rn((double)dy, (double)dy)),
-                         __dmul_rn((double)dz, (double)dz));
-    if (!((double)r2 <= pc.rc2d)) return;
-  } else {
-    dx = (real)((float)dsx * pc.h[0]);
-    dy = (real)((float)dsy * pc.h[1]);
-    dz = (real)((float)dsz * pc.h[2]);
-    r2 = mad(dx, dx, mad(dy, dy, dz * dz));
-    if ((float)r2 > pc.rc2_hi) return;
-    if ((float)r2 >= pc.rc2_lo) {  // exact decision inside the band
-      if (!(exact_r2(pc, dsx, dsy, dsz) <= pc.rc2d)) return;
-    }
-  }
-  acc.nbr += 1;
-  pair_force<real, LJ, COUL, MULTI>(a, tab, dx, dy, dz, r2, qi, ti, j, acc);
 }
 
 }  // namespace rbe
