@@ -85,7 +85,6 @@ struct ScanArgs {
   int32_t *cnt;           // cleared for the next binning as it is read
   int32_t *start, *blk;
   int64_t ncell, nblk;
-  int top;                // the blocks' totals are scanned by a pass of their own
   const int32_t *gate;
 };
 struct ScatterArgs {
@@ -201,25 +200,35 @@ __device__ __forceinline__ void scan_add_body(const ScanArgs &a, int bx, int) {
   const int32_t *blk = a.blk + which * a.nblk;
   int32_t *out = a.start + which * (ncell + 1);
   int32_t add = 0;
-  if (a.top) {
-    add = blk[bx];
-  } else {
-    for (int k = threadIdx.x; k < bx; k += kScanThreads) add += blk[k];
-    add = __reduce_add_sync(0xffffffffu, add);
-    if ((threadIdx.x & 31) == 0) warp_tot[threadIdx.x >> 5] = add;
-    __syncthreads();
-    add = 0;
+  for (int k = threadIdx.x; k < bx; k += kScanThreads) add += blk[k];
+  add = __reduce_add_sync(0xffffffffu, add);
+  if ((threadIdx.x & 31) == 0) warp_tot[threadIdx.x >> 5] = add;
+  __syncthreads();
+  add = 0;
 #pragma unroll
-    for (int w = 0; w < kScanThreads / 32; ++w) add += warp_tot[w];
-  }
+  for (int w = 0; w < kScanThreads / 32; ++w) add += warp_tot[w];
   const int64_t base = (int64_t)bx * kScanBlock;
   for (int k = threadIdx.x; k < kScanBlock; k += kScanThreads) {
     const int64_t idx = base + k;
     if (idx < ncell) out[idx] += add;
   }
-  if (!a.top && bx == a.nblk - 1 && threadIdx.x == 0) out[ncell] = add + blk[bx];
+  if (bx == a.nblk - 1 && threadIdx.x == 0) out[ncell] = add + blk[bx];
 }
 RBE_BATCHED_KERNEL(__launch_bounds__(kScanThreads), scan_add_kernel, ScanArgs, scan_add_body)
+
+// The same after the totals' own pass: each block's offset is there.
+__device__ __forceinline__ void scan_offset_body(const ScanArgs &a, int bx, int) {
+  if (gated_off(a.gate)) return;
+  const int which = blockIdx.y;
+  int32_t *out = a.start + which * (a.ncell + 1);
+  const int32_t add = a.blk[which * a.nblk + bx];
+  const int64_t base = (int64_t)bx * kScanBlock;
+  for (int k = threadIdx.x; k < kScanBlock; k += kScanThreads) {
+    const int64_t idx = base + k;
+    if (idx < a.ncell) out[idx] += add;
+  }
+}
+RBE_BATCHED_KERNEL(__launch_bounds__(kScanThreads), scan_offset_kernel, ScanArgs, scan_offset_body)
 
 __device__ __forceinline__ void bin_scatter_body(const ScatterArgs &a, int bx, int) {
   const int64_t i = (int64_t)bx * blockDim.x + threadIdx.x;
@@ -484,7 +493,7 @@ cudaError_t launch_bin_count(Ctx &c) {
   }
   const int64_t nblk = c.scan_nblk;
   const bool top = nblk > kScanDirect;
-  const ScanArgs sa{c.cell_count, c.cell_start, c.scan_blk, nc, nblk, top ? 1 : 0, gate};
+  const ScanArgs sa{c.cell_count, c.cell_start, c.scan_blk, nc, nblk, gate};
   e = dispatch(c, scan_block_kernel, scan_block_kernel_b, dim3((unsigned)nblk, 2),
                dim3(kScanThreads), 0, sa);
   if (e != cudaSuccess) return e;
@@ -492,8 +501,11 @@ cudaError_t launch_bin_count(Ctx &c) {
   // a class)
   e = dispatch(c, scan_top_kernel, scan_top_kernel_b, dim3(top ? 2u : 0u), dim3(kScanThreads), 0, sa);
   if (e != cudaSuccess) return e;
-  return dispatch(c, scan_add_kernel, scan_add_kernel_b, dim3(nblk > 1 ? (unsigned)nblk : 0u, 2),
-                  dim3(kScanThreads), 0, sa);
+  e = dispatch(c, scan_offset_kernel, scan_offset_kernel_b, dim3(top ? (unsigned)nblk : 0u, 2),
+               dim3(kScanThreads), 0, sa);
+  if (e != cudaSuccess) return e;
+  return dispatch(c, scan_add_kernel, scan_add_kernel_b,
+                  dim3(nblk > 1 && !top ? (unsigned)nblk : 0u, 2), dim3(kScanThreads), 0, sa);
 }
 
 // The particles moved to their cells' ranges, in order, in the other buffers (which become current).

@@ -12,8 +12,9 @@
 //     cell-ordered particles; a warp scan flattens the runs into one candidate list.
 //  2. Test: 32 candidates at a time, one per lane, from their packed (s, q) records: the
 //     exact minimum-image integer displacement, the cutoff decided in FP32 outside a band
-//     around r_c^2 and by the oracle's FP64 expression inside it (always FP64 in the FP64
-//     form). Hits are compacted (ballot) into a small per-warp buffer in shared memory.
+//     around r_c^2 and by the oracle's FP64 expression inside it (in the FP64 form too: the
+//     band covers FP32's rounding of the exact integer displacement). Hits are compacted
+//     (ballot) into a small per-warp buffer in shared memory.
 //  3. Evaluate: whenever 32 hits are buffered (and once at the end) every lane evaluates one
 //     of them (erfc, exp and a reciprocal square root), so the expensive terms run on full
 //     warps. A warp sum gives F_i, added to the force of i's slot in the full set: to F after

@@ -441,7 +441,7 @@ __device__ __forceinline__ int cp_segments(const ClusterArgs &a, int lane, int c
 // 33 instructions (49 with scalar pairs); the reaction of a visit is reduced while the next
 // visit's j records load; a block's start reads its super-cluster from one record and its
 // stencil rows by cell. On 2^20 particles the LJ pass went from 0.99e9 to 0.89e9 instructions
-// and from 1,101 to 957 us (issue 75% of the slots, FMA pipe 48%). Per visit (3.3e6 of them):
+// and from 1,101 to 959 us (issue 75% of the slots, FMA pipe 48%). Per visit (3.3e6 of them):
 // the pair loop about 120 instructions, its branches 24, the loads and conversions 38, the
 // reaction 31.
 

@@ -544,8 +544,8 @@ static cudaError_t kick_impl(Ctx &c, int do_kick) {
   }
   const KickArgs<float, float> a{c.vf[b], c.F, c.invm[b], c.N, hdk, 1.0 / c.kappa, do_kick,
                                  c.epart + c.off_ke};
-  // (a batch keeps the one-particle kernel: the same results, and replicas of any N share a
-  //  class)
+  // (a batch keeps the scalar accesses, four particles a thread as here: the same results, and
+  //  replicas of any N share a class)
   if (c.N % 4 == 0 && !c.rec) return dispatch(c, kick4_kernel, kick4_kernel_b, g, t, 0, a);
   return dispatch(c, kick_kernel<float, float>, kick_kernel_b<float, float>, g, t, 0, a);
 }

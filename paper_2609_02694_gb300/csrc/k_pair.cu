@@ -10,7 +10,7 @@
 // warp). Lanes sharing a cell row (c_y, c_z) form a group, and the group walks the union
 // of its members' stencils: for every (dy, dz) row, one contiguous run of cells in x.
 //  1. Stage: the warp loads 32 candidates j at a time (a chunk) into a ring of four
-//     chunk positions in shared memory. Each lane converts one of them to coordinates
+//     (FP64 form: sixteen) chunk positions in shared memory. Each lane converts one of them to coordinates
 //     relative to the group leader: half-precision test copies, exact integers.
 //  2. Test: every lane tests its own i against the staged j (broadcast reads, two
 //     candidates per half-precision instruction) with a cutoff widened beyond the worst
@@ -287,7 +287,7 @@ __device__ __forceinline__ void pair_body(const PairArgs &a, int bx, int) {
         //    current mask, or the next queued mask when the current one is spent. Every lane
         //    with anything pending evaluates in each iteration, so a lane that is light on the
         //    oldest chunk works ahead on newer ones: the warp's trip count follows its
-        //    heaviest lane over four chunks. Each lane evaluates its hits in a fixed order
+        //    heaviest lane over the ring's chunks. Each lane evaluates its hits in a fixed order
         //    (chunks in order, within a chunk the highest candidate first).
         //    At most kWin masks are queued: after a drain only the kWin - 1 newest chunks can
         //    hold pending hits, and the chunk being tested adds one.

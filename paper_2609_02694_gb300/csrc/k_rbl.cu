@@ -14,9 +14,11 @@
 // Work decomposition: one thread per i. Lanes of a warp whose cells share a row (c_y, c_z)
 // and lie within `gs` cells in x form a group; gs > 1 only in dilute systems, so that a
 // group fills the warp. The group walks the union of its members' 27-cell stencils: the
-// 9 rows (dz, dy) in canonical order, each a run of gs + 2 cells in x. Every candidate
-// carries its x offset in that run, and a lane keeps only candidates of its own three x
-// cells; in canonical order these form exactly the lane's own S_i order. Candidates are
+// 9 rows (dz, dy) in canonical order, each a run of gs + 2 cells in x. A lane's members lie in
+// its own three x cells of each run: any other cell of the run is a whole cell away, cells are at
+// least r_s wide, and two particles with a cell between them are more than r_s apart by the grid's
+// integers too. In canonical order they form exactly the lane's own S_i order. (The FP32 forms
+// rest on that distance; the FP64 form also masks by the candidates' x offsets.) Candidates are
 // staged in shared memory in FP32 coordinates relative to the group leader. Membership is
 // decided exactly: FP32 outside a band around r_core^2 and r_s^2 (+-1e-5, or the FP32
 // error bound of the group's extent where that is larger), the FP64 oracle expression

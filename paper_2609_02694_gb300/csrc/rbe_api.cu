@@ -86,7 +86,8 @@ void axis_table(double L, double alpha, int M, std::vector<uint64_t> &T, double 
 }
 
 // Chebyshev interpolant of erfcx(z) = exp(z^2) erfc(z) on z in [0, sqrt(alpha) r_top], as a
-// polynomial in t = 2 z / z_top - 1, kept when it deviates by less than 1e-7 relative.
+// polynomial in t = 2 z / z_top - 1, kept when it deviates by less than 1e-7 relative (the FP64
+// polynomial; ErfcFit states what FP32 makes of it).
 void erfc_fit(double alpha, double rc, ErfcFit &f) {
   constexpr int n = kErfcDeg + 1;
   const double r_top = rc * (1.0 + 1e-4), z_top = std::sqrt(alpha) * r_top;
@@ -903,10 +904,10 @@ int rbe_forces(rbe_handle h, uint64_t step, float *F_out, int F_on_device, doubl
                                    c.stream));
   }
   if (!host && !scalars) return RBE_OK;
-  if (!F_out || c.N == 0)
+  if (!F_out)
     RBE_CUDA_TRY(cudaMemcpyAsync(c.flags_host, c.err, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
   if (scalars) {
-    rc = copy_scalars(c, energies, virial, F_out && c.N > 0);
+    rc = copy_scalars(c, energies, virial, F_out != nullptr);
     if (rc != RBE_OK) return rc;
   } else {
     RBE_CUDA_TRY(cudaStreamSynchronize(c.stream));
@@ -1007,7 +1008,6 @@ int rbe_get_energies(rbe_handle h, double *energies, double *virial) {
 int rbe_get_state(rbe_handle h, double *pos, double *vel, uint32_t *s_frac) {
   if (!h) return RBE_ERR_INVALID;
   Ctx &c = *h;
-  if (c.N == 0) return read_device_flags(c);
   // one launch into device staging, then the copies (a launch, a copy and a wait for each array
   // took 390 us for 100,000 particles, 205 so; through pinned staging 399 us for 60,000, 66 so)
   const size_t n = 3 * (size_t)c.N, bd = sizeof(double) * n, bu = sizeof(uint32_t) * n;
@@ -1390,8 +1390,6 @@ int rbe_get_memory(rbe_handle h, int64_t *bytes) {
   return RBE_OK;
 }
 
-// A class: replicas whose Verlet steps launch the same kernels in the same shapes. Each of
-// its launches runs once per step over the concatenated grids of all its replicas.
 // A class: replicas whose Verlet steps launch the same kernels in the same shapes. Each of
 // its kernels runs once per step over the concatenated grids of all its replicas.
 struct BatchClass {

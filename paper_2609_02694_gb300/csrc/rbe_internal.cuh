@@ -77,8 +77,10 @@ struct PairConst {
 
 // erfc(z) = exp(-z^2) erfcx(z) with erfcx(z), z = sqrt(alpha) r, as one polynomial in
 // t = r ts - 1 in [-1, 1] for r <= r_c: the Chebyshev interpolant of degree 14, formed on the
-// host in FP64 (erfc_fit). `ok`: within 1e-7 of erfcx over the range (z up to about 3.7); a
-// larger sqrt(alpha) r_c takes erfcf and expf.
+// host in FP64 (erfc_fit). `ok`: that polynomial is within 1e-7 of erfcx over the range (z up to
+// about 3.7); a larger sqrt(alpha) r_c takes erfcf and expf. Its FP32 coefficients and Horner steps
+// are within 1.9e-7 of erfcx up to z = 3 and 3.3e-7 up to 3.7 (at the top of the range; 6e-8 on
+// average), which the exponential of the exact r^2 repays: erfcf takes a rounded sqrt(alpha) r.
 constexpr int kErfcDeg = 14;
 struct ErfcFit {
   float c[kErfcDeg + 1];
