@@ -549,8 +549,8 @@ __global__ void __launch_bounds__(kRblWarps * 32, 16) rbl64_kernel(const RblArgs
 //    sums (9 FP64 additions a warp instead of 35): FP64 runs at 1/64 of the FP32 rate, and a
 //    block's few dozen FP64 instructions cost as much as its classification in a dilute system.
 // Measured against the scalar kernel: 1,000,003 particles at 0.1 A^-3 (r_core 5, r_s 10, p 10)
-// 3,250 -> 1,840 us (2.47e9 -> 1.42e9 instructions), 200,000 and 1,400,000 ions of the LJ
-// electrolyte 261 -> 131 and 1,343 -> 682 us.
+// 3,250 -> 1,810 us (2.47e9 -> 1.42e9 instructions), 200,000 and 1,400,000 ions of the LJ
+// electrolyte 261 -> 129 and 1,343 -> 680 us.
 
 constexpr int kRblMaxWin = kRblMaxChunks / 2;
 

@@ -263,7 +263,8 @@ int make_branch(Ctx &c) {
 // 5,000 charged particles 5,148 / 2,230 / 2,315, 30,001 (10% charged) 2,044 / 1,129 / 1,148, FP32 on
 // 10,001 charged 364 / 252 / 266; per-particle kernel, FP32, 90,000 charged 821 / 650 / 673; Verlet
 // list, FP64, 30,001 charged 5,809 / 4,662 / 4,856. (The FP32 Verlet list takes no shared memory and
-// waits on memory: the chain first is best, 100,000 charged particles 5% below one branch.)
+// waits on memory: the chain first is best, 100,000 charged particles 5% below one branch.) Past one
+// wave of blocks the two orders are within 2%, the later fork 1 to 5% ahead in a step.
 int pipeline_forked(Ctx &c, bool forces_only) {
   const bool cp = !c.rbl && !c.vl_on && cpair_usable(c);
   const bool late = !cp && (!c.vl_on || c.precision == RBE_FP64);
