@@ -56,7 +56,7 @@ struct ClusterArgs {
   PairSet set;                 // full sorted set
   Grid grid;
   PairConst pc;
-  float ljA, ljB, ljA12, ljB6;
+  float ljA12, ljB6;
   double ljAd, ljBd, ljA12d, ljB6d;
   const LJTable *table;        // device copy, multi-type only
   const int32_t *cl_base;      // nrows + 1: first global cluster of each row
@@ -441,7 +441,7 @@ __device__ __forceinline__ int cp_segments(const ClusterArgs &a, int lane, int c
 // 33 instructions (49 with scalar pairs); the reaction of a visit is reduced while the next
 // visit's j records load; a block's start reads its super-cluster from one record and its
 // stencil rows by cell. On 2^20 particles the LJ pass went from 0.99e9 to 0.89e9 instructions
-// and from 1,101 to 959 us (issue 75% of the slots, FMA pipe 48%). Per visit (3.3e6 of them):
+// and from 1,101 to 955 us (issue 75% of the slots, FMA pipe 48%). Per visit (3.3e6 of them):
 // the pair loop about 120 instructions, its branches 24, the loads and conversions 38, the
 // reaction 31.
 
@@ -746,7 +746,7 @@ __device__ __forceinline__ void cpair32_body(const ClusterArgs &a, int bx, int n
               acc.u1 = fma2(B, ir6, acc.u1);
             } else {
               // (12 A stays in the factor: forces in units of 12 A would leave FP32's range in
-              // large units of length, at 340 pm say; they were 0.2% faster)
+              // large units of length, at 340 pm say, and were no faster)
               const f32x2 t = fma2(pk(a.ljA12), ir6, pk(-a.ljB6));
               g = mul2(mul2(ir6, ir2), t);
               acc.u0 = fma2(ir6, t, acc.u0);
@@ -1355,7 +1355,7 @@ cudaError_t launch_cluster_pair(Ctx &c, bool coul, bool multi, bool want_counts)
   a.set.cell_start = c.cell_start; a.set.map = nullptr; a.set.n = c.N;
   a.grid = c.grid;
   a.pc = c.pc;
-  a.ljA = c.lj.A[0]; a.ljB = c.lj.B[0]; a.ljA12 = c.lj.A12[0]; a.ljB6 = c.lj.B6[0];
+  a.ljA12 = c.lj.A12[0]; a.ljB6 = c.lj.B6[0];
   a.ljAd = c.lj.Ad[0]; a.ljBd = c.lj.Bd[0]; a.ljA12d = c.lj.A12d[0]; a.ljB6d = c.lj.B6d[0];
   a.table = reinterpret_cast<const LJTable *>(c.lj_dev);
   a.cl_base = c.cl_base; a.sc_base = c.sc_base; a.sc_info = c.sc_info; a.cl_lo = c.cl_lo; a.cl_hi = c.cl_hi;
